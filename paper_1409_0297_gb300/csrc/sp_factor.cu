@@ -15,6 +15,7 @@
 #include <cooperative_groups.h>
 
 #include <functional>
+#include <type_traits>
 #include <vector>
 
 #include <algorithm>
@@ -182,208 +183,7 @@ __global__ void front_scale_kernel(const T* fronts, long mm, double* scale) {
               (unsigned long long)__double_as_longlong(mx));
 }
 
-// LU of the panel columns [j0, j0+jb) of every front (one CTA per front).  The
-// panel rows [j0, m) are staged in shared memory (column-major, leading
-// dimension rows = m - j0); pivot rows are searched among the eliminated rows
-// [j, k) only.  Row swaps inside the panel happen in shared memory; the same
-// swaps are applied to the columns left and right of the panel by the row-block
-// solve kernel (LAPACK-style full-row interchanges).
-template <class T>
-__global__ void __launch_bounds__(256) lu_panel_kernel(T* fronts, int m, int k, int j0, int jb,
-                                                       int* piv, const double* scale,
-                                                       double ptol, int* status) {
-  extern __shared__ unsigned char smraw[];
-  T* P = reinterpret_cast<T*>(smraw);
-  __shared__ double wv[8];
-  __shared__ int wi[8];
-  __shared__ int spiv[kNB];
-  T* A = fronts + (long)blockIdx.x * m * m;
-  const int rows = m - j0;
-  const int kl = k - j0;  // pivot candidates are local rows < kl
-  const double thresh = ptol * scale[blockIdx.x];
-  for (long e = threadIdx.x; e < (long)rows * jb; e += blockDim.x) {
-    int r = (int)(e % rows), c = (int)(e / rows);
-    P[e] = A[(j0 + r) + (long)(j0 + c) * m];
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int jj = 0; jj < jb; ++jj) {
-    T* pc = P + (long)jj * rows;
-    double best = -1.0;
-    int bi = jj;
-    for (int r = jj + threadIdx.x; r < kl; r += blockDim.x) {
-      double v = fabs((double)pc[r]);
-      if (v > best) {
-        best = v;
-        bi = r;
-      }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      double ov = __shfl_down_sync(0xffffffffu, best, o);
-      int oi = __shfl_down_sync(0xffffffffu, bi, o);
-      if (ov > best || (ov == best && oi < bi)) {
-        best = ov;
-        bi = oi;
-      }
-    }
-    if (lane == 0) {
-      wv[warp] = best;
-      wi[warp] = bi;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double b0 = wv[0];
-      int i0 = wi[0];
-      for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-        if (wv[w] > b0 || (wv[w] == b0 && wi[w] < i0)) {
-          b0 = wv[w];
-          i0 = wi[w];
-        }
-      spiv[jj] = i0;
-      piv[(long)blockIdx.x * k + j0 + jj] = j0 + i0;
-      if (!(b0 > thresh)) atomicOr(status, 1);
-    }
-    __syncthreads();
-    const int p = spiv[jj];
-    if (p != jj)
-      for (int c = threadIdx.x; c < jb; c += blockDim.x) {
-        T t = P[jj + (long)c * rows];
-        P[jj + (long)c * rows] = P[p + (long)c * rows];
-        P[p + (long)c * rows] = t;
-      }
-    __syncthreads();
-    T pv = pc[jj];
-    if (!(fabs((double)pv) > 0.0)) pv = (T)(thresh > 0 ? thresh : 1e-30);
-    const T inv = (T)1 / pv;
-    for (int r = jj + 1 + threadIdx.x; r < rows; r += blockDim.x) {
-      T l = pc[r] * inv;
-      pc[r] = l;
-      for (int c = jj + 1; c < jb; ++c) P[r + (long)c * rows] -= l * P[jj + (long)c * rows];
-    }
-    __syncthreads();
-  }
-  for (long e = threadIdx.x; e < (long)rows * jb; e += blockDim.x) {
-    int r = (int)(e % rows), c = (int)(e / rows);
-    A[(j0 + r) + (long)(j0 + c) * m] = P[e];
-  }
-}
-
-// Panel LU of a large front by a cluster of kCL CTAs (thread-block cluster, one
-// front per cluster).  The panel rows [j0, m) are split in kCL contiguous chunks
-// of physical rows ("slots"), each staged in its CTA's shared memory.  Rows are
-// never moved during the panel: every CTA keeps the same position <-> slot maps
-// and applies the pivot interchanges to the maps only.  Per pivot column each
-// CTA folds its best candidate into a 64-bit key (magnitude rounded to FP32 in
-// the high word, position in the low word; double-buffered), one cluster
-// barrier, then warp 0 of every CTA reads the kCL keys and the pivot row through
-// distributed shared memory (the pivot row is final from then on) and updates
-// the maps; after one block barrier each thread updates its own slots.  The
-// panel is written back in position order.  The pivot is a largest-magnitude
-// entry of the column up to FP32 rounding of the magnitudes (ties and
-// near-ties go to the smallest position).
-constexpr int kCL = 8;
-template <class T>
-__global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(256)
-    lu_panel_cluster_kernel(T* fronts, int m, int k, int j0, int jb, int* piv,
-                            const double* scale, double ptol, int* status) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cl = cg::this_cluster();
-  const int rank = (int)cl.block_rank();
-  const int f = blockIdx.x / kCL;
-  T* A = fronts + (long)f * m * m;
-  const int rows = m - j0, kl = k - j0;
-  const int chunk = (rows + kCL - 1) / kCL;
-  const int rbeg = rank * chunk, rend = min(rows, rbeg + chunk);
-  const int nmy = max(0, rend - rbeg);
-  extern __shared__ unsigned char smraw[];
-  T* P = reinterpret_cast<T*>(smraw);                        // chunk x jb, column-major
-  int* pos2slot = reinterpret_cast<int*>(P + (long)chunk * jb);  // rows
-  int* slot2pos = pos2slot + rows;                            // rows
-  // candidate key: (float bits of |value|) << 32 | (0xffffffff - position), so the
-  // largest key is the largest magnitude, ties to the smallest position
-  __shared__ unsigned long long ckey[2];
-  __shared__ T prow[kNB];
-  __shared__ int s_slot;
-  const double thresh = ptol * scale[f];
-  for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-    pos2slot[i] = i;
-    slot2pos[i] = i;
-  }
-  if (threadIdx.x < 2) ckey[threadIdx.x] = 0ull;
-  for (long e = threadIdx.x; e < (long)nmy * jb; e += blockDim.x) {
-    int r = (int)(e % nmy), c = (int)(e / nmy);
-    P[r + (long)c * chunk] = A[(j0 + rbeg + r) + (long)(j0 + c) * m];
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int jj = 0; jj < jb; ++jj) {
-    // best candidate among my slots whose position is in [jj, kl)
-    unsigned long long key = 0ull;
-    for (int sl = rbeg + threadIdx.x; sl < rend; sl += blockDim.x) {
-      const int ps = slot2pos[sl];
-      if (ps < jj || ps >= kl) continue;
-      float v = (float)fabs((double)P[(sl - rbeg) + (long)jj * chunk]);
-      unsigned long long kk = ((unsigned long long)__float_as_uint(v) << 32) |
-                              (unsigned long long)(0xffffffffu - (unsigned)ps);
-      key = kk > key ? kk : key;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      unsigned long long ok = __shfl_down_sync(0xffffffffu, key, o);
-      key = ok > key ? ok : key;
-    }
-    if (lane == 0 && key) atomicMax(&ckey[jj & 1], key);
-    cl.sync();  // candidates of column jj published
-    if (warp == 0) {
-      unsigned long long kb = 0ull;
-      if (lane < kCL) kb = *cl.map_shared_rank(&ckey[jj & 1], lane);
-      for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long ok = __shfl_down_sync(0xffffffffu, kb, o);
-        kb = ok > kb ? ok : kb;
-      }
-      kb = __shfl_sync(0xffffffffu, kb, 0);
-      const int p = kb ? (int)(0xffffffffu - (unsigned)(kb & 0xffffffffull)) : jj;
-      const double b0 = kb ? (double)__uint_as_float((unsigned)(kb >> 32)) : -1.0;
-      const int sb = pos2slot[p];
-      // the pivot row (final from now on) from its owner's shared memory
-      const int owner = sb / chunk;
-      if (lane < jb) prow[lane] = cl.map_shared_rank(P, owner)[(sb - owner * chunk) + (long)lane * chunk];
-      __syncwarp();
-      if (lane == 0) {
-        const int sa = pos2slot[jj];
-        pos2slot[jj] = sb;
-        pos2slot[p] = sa;
-        slot2pos[sb] = jj;
-        slot2pos[sa] = p;
-        s_slot = sb;
-        ckey[(jj + 1) & 1] = 0ull;  // last read before this iteration's barrier
-        if (rank == 0) {
-          piv[(long)f * k + j0 + jj] = j0 + p;
-          if (!(b0 > thresh)) atomicOr(status, 1);
-        }
-      }
-    }
-    __syncthreads();
-    T pv = prow[jj];
-    if (!(fabs((double)pv) > 0.0)) pv = (T)(thresh > 0 ? thresh : 1e-30);
-    const T inv = (T)1 / pv;
-    for (int sl = rbeg + threadIdx.x; sl < rend; sl += blockDim.x) {
-      if (slot2pos[sl] <= jj) continue;
-      T* pr = P + (sl - rbeg);
-      T l = pr[(long)jj * chunk] * inv;
-      pr[(long)jj * chunk] = l;
-      for (int c = jj + 1; c < jb; ++c) pr[(long)c * chunk] -= l * prow[c];
-    }
-  }
-  // the pivot rows read by other CTAs are final, but keep this CTA's shared
-  // memory alive until every CTA has read its last pivot row
-  cl.sync();
-  for (long e = threadIdx.x; e < (long)nmy * jb; e += blockDim.x) {
-    int r = (int)(e % nmy), c = (int)(e / nmy);
-    A[(j0 + slot2pos[rbeg + r]) + (long)(j0 + c) * m] = P[r + (long)c * chunk];
-  }
-}
-
-// Panel LU of a front too tall for the cluster panel: G CTAs per front in one
+// Panel LU of a front too tall for the register panel below: G CTAs per front in one
 // cooperative launch (every CTA resident), the fronts of a level in groups of
 // nfl per launch.  CTA g stages the panel rows ("slots") [g c, (g+1) c) of rows
 // [j0, m) in shared memory; rows never move during the panel.  A slot is a pivot
@@ -600,6 +400,360 @@ __global__ void __launch_bounds__(256) lu_panel_grid_kernel(T* fronts, int m, in
       if (ds[i] == sl) pos = dp[i];
     A[(j0 + pos) + (long)(j0 + c) * m] = P[r + (long)c * chunk];
   }
+}
+
+// ---- panel LU with the panel in registers ------------------------------------------
+// LU of the panel columns [j0, j0 + jb) of every front, rows [j0, m) ("slots", local
+// index 0 .. rows - 1), by a cluster of C CTAs of NT threads per front (C = 1: an
+// ordinary launch).  Thread t of CTA q keeps R whole panel rows in registers, slot
+// q NT R + r NT + t (r < R), so a pivot step touches shared memory only to publish one
+// candidate row.  Rows never move: a slot is a pivot candidate while its position is
+// below k (interchanges only exchange positions below k, so: slot < k - j0) and it has
+// not been a pivot; the positions are replayed once at the end.
+//
+// Pivot step.  Each warp reduces its candidates' magnitude bits and the owner of the
+// largest posts its row; one CTA barrier; every
+// warp picks the CTA's best.  With C > 1 each CTA then pushes its best row and key into
+// all C CTAs with st.async on the receiver's mbarrier (double-buffered by the step's
+// parity: a CTA pushes step j + 2 only after it holds every push of step j + 1, which
+// its peers sent after they had read step j), so a step costs one CTA barrier and one
+// one-way trip through distributed shared memory.  Every wait gives up after wait_ns
+// (status bit 2, identity interchanges, no write-back).
+//
+// The 32 columns are taken in four blocks of eight: the eight steps are unrolled with
+// the current block in registers 0-7, the columns right of it updated in groups of
+// eight (finished groups skipped), then the registers rotate by eight; the code stays
+// at eight unrolled steps.  The pivot is a largest-magnitude entry of the column (FP64:
+// up to the 20 leading mantissa bits of the magnitude), ties to the first CTA, warp, lane
+// and row.
+//
+// What bounds it: the chain of pivot steps (FP32) and the SM's two FP64 FMAs per cycle
+// (FP64), so FP32 panels take the fewest CTAs whose registers hold them and FP64 panels
+// as many as the level leaves free (panel_shape).
+constexpr int kPanelMaxC = 16;
+
+__device__ __forceinline__ unsigned mag_bits(float v) {
+  const unsigned u = __float_as_uint(v) & 0x7fffffffu;
+  return u > 0x7f800000u ? 0u : u;  // a NaN is never the largest
+}
+__device__ __forceinline__ unsigned mag_bits(double v) {
+  const unsigned u = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  return u > 0x7ff00000u || (u == 0x7ff00000u && __double2loint(v) != 0) ? 0u : u;
+}
+// 1 / v: FP64 from the hardware's approximate reciprocal (20 bits) and two Newton steps
+// r += r (1 - v r), which double the correct bits (20 -> 40 -> full); magnitudes whose
+// reciprocal could leave the normal range by division.  A step waits for it, and every
+// FP64 instruction holds a warp's quarter of the SM for 64 cycles.
+__device__ __forceinline__ float panel_recip(float v) { return 1.0f / v; }
+__device__ __forceinline__ double panel_recip(double v) {
+  const unsigned e = ((unsigned)__double2hiint(v) >> 20) & 0x7ffu;
+  if (e - 64u > 1918u) return 1.0 / v;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+  r = fma(r, fma(-v, r, 1.0), r);
+  r = fma(r, fma(-v, r, 1.0), r);
+  return r;
+}
+// v != 0 without an FP64 instruction
+__device__ __forceinline__ bool nonzero(float v) { return fabsf(v) > 0.f; }
+__device__ __forceinline__ bool nonzero(double v) {
+  return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) != 0;
+}
+// the panel row's columns [8 g, 8 g + 8) of `src` in shared memory (16-byte aligned)
+__device__ __forceinline__ void load8(const float* src, float* v) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const float4 t = reinterpret_cast<const float4*>(src)[i];
+    v[4 * i] = t.x;
+    v[4 * i + 1] = t.y;
+    v[4 * i + 2] = t.z;
+    v[4 * i + 3] = t.w;
+  }
+}
+__device__ __forceinline__ void load8(const double* src, double* v) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const double2 t = reinterpret_cast<const double2*>(src)[i];
+    v[2 * i] = t.x;
+    v[2 * i + 1] = t.y;
+  }
+}
+__device__ __forceinline__ void store8(float* dst, const float* v) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    reinterpret_cast<float4*>(dst)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+}
+__device__ __forceinline__ void store8(double* dst, const double* v) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    reinterpret_cast<double2*>(dst)[i] = make_double2(v[2 * i], v[2 * i + 1]);
+}
+__device__ __forceinline__ unsigned smem_addr(const void* p) {
+  return (unsigned)__cvta_generic_to_shared(p);
+}
+// address in CTA `rank` of the cluster of the same shared-memory location
+__device__ __forceinline__ unsigned peer_addr(unsigned a, int rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void push(unsigned dst, unsigned bar, unsigned v) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(dst),
+               "r"(v), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void push(unsigned dst, unsigned bar, unsigned long long v) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst),
+               "l"(v), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void push(unsigned dst, unsigned bar, float v) {
+  push(dst, bar, __float_as_uint(v));
+}
+__device__ __forceinline__ void push(unsigned dst, unsigned bar, double v) {
+  push(dst, bar, (unsigned long long)__double_as_longlong(v));
+}
+// bounded wait for the phase of the given parity
+__device__ __forceinline__ bool bar_wait(unsigned bar, unsigned parity, unsigned long long wait_ns) {
+  const unsigned long long t0 = gtimer_ns();
+  while (true) {
+    unsigned done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if (gtimer_ns() - t0 > wait_ns) return false;
+  }
+}
+
+template <class T, int NT, int R>
+__global__ void __launch_bounds__(NT)
+    lu_panel_reg_kernel(T* fronts, int m, int k, int j0, int jb, int C, int* piv, int* perm,
+                        const double* scale, double ptol, int* status, unsigned long long wait_ns) {
+  constexpr int W = NT / 32;
+  const int q = C > 1 ? (int)(blockIdx.x % C) : 0;
+  const long f = blockIdx.x / C;
+  T* A = fronts + f * (long)m * m + j0 + (long)j0 * m;
+  const int rows = m - j0, kl = k - j0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int s0 = q * NT * R + tid;  // slot of row r: s0 + r NT
+  __shared__ __align__(16) T wrow[2][W][kNB];   // posted candidate row of each warp
+  __shared__ unsigned wmag[2][W];
+  __shared__ int wslot[2][W];
+  __shared__ __align__(16) T crow[2][kPanelMaxC][kNB];  // pushed rows of the cluster's CTAs
+  __shared__ __align__(8) unsigned long long ckey[2][kPanelMaxC];
+  __shared__ __align__(8) unsigned long long cbar[2];
+  __shared__ int spiv[kNB];   // pivot slots in order
+  __shared__ T spv[kNB];      // pivots
+  __shared__ int spos[kNB];   // final position of the slots 0 .. 31
+  const double thresh = ptol * scale[f];
+  if (C > 1) {
+    if (tid == 0) {
+      for (int i = 0; i < 2; ++i)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&cbar[i])) : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+  }
+  T a[R][kNB];
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int c = 0; c < kNB; ++c) {
+      const int sl = s0 + r * NT;
+      a[r][c] = (sl < rows && c < jb) ? A[sl + (long)c * m] : (T)0;
+    }
+  int pj[R];  // pivot step of the row, -1: not a pivot
+#pragma unroll
+  for (int r = 0; r < R; ++r) pj[r] = -1;
+  bool ok = true, stop = false;  // this warp's last wait; the CTA gave up
+#pragma unroll 1
+  for (int o = 0; o < kNB / 8; ++o) {
+    const int live = kNB / 8 - o;  // column groups of eight not finished (the current one included)
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int jj = 8 * o + u;
+      if (jj < jb && !stop) {
+        const int buf = u & 1;
+        // this thread's candidate: magnitude + 1 (0: none), smallest slot first
+        unsigned mg = 0;
+        int sl = 0x7fffffff;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int s = s0 + r * NT;
+          if (pj[r] < 0 && s < kl) {
+            const unsigned v = mag_bits(a[r][u]) + 1u;
+            if (v > mg) {
+              mg = v;
+              sl = s;
+            }
+          }
+        }
+        const unsigned wm = __reduce_max_sync(0xffffffffu, mg);
+        const int wl = __ffs(__ballot_sync(0xffffffffu, mg == wm)) - 1;  // first lane that holds it
+        if (lane == wl) {
+#pragma unroll
+          for (int r = 0; r < R; ++r)
+            if (s0 + r * NT == sl) {
+#pragma unroll
+              for (int g = 0; g < kNB / 8; ++g)
+                if (g < live) store8(&wrow[buf][warp][8 * g], &a[r][8 * g]);
+            }
+          wmag[buf][warp] = wm;
+          wslot[buf][warp] = sl;
+        }
+        if (C > 1) {
+          // a warp whose last wait gave up stops its whole CTA here
+          stop = __syncthreads_or(!ok) != 0;
+          if (stop) continue;
+        } else if (W > 1) {
+          __syncthreads();
+        } else {
+          __syncwarp();
+        }
+        // the CTA's best
+        unsigned best = wm;
+        int wb = 0;
+        if (W > 1) {
+          const unsigned bm = lane < W ? wmag[buf][lane] : 0u;
+          best = __reduce_max_sync(0xffffffffu, bm);
+          wb = __ffs(__ballot_sync(0xffffffffu, lane < W && bm == best)) - 1;
+        }
+        int bslot = wslot[buf][wb];
+        const T* prow = wrow[buf][wb];
+        if (C > 1) {
+          // push the row and its key to every CTA of the cluster (destinations spread
+          // over the warps), then wait for the C pushes of this step
+          const unsigned rdst = smem_addr(&crow[buf][q][lane]);
+          const unsigned kdst = smem_addr(&ckey[buf][q]), bar = smem_addr(&cbar[buf]);
+          const T rv = wrow[buf][wb][lane];
+          const unsigned long long key =
+              best ? ((unsigned long long)best << 32) | (0xffffffffu - (unsigned)bslot) : 0ull;
+          if (tid == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                         "r"((unsigned)(C * (kNB * sizeof(T) + 8)))
+                         : "memory");
+          for (int dst = warp; dst < C; dst += W) {
+            const unsigned rb = peer_addr(bar, dst);
+            push(peer_addr(rdst, dst), rb, rv);
+            if (lane == 0) push(peer_addr(kdst, dst), rb, key);
+          }
+          ok = bar_wait(bar, (jj >> 1) & 1, wait_ns);
+          ok = __all_sync(0xffffffffu, ok);
+          const unsigned long long kk = lane < C ? ckey[buf][lane] : 0ull;
+          const unsigned khi = (unsigned)(kk >> 32);
+          best = __reduce_max_sync(0xffffffffu, khi);
+          const int cb = __ffs(__ballot_sync(0xffffffffu, lane < C && khi == best)) - 1;
+          bslot = (int)(0xffffffffu - (unsigned)ckey[buf][cb]);
+          prow = crow[buf][cb];
+        }
+        if (ok) {
+          T pv = prow[u];
+          if (tid == 0) {
+            spiv[jj] = best ? bslot : -1;  // there is a candidate inside k columns, always
+            spv[jj] = best ? pv : (T)0;
+          }
+          if (!nonzero(pv)) pv = (T)(thresh > 0 ? thresh : 1e-30);
+          const T inv = panel_recip(pv);
+          T l[R];
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            if (s0 + r * NT == bslot) pj[r] = jj;
+            l[r] = pj[r] < 0 ? a[r][u] * inv : (T)0;
+            if (pj[r] < 0) a[r][u] = l[r];
+          }
+#pragma unroll
+          for (int g = 0; g < kNB / 8; ++g)
+            if (g < live) {
+              T p[8];
+              load8(prow + 8 * g, p);
+#pragma unroll
+              for (int c = 0; c < 8; ++c) {
+                if (8 * g + c <= u) continue;
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                  if (pj[r] < 0) a[r][8 * g + c] = fma(-l[r], p[c], a[r][8 * g + c]);
+              }
+            }
+        }
+      }
+    }
+    // the finished block of eight columns goes to the back
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      T t[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) t[c] = a[r][c];
+#pragma unroll
+      for (int c = 0; c < kNB - 8; ++c) a[r][c] = a[r][c + 8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) a[r][kNB - 8 + c] = t[c];
+    }
+  }
+  int* pvf = piv + f * k + j0;
+  if (C > 1 && __syncthreads_or(!ok || stop)) {
+    // later kernels of the factorisation still read this panel's interchanges
+    if (tid == 0) atomicOr(status, 2);
+    if (q == 0)
+      for (int c = tid; c < jb; c += NT) pvf[c] = j0 + c;
+  } else {
+    // Replay of the interchanges: step j moves the pivot's slot to position j and the
+    // slot there to the pivot's old position.  Only the slots 0 .. 31 (whose position
+    // lane i tracks) and the pivots ever leave their own position.
+    if (W > 1) __syncthreads();
+    else __syncwarp();
+    if (warp == 0) {
+      if (q == 0 && lane < jb && !(fabs((double)spv[lane]) > thresh)) atomicOr(status, 1);
+      int pos = lane, fin = 0, pslot = lane, pdst = 0;
+      const int psb = lane < jb ? spiv[lane] : -1;
+      for (int j = 0; j < jb; ++j) {
+        int sb = __shfl_sync(0xffffffffu, psb, j);
+        const unsigned at = __ballot_sync(0xffffffffu, pos == j && !fin);
+        const int ia = at ? __ffs(at) - 1 : j;  // slot at position j
+        if (sb < 0) sb = ia;
+        const int pb = __shfl_sync(0xffffffffu, pos, sb & 31);
+        const int p = sb < kNB ? pb : sb;
+        if (lane == ia) pos = p;
+        if (lane == sb) {
+          pos = j;
+          fin = 1;
+        }
+        if (lane == j) {
+          pslot = sb;
+          pdst = p;
+        }
+      }
+      if (q == 0 && lane < jb) pvf[lane] = j0 + pdst;
+      spos[lane] = pos;
+      if (q == 0) {  // the row permutation of the eliminated block, kept up to date
+        int* pm = perm + f * k + j0;
+        const int vs = lane < kl ? pm[lane] : 0;                 // at slot `lane`
+        const int vp = lane < jb ? pm[pslot] : 0;                // at this step's pivot slot
+        __syncwarp();
+        if (lane < kl && !fin) pm[pos] = vs;
+        if (lane < jb) pm[lane] = vp;
+      }
+    }
+    if (W > 1) __syncthreads();
+    else __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int sl = s0 + r * NT;
+      if (sl < rows) {
+        const int pos = pj[r] >= 0 ? pj[r] : (sl < kNB ? spos[sl] : sl);
+#pragma unroll
+        for (int c = 0; c < kNB; ++c)
+          if (c < jb) A[pos + (long)c * m] = a[r][c];
+      }
+    }
+  }
+  // no CTA leaves while a peer may still push into its shared memory
+  if (C > 1)
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
 // ---- tournament pivoting of the grid panel (FP32 forms) -------------------------
@@ -1145,6 +1299,11 @@ __global__ void __launch_bounds__(256) gemm_gen_kernel(int M, int N, int K, T al
   }
 }
 
+__global__ void perm_identity_kernel(int* perm, int k, long np) {
+  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < np) perm[i] = (int)(i % k);
+}
+
 __global__ void lu_perm_kernel(const int* piv, int* perm, int k, int nf) {
   int f = blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= nf) return;
@@ -1381,9 +1540,6 @@ void invert_triangles(DevLevel& L, T* scratch, int Bsz, cudaStream_t st) {
   trinv_store_kernel<T><<<g, 256, 0, st>>>(F, m, Xl, Xu, sX, k, Bsz);
 }
 
-// Panel staging: one CTA when the 32-column panel fits in 160 KB of shared
-// memory, else a cluster of kCL CTAs (each holding m / kCL rows) when that fits,
-// else the cooperative grid panel working in global memory.
 template <class T>
 int panel_width(int m) {
   return m > 0 ? kNB : 0;
@@ -1412,12 +1568,142 @@ void calu_shape(int nf, int rows, int* nfl, int* G) {
   *G = std::max(1, std::min(kGridPanelMaxG, std::min(kGridPanelCTAs / *nfl, (rows + 31) / 32)));
 }
 
+// Fronts that may need the grid panel (their publication slots are allocated): those
+// too tall for the registers of eight CTAs at the smaller row count of FP64 or FP32.
+// panel_pivoting = 1 takes the tournament on all of them.
 template <class T>
-int panel_kind(int m) {  // 0 one CTA, 1 cluster, 2 grid
-  if ((size_t)m * kNB * sizeof(T) <= 160 * 1024) return 0;
-  if ((size_t)((m + kCL - 1) / kCL) * kNB * sizeof(T) + 2 * sizeof(int) * (size_t)m <= 160 * 1024)
-    return 1;
-  return 2;
+bool grid_panel_front(int m) {
+  return (size_t)((m + 7) / 8) * kNB * sizeof(T) + 2 * sizeof(int) * (size_t)m > 160 * 1024;
+}
+
+// Largest cluster of the register panel on the current device: 16 CTAs (not a portable
+// size) when one of its largest form can be resident, else 8.
+int panel_max_cluster() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 8;
+  static int cache[64] = {0};
+  if (cache[dev]) return cache[dev];
+  int best = 8;
+  auto kern = lu_panel_reg_kernel<double, 256, 3>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kPanelMaxC);
+    cfg.blockDim = dim3(256);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kPanelMaxC;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n >= 1) best = kPanelMaxC;
+  }
+  cudaGetLastError();  // a refused query leaves no error behind
+  cache[dev] = best;
+  return best;
+}
+
+// CTAs per front (C), threads (NT) and rows per thread (R) of the register panel for
+// `rows` panel rows of nf fronts; false: too tall.  A step costs ~1000 cycles on one CTA
+// and ~600 more through a cluster (32 columns: 24 us at 256 rows, 34 us at 1024 on one
+// CTA and 36 us on a cluster of four).  FP32: one CTA up to 1024 rows; beyond, CTAs of
+// 256 rows while the level leaves SMs free (2044 rows: 33 us on eight CTAs, 43 us on
+// two), else up to 1536 rows per CTA.  FP64: the rank-1 updates run at two FMAs per SM
+// cycle, so a level with few fronts splits each over as many SMs as there are, down to
+// ~96 rows per CTA (2044 rows: 61 us on 16 CTAs, 80 us on eight).
+template <class T>
+bool panel_shape(int nf, int rows, int* C, int* NT, int* R) {
+  const int maxc = panel_max_cluster();
+  int c = 1;
+  const int most = sizeof(T) == 4 ? 1536 : 768;   // rows a CTA's registers hold
+  const int aim = sizeof(T) == 4 ? 256 : 96;      // rows per CTA where SMs are free
+  const bool spread = sizeof(T) == 8 || rows > 1024;
+  while (rows > c * most || (spread && rows > c * aim && (long)nf * c * 2 <= 152 && c < maxc)) c *= 2;
+  if (c > maxc) return false;
+  const int rc = (rows + c - 1) / c;
+  static const int s32[7][2] = {{32, 1}, {32, 2}, {64, 2}, {128, 2}, {256, 2}, {256, 4}, {256, 6}};
+  // 513 .. 768 rows of many fronts: 128 x 6 leaves fewer idle rows (512 fronts of 729
+  // rows: 82 us against 117 us as 256 x 4)
+  if (sizeof(T) == 4 && rc > 512 && rc <= 768 && nf > 152) {
+    *C = c;
+    *NT = 128;
+    *R = 6;
+    return true;
+  }
+  static const int s64[6][2] = {{32, 1}, {64, 1}, {128, 1}, {128, 2}, {128, 3}, {256, 3}};
+  const int (*sh)[2] = sizeof(T) == 4 ? s32 : s64;
+  const int n = sizeof(T) == 4 ? 7 : 6;
+  for (int i = 0; i < n; ++i)
+    if (rc <= sh[i][0] * sh[i][1]) {
+      *C = c;
+      *NT = sh[i][0];
+      *R = sh[i][1];
+      return true;
+    }
+  return false;
+}
+
+// whether the level's panels are the register panel (decided by its tallest)
+template <class T>
+bool panel_in_registers(const DevLevel& L, const FactorWork& W) {
+  int c, nt, r;
+  if (sizeof(T) == 4 && W.calu && grid_panel_front<T>(L.m)) return false;
+  return panel_shape<T>(L.nf, L.m, &c, &nt, &r);
+}
+
+template <class T, int NT, int R>
+void launch_panel_reg(DevLevel& L, T* F, int j0, int jb, int C, double ptol, int* status,
+                      const FactorWork& W, cudaStream_t st) {
+  auto kern = lu_panel_reg_kernel<T, NT, R>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(L.nf * C));
+  cfg.blockDim = dim3(NT);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  if (C > 1) {
+    static bool attr = false;
+    if (!attr) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      attr = true;
+    }
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+  cudaLaunchKernelEx(&cfg, kern, F, L.m, L.k, j0, jb, C, L.piv, L.perm, (const double*)L.scale, ptol,
+                     status, W.wait_ns);
+}
+
+template <class T>
+void panel_reg(DevLevel& L, T* F, int j0, int jb, double ptol, int* status, const FactorWork& W,
+               cudaStream_t st) {
+  int C, NT, R;
+  if (!panel_shape<T>(L.nf, L.m - j0, &C, &NT, &R)) return;  // panel_in_registers: cannot happen
+  auto go = [&](auto nt, auto r) {
+    launch_panel_reg<T, decltype(nt)::value, decltype(r)::value>(L, F, j0, jb, C, ptol, status, W, st);
+  };
+  using std::integral_constant;
+  if constexpr (sizeof(T) == 4) {
+    if (NT == 32 && R == 1) go(integral_constant<int, 32>{}, integral_constant<int, 1>{});
+    else if (NT == 32) go(integral_constant<int, 32>{}, integral_constant<int, 2>{});
+    else if (NT == 64) go(integral_constant<int, 64>{}, integral_constant<int, 2>{});
+    else if (NT == 128 && R == 2) go(integral_constant<int, 128>{}, integral_constant<int, 2>{});
+    else if (NT == 128) go(integral_constant<int, 128>{}, integral_constant<int, 6>{});
+    else if (R == 2) go(integral_constant<int, 256>{}, integral_constant<int, 2>{});
+    else if (R == 4) go(integral_constant<int, 256>{}, integral_constant<int, 4>{});
+    else go(integral_constant<int, 256>{}, integral_constant<int, 6>{});
+  } else {
+    if (NT == 32) go(integral_constant<int, 32>{}, integral_constant<int, 1>{});
+    else if (NT == 64) go(integral_constant<int, 64>{}, integral_constant<int, 1>{});
+    else if (NT == 128 && R == 1) go(integral_constant<int, 128>{}, integral_constant<int, 1>{});
+    else if (NT == 128 && R == 2) go(integral_constant<int, 128>{}, integral_constant<int, 2>{});
+    else if (NT == 128) go(integral_constant<int, 128>{}, integral_constant<int, 3>{});
+    else go(integral_constant<int, 256>{}, integral_constant<int, 3>{});
+  }
 }
 
 // Panel LU of columns [j0, j0+jb) followed by the interchanges and the row-block
@@ -1428,8 +1714,9 @@ void panel_step(DevLevel& L, T* F, int j0, int jb, int c_lo, int c_hi, double pt
   double pf = 0;
   for (int j = j0; j < j0 + jb; ++j) pf += (double)(L.m - j - 1) * (1.0 + 2.0 * (j0 + jb - j - 1));
   ProfScope pp(PROF_LU_PANEL, st);
-  const int kind = panel_kind<T>(L.m);
-  if (kind == 2 && sizeof(T) == sizeof(float) && W.calu) {
+  if (panel_in_registers<T>(L, W)) {
+    panel_reg<T>(L, F, j0, jb, ptol, status, W, st);
+  } else if (sizeof(T) == sizeof(float) && W.calu) {
     const int rows = L.m - j0;
     if (rows >= (1 << 20)) return;  // slot field of the pivot key; factor_level_t rejects it
     int nfl, G;
@@ -1454,7 +1741,7 @@ void panel_step(DevLevel& L, T* F, int j0, int jb, int c_lo, int c_hi, double pt
       cudaLaunchKernelEx(&cfg, lu_panel_calu_kernel, (float*)F, L.m, L.k, j0, jb, f0, G, L.piv,
                          (const double*)L.scale, ptol, status, W.gpub, W.wait_ns);
     }
-  } else if (kind == 2) {
+  } else {
     const int rows = L.m - j0;
     if (rows >= (1 << 20)) return;  // slot field of the pivot word; factor_level_t rejects it
     int nfl, G;
@@ -1480,14 +1767,6 @@ void panel_step(DevLevel& L, T* F, int j0, int jb, int c_lo, int c_hi, double pt
       cudaLaunchKernelEx(&cfg, lu_panel_grid_kernel<T>, F, L.m, L.k, j0, jb, f0, G, L.piv,
                          (const double*)L.scale, ptol, status, W.gpub, W.wait_ns);
     }
-  } else if (kind == 1) {
-    size_t sm = sizeof(T) * (size_t)((L.m - j0 + kCL - 1) / kCL) * jb +
-                2 * sizeof(int) * (size_t)(L.m - j0);
-    lu_panel_cluster_kernel<T><<<L.nf * kCL, 256, sm, st>>>(F, L.m, L.k, j0, jb, L.piv, L.scale,
-                                                            ptol, status);
-  } else {
-    size_t sm = sizeof(T) * (size_t)(L.m - j0) * jb;
-    lu_panel_kernel<T><<<L.nf, 256, sm, st>>>(F, L.m, L.k, j0, jb, L.piv, L.scale, ptol, status);
   }
   pp.done(pf * L.nf, 1, st);
   const int nleft = std::max(0, std::min(j0, c_hi) - c_lo);
@@ -1541,9 +1820,6 @@ cudaError_t factor_level_t(int d, DevLevel& L, const DevLevel* child, const doub
                            const FactorWork& W, cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(lu_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(lu_panel_cluster_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         200 * 1024);
     cudaFuncSetAttribute(lu_panel_grid_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)kGridPanelSmem + 1024);
     cudaFuncSetAttribute(lu_panel_calu_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1582,6 +1858,10 @@ cudaError_t factor_level_t(int d, DevLevel& L, const DevLevel* child, const doub
     front_scale_kernel<T><<<gs, 256, 0, st>>>(F, mm, L.scale);
   }
   pa.done(abytes, na + 1, st);
+  if (panel_in_registers<T>(L, W)) {
+    const long np = (long)L.nf * k;
+    perm_identity_kernel<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(L.perm, k, np);
+  }
   const int NB = panel_width<T>(m);
   if (NB == 0 || m >= (1 << 20)) return cudaErrorInvalidValue;
   const int OB = factor_outer_block(sizeof(T) == sizeof(float) ? SP_PREC_FP32 : SP_PREC_FP64, W.tc,
@@ -1691,7 +1971,9 @@ cudaError_t factor_level_t(int d, DevLevel& L, const DevLevel* child, const doub
       }
     }
   }
-  lu_perm_kernel<<<(L.nf + 127) / 128, 128, 0, st>>>(L.piv, L.perm, L.k, L.nf);
+  // the register panels keep the row permutation themselves
+  if (!panel_in_registers<T>(L, W))
+    lu_perm_kernel<<<(L.nf + 127) / 128, 128, 0, st>>>(L.piv, L.perm, L.k, L.nf);
   ProfScope pi(PROF_LU_TRINV, st);
   double bw = 0;
   if (L.inv) {
@@ -1767,7 +2049,7 @@ size_t grid_panel_pub_words(int nf) {
 }
 
 bool factor_grid_panel(int prec, int m) {
-  return prec == SP_PREC_FP32 ? panel_kind<float>(m) == 2 : panel_kind<double>(m) == 2;
+  return prec == SP_PREC_FP32 ? grid_panel_front<float>(m) : grid_panel_front<double>(m);
 }
 
 int factor_panel_width(int prec, int m) {
