@@ -1166,20 +1166,16 @@ __global__ void __launch_bounds__(256) gemm_sub_kernel(int M, int N, int K, cons
   __shared__ T As[kNB][TILE];
   __shared__ T Bs[kNB][TILE + 1];
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  // FP32: this thread's C entries are loaded first, so their latency overlaps the
-  // staging of A and B and the products (the update is bound by C traffic); FP64
-  // is bound by the FP64 pipe and keeps its registers for occupancy
-  constexpr bool kPre = sizeof(T) == sizeof(float);
+  // this thread's C entries are loaded first, so their latency overlaps the staging of
+  // A and B and the products (the update is bound by C traffic)
   T cpre[R][R];
-  if constexpr (kPre) {
 #pragma unroll
-    for (int b = 0; b < R; ++b) {
-      const int c = c0 + ty + 16 * b;
+  for (int b = 0; b < R; ++b) {
+    const int c = c0 + ty + 16 * b;
 #pragma unroll
-      for (int a = 0; a < R; ++a) {
-        const int r = r0 + tx + 16 * a;
-        cpre[a][b] = (r < M && c < N) ? C[r + (long)c * ldc] : (T)0;
-      }
+    for (int a = 0; a < R; ++a) {
+      const int r = r0 + tx + 16 * a;
+      cpre[a][b] = (r < M && c < N) ? C[r + (long)c * ldc] : (T)0;
     }
   }
   for (int e = threadIdx.x; e < K * TILE; e += blockDim.x) {
@@ -1216,10 +1212,7 @@ __global__ void __launch_bounds__(256) gemm_sub_kernel(int M, int N, int K, cons
 #pragma unroll
     for (int a = 0; a < R; ++a) {
       int r = r0 + tx + 16 * a;
-      if (r < M) {
-        if constexpr (kPre) C[r + (long)c * ldc] = cpre[a][b] - acc[a][b];
-        else C[r + (long)c * ldc] -= acc[a][b];
-      }
+      if (r < M) C[r + (long)c * ldc] = cpre[a][b] - acc[a][b];
     }
   }
 }
@@ -1429,21 +1422,300 @@ __global__ void trinv_store_kernel(T* fronts, int m, const T* Xl, const T* Xu, l
   fronts[f * (long)m * m + r + c * m] = (r > c) ? Xl[x] : Xu[x];
 }
 
+// ---- FP64 products on the tensor cores -----------------------------------------------
+// C = beta C +- A B in FP64 from exact integer products (the error-free splitting of
+// Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication by
+// using fast routines of matrix multiplication", Numer. Algorithms 59, 2012).  FP64 FMAs
+// run at two per SM cycle here, FP16 tensor-core products at a thousand.
+//
+// Per 32-deep chunk, a row of A (a column of B) is written on a common exponent E, the
+// largest of its 32 entries: x = X 2^(E - 1084) with |X| < 2^62 an integer that keeps all
+// 53 bits of every entry down to 2^-9 of the largest and 62 bits below that on.  X is cut
+// into seven balanced digits of nine bits, X = sum_i f_i 2^(9 i), |f_i| <= 256, each an
+// exact FP16 number.  The sums S_h = sum_{i + j = h + 6} sum_k f_i(A) f_j(B), h = 0 .. 6, are
+// then exact in the FP32 accumulators of mma.sync (at most 7 x 32 x 2^16 < 2^24), and
+// sum_k A B = 2^(Ea + Eb - 2114) sum_h S_h 2^(9 h) up to the digit pairs with i + j < 6,
+// less than 2^-56 of (row maximum) x (column maximum).  The sum of the S_h is formed as a
+// 64-bit integer and enters C with two FP64 FMAs.
+//
+// One CTA: a 64 x 64 tile, eight warps of 16 x 32 (two halves of 16 x 16, so the 56
+// accumulators of a half fit beside the fragments and two CTAs share an SM).  The tile's
+// digits are cut once into shared memory (rows of 32 halves, 80 bytes apart: conflict-free
+// for ldmatrix), 28 products of 16 x 16 x 16 per 16 x 16 block and 16 of depth.  What
+// bounds it: three FP64 instructions, ~25 integer ones and 28 / 16 x 2 tensor
+// instructions per output and chunk, where the FMA loop took 32 FP64 instructions.
+// Rows whose entries leave [2^-477, 2^477], and infinities and NaNs, take the FMA loop.
+constexpr int kDig = 7;          // digits of a number
+constexpr int kDigT = 64;        // tile
+constexpr int kDigPitch = 40;    // halves between the 32-deep rows of a digit plane
+constexpr int kDigPlane = kDigT * kDigPitch;
+constexpr int kDigElo = 546, kDigEhi = 1500;  // biased exponents of a row's largest entry
+constexpr size_t kDigSmem = 2 * kDig * kDigPlane * sizeof(__half);
+
+__device__ __forceinline__ int f64_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// the seven digits of eight numbers on the exponent E, written as eight consecutive halves
+// of seven planes (dst: the first plane's 16 bytes)
+__device__ __forceinline__ void cut_digits(const double* x, int E, __half* dst) {
+  unsigned w[kDig][4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    unsigned f[2][kDig];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const double v = x[2 * p + h];
+      const int hi = __double2hiint(v);
+      const int ex = (hi >> 20) & 0x7ff, d = E - ex;
+      unsigned long long m =
+          ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
+      m = (ex == 0 || d > 62) ? 0ull : (m << 9) >> d;
+      // every digit shifted by +256, so the fields below are unsigned
+      constexpr unsigned long long kBias =
+          256ull * (1ull | 1ull << 9 | 1ull << 18 | 1ull << 27 | 1ull << 36 | 1ull << 45 | 1ull << 54);
+      const unsigned long long u = hi < 0 ? kBias - m : kBias + m;
+      const unsigned lo = (unsigned)u, up = (unsigned)(u >> 32);
+      f[h][0] = lo & 511u;
+      f[h][1] = (lo >> 9) & 511u;
+      f[h][2] = (lo >> 18) & 511u;
+      f[h][3] = __funnelshift_r(lo, up, 27) & 511u;
+      f[h][4] = (up >> 4) & 511u;
+      f[h][5] = (up >> 13) & 511u;
+      f[h][6] = up >> 22;
+    }
+#pragma unroll
+    for (int i = 0; i < kDig; ++i) {
+      // 0x6400 | f is the FP16 number 1024 + f; minus 1280 leaves the digit f - 256
+      const unsigned t = (f[0][i] | (f[1][i] << 16)) | 0x64006400u;
+      const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&t), __half2half2(__ushort_as_half(0x6500)));
+      w[i][p] = *reinterpret_cast<const unsigned*>(&v);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < kDig; ++i)
+    *reinterpret_cast<uint4*>(dst + i * kDigPlane) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+}
+
+__device__ __forceinline__ void ldmatrix4(unsigned* r, unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ void mma_f16(float* c, const unsigned* a, unsigned b0, unsigned b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// acc +- 2^(es - 1023) sum_h S_h 2^(9 h - 14): es the biased exponent of the unit of the
+// 64-bit sum T (its 14 lowest bits are below the dropped digit pairs)
+__device__ __forceinline__ double add_digits(double acc, const float* S, int es, unsigned neg) {
+  const int s0 = __float2int_rn(S[0]), s1 = __float2int_rn(S[1]), s2 = __float2int_rn(S[2]);
+  const int s3 = __float2int_rn(S[3]), s4 = __float2int_rn(S[4]), s5 = __float2int_rn(S[5]);
+  const int s6 = __float2int_rn(S[6]);
+  const long long low = (long long)s3 * 8192 + (long long)(s2 * 16 + ((s1 + (s0 >> 9) + 16) >> 5));
+  const long long top = (long long)(s6 * 512 + s5) * 512 + s4;
+  const long long T = (top << 22) + low;
+  // T = hi 2^32 + lo as two exact doubles: 2^52 + lo, and hi - 2^20 (its 2^52 cancels)
+  const double dl = __hiloint2double(0x43300000, (int)(unsigned)T);
+  const double dh = __hiloint2double(0x43300000, (int)(T >> 32) ^ (int)0x80000000) -
+                    (4503599627370496.0 + 2147483648.0 + 1048576.0);
+  const double sl = __hiloint2double((int)(((unsigned)es << 20) | neg), 0);
+  const double sh = __hiloint2double((int)(((unsigned)(es + 32) << 20) | neg), 0);
+  return fma(sl, dl, fma(sh, dh, acc));
+}
+
+// ONE: K <= 32 (one chunk; C read while the products run).  Arguments as gemm_gen_kernel,
+// alpha = -1 (neg = the sign bit) or 1.
+template <bool ONE>
+__global__ void __launch_bounds__(256, ONE ? 2 : 1)
+    gemm_f64_kernel(int M, int N, int K, unsigned neg, int beta_one, const double* A, int lda,
+                    long sA, const double* B, int ldb, long sB, double* C, int ldc, long sC,
+                    int tilesM, int tri_a, int tri_b, int nb2, long sA2, long sB2, long sC2) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __half* Ad = reinterpret_cast<__half*>(smraw);
+  __half* Bd = Ad + kDig * kDigPlane;
+  __shared__ int eA[4][kDigT], eB[kDigT];
+  __shared__ int s_plain;
+  const long bo = blockIdx.y / nb2, bi = blockIdx.y % nb2;
+  A += bo * sA + bi * sA2;
+  B += bo * sB + bi * sB2;
+  C += bo * sC + bi * sC2;
+  const int r0 = (blockIdx.x % tilesM) * kDigT, c0 = (blockIdx.x / tilesM) * kDigT;
+  int klo = 0, khi = K;
+  if (tri_a == 1) khi = min(khi, r0 + kDigT);
+  if (tri_a == 2) klo = max(klo, r0);
+  if (tri_b == 1) klo = max(klo, c0);
+  if (tri_b == 2) khi = min(khi, c0 + kDigT);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // this thread's outputs: half s, n-tile t, register i: row rw + 8 (i / 2), column
+  // cw + 16 s + 8 t + (i & 1)
+  const int rw = (warp & 3) * 16 + (lane >> 2), cw = (warp >> 2) * 32 + 2 * (lane & 3);
+  auto out_at = [&](int s, int i) -> long {
+    const int r = r0 + rw + 8 * ((i >> 1) & 1), c = c0 + cw + 16 * s + 8 * (i >> 2) + (i & 1);
+    return r < M && c < N ? r + (long)c * ldc : -1;
+  };
+  double acc[ONE ? 1 : 2][8];
+  if (!ONE) {
+#pragma unroll
+    for (int s = 0; s < (ONE ? 1 : 2); ++s)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const long at = out_at(s, i);
+        acc[s][i] = beta_one && at >= 0 ? C[at] : 0.0;
+      }
+  }
+  const int ai = tid & 63, ak = (tid >> 6) * 8;       // A: row, first of eight columns
+  const int bc = tid >> 2, bk = (tid & 3) * 8;        // B: column, first of eight rows
+  const unsigned a_frag = smem_addr(Ad + ((warp & 3) * 16 + (lane & 15)) * kDigPitch + (lane >> 4) * 8);
+  const unsigned b_frag = smem_addr(
+      Bd + ((warp >> 2) * 32 + (lane >> 4) * 8 + (lane & 7)) * kDigPitch + ((lane >> 3) & 1) * 8);
+  for (int k0 = klo; k0 < khi; k0 += 32) {
+    const int kc = min(32, khi - k0);
+    double xa[8], xb[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      xa[j] = (r0 + ai < M && ak + j < kc) ? A[r0 + ai + (long)(k0 + ak + j) * lda] : 0.0;
+      xb[j] = (c0 + bc < N && bk + j < kc) ? B[k0 + bk + j + (long)(c0 + bc) * ldb] : 0.0;
+    }
+    if (tid == 0) s_plain = 0;
+    int ea = 0, eb = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      ea = max(ea, f64_exp(xa[j]));
+      eb = max(eb, f64_exp(xb[j]));
+    }
+    eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, 1));
+    eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, 2));
+    eA[tid >> 6][ai] = ea;
+    if ((tid & 3) == 0) eB[bc] = eb;
+    __syncthreads();  // exponents written; the previous chunk's digits are read
+    ea = max(max(eA[0][ai], eA[1][ai]), max(eA[2][ai], eA[3][ai]));
+    if ((ea != 0 && (ea < kDigElo || ea > kDigEhi)) || (eb != 0 && (eb < kDigElo || eb > kDigEhi)))
+      s_plain = 1;
+    cut_digits(xa, ea, Ad + ai * kDigPitch + ak);
+    cut_digits(xb, eb, Bd + bc * kDigPitch + bk);
+    __syncthreads();
+    if (s_plain) {  // an exponent outside the range of the scales (uniform)
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const long at = out_at(s, i);
+          if (at < 0) continue;
+          const long r = at % ldc, c = at / ldc;
+          double v = 0.0;
+          for (int k = k0; k < k0 + kc; ++k) v = fma(A[r + (long)k * lda], B[k + c * ldb], v);
+          if (neg) v = -v;
+          if (ONE) C[at] = beta_one ? C[at] + v : v;
+          else acc[ONE ? 0 : s][i] += v;
+        }
+      __syncthreads();
+      continue;
+    }
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      if (ONE) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const long at = out_at(s, i);
+          acc[0][i] = beta_one && at >= 0 ? C[at] : 0.0;
+        }
+      }
+      float P[kDig][2][4];
+#pragma unroll
+      for (int h = 0; h < kDig; ++h)
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) P[h][t][i] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) {
+        if (ks * 16 < kc) {
+          unsigned fa[kDig][4];
+#pragma unroll
+          for (int i = 0; i < kDig; ++i) ldmatrix4(fa[i], a_frag + 2 * (i * kDigPlane + ks * 16));
+#pragma unroll
+          for (int j = 0; j < kDig; ++j) {
+            unsigned fb[4];
+            ldmatrix4(fb, b_frag + 2 * (j * kDigPlane + s * 16 * kDigPitch + ks * 16));
+#pragma unroll
+            for (int i = 0; i < kDig; ++i)
+              if (i + j >= kDig - 1) {
+                mma_f16(P[i + j - (kDig - 1)][0], fa[i], fb[0], fb[1]);
+                mma_f16(P[i + j - (kDig - 1)][1], fa[i], fb[2], fb[3]);
+              }
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int row = rw + 8 * ((i >> 1) & 1), col = cw + 16 * s + 8 * (i >> 2) + (i & 1);
+        const int er = max(max(eA[0][row], eA[1][row]), max(eA[2][row], eA[3][row]));
+        const int es = max(er + eB[col] - 1077, 1);
+        float v[kDig];
+#pragma unroll
+        for (int h = 0; h < kDig; ++h) v[h] = P[h][i >> 2][i & 3];
+        double& o = acc[ONE ? 0 : s][i];
+        o = add_digits(o, v, es, neg);
+        if (ONE) {
+          const long at = out_at(s, i);
+          if (at >= 0) C[at] = o;
+        }
+      }
+    }
+    if (!ONE) __syncthreads();  // digits and exponents read before the next chunk's
+  }
+  if (!ONE) {
+#pragma unroll
+    for (int s = 0; s < (ONE ? 1 : 2); ++s)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const long at = out_at(s, i);
+        if (at >= 0) C[at] = acc[s][i];
+      }
+  }
+}
+
+void gemm_f64(int M, int N, int K, bool minus, bool beta_one, const double* A, int lda, long sA,
+              const double* B, int ldb, long sB, double* C, int ldc, long sC, int batch, int tri_a,
+              int tri_b, cudaStream_t st, int nb2 = 1, long sA2 = 0, long sB2 = 0, long sC2 = 0) {
+  const int tilesM = (M + kDigT - 1) / kDigT, tilesN = (N + kDigT - 1) / kDigT;
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(gemm_f64_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDigSmem);
+    cudaFuncSetAttribute(gemm_f64_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDigSmem);
+    attr = true;
+  }
+  dim3 g((unsigned)(tilesM * tilesN), (unsigned)(batch * nb2));
+  const unsigned neg = minus ? 0x80000000u : 0u;
+  if (K <= 32 && beta_one)
+    gemm_f64_kernel<true><<<g, 256, kDigSmem, st>>>(M, N, K, neg, 1, A, lda, sA, B, ldb, sB, C, ldc, sC,
+                                                    tilesM, tri_a, tri_b, nb2, sA2, sB2, sC2);
+  else
+    gemm_f64_kernel<false><<<g, 256, kDigSmem, st>>>(M, N, K, neg, beta_one ? 1 : 0, A, lda, sA, B, ldb,
+                                                     sB, C, ldc, sC, tilesM, tri_a, tri_b, nb2, sA2, sB2,
+                                                     sC2);
+}
+
 template <class T>
 void gemm_sub(int M, int N, int K, const T* A, int lda, long sA, const T* B, int ldb, long sB,
               T* C, int ldc, long sC, int batch, cudaStream_t st, int tile = 0) {
   if (M <= 0 || N <= 0 || K <= 0) return;
-  // padded work of 64- and 32-wide tiles relative to M N
-  const double w64 = (double)((M + 63) / 64 * 64) * ((N + 63) / 64 * 64);
-  const double w32 = (double)((M + 31) / 32 * 32) * ((N + 31) / 32 * 32);
-  if (tile == 32 || (tile == 0 && w64 > 1.1 * w32)) {
-    int tilesM = (M + 31) / 32, tilesN = (N + 31) / 32;
-    dim3 g(tilesM * tilesN, batch);
-    gemm_sub_kernel<T, 32><<<g, 256, 0, st>>>(M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, tilesM);
+  if constexpr (sizeof(T) == sizeof(double)) {
+    gemm_f64(M, N, K, true, true, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, 0, 0, st);
   } else {
-    int tilesM = (M + 63) / 64, tilesN = (N + 63) / 64;
+    // padded work of 64- and 32-wide tiles relative to M N
+    const double w64 = (double)((M + 63) / 64 * 64) * ((N + 63) / 64 * 64);
+    const double w32 = (double)((M + 31) / 32 * 32) * ((N + 31) / 32 * 32);
+    const int t = tile == 32 || (tile == 0 && w64 > 1.1 * w32) ? 32 : 64;
+    const int tilesM = (M + t - 1) / t, tilesN = (N + t - 1) / t;
     dim3 g(tilesM * tilesN, batch);
-    gemm_sub_kernel<T, 64><<<g, 256, 0, st>>>(M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, tilesM);
+    if (t == 32)
+      gemm_sub_kernel<T, 32><<<g, 256, 0, st>>>(M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, tilesM);
+    else
+      gemm_sub_kernel<T, 64><<<g, 256, 0, st>>>(M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, tilesM);
   }
 }
 
@@ -1453,21 +1725,19 @@ void gemm_gen(int M, int N, int K, T alpha, bool beta_one, const T* A, int lda, 
               int tri_b, cudaStream_t st, int nb2 = 1, long sA2 = 0, long sB2 = 0, long sC2 = 0,
               int tile = 0) {
   if (M <= 0 || N <= 0 || K <= 0 || batch <= 0 || nb2 <= 0) return;
-  int tilesM = (M + kTile - 1) / kTile, tilesN = (N + kTile - 1) / kTile;
-  if (tile == 32 || (tile == 0 && (long)tilesM * tilesN * batch * nb2 < 304)) {
-    // small problem: 32 x 32 tiles give four times the CTAs
-    tilesM = (M + 31) / 32;
-    tilesN = (N + 31) / 32;
+  if constexpr (sizeof(T) == sizeof(double)) {  // every caller's alpha is 1 or -1
+    gemm_f64(M, N, K, alpha < 0, beta_one, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, tri_a, tri_b, st,
+             nb2, sA2, sB2, sC2);
+  } else {
+    // a small problem takes 32 x 32 tiles: four times the CTAs
+    const long big = (long)((M + kTile - 1) / kTile) * ((N + kTile - 1) / kTile) * batch * nb2;
+    const int t = tile == 32 || (tile == 0 && big < 304) ? 32 : kTile;
+    const int tilesM = (M + t - 1) / t, tilesN = (N + t - 1) / t;
     dim3 g(tilesM * tilesN, batch * nb2);
-    gemm_gen_kernel<T, 32><<<g, 256, 0, st>>>(M, N, K, alpha, beta_one ? 1 : 0, A, lda, sA, B, ldb,
-                                              sB, C, ldc, sC, tilesM, tri_a, tri_b, nb2, sA2, sB2,
-                                              sC2);
-    return;
+    auto kern = t == 32 ? gemm_gen_kernel<T, 32> : gemm_gen_kernel<T, kTile>;
+    kern<<<g, 256, 0, st>>>(M, N, K, alpha, beta_one ? 1 : 0, A, lda, sA, B, ldb, sB, C, ldc, sC, tilesM,
+                            tri_a, tri_b, nb2, sA2, sB2, sC2);
   }
-  dim3 g(tilesM * tilesN, batch * nb2);
-  gemm_gen_kernel<T, kTile><<<g, 256, 0, st>>>(M, N, K, alpha, beta_one ? 1 : 0, A, lda, sA, B, ldb,
-                                               sB, C, ldc, sC, tilesM, tri_a, tri_b, nb2, sA2, sB2,
-                                               sC2);
 }
 
 // Replace the diagonal blocks (size Bsz, a power of two >= 32) of L11 and U11 of
