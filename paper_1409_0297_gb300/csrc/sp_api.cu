@@ -843,6 +843,7 @@ static sp_status setup_impl(int d, int n, int b, int P, const double* shifts, sp
     SP_CK(dalloc(c.get(), &D.front, fsz * (size_t)D.nf * S.m * S.m));
     SP_CK(dalloc(c.get(), &D.perm, sizeof(int) * (size_t)D.nf * std::max(1, S.k)));
     SP_CK(dalloc(c.get(), &D.piv, sizeof(int) * (size_t)D.nf * std::max(1, S.k)));
+    SP_CK(dalloc(c.get(), &D.pmap, sizeof(int) * 64 * (size_t)D.nf * std::max(1, (S.k + 31) / 32)));
     SP_CK(dalloc(c.get(), &D.scale, sizeof(double) * D.nf));
     SP_CK(dalloc(c.get(), &D.upd, vsz * RH * (size_t)D.nf * std::max(1, S.m - S.k)));
     SP_CK(dalloc(c.get(), &D.y, vsz * RH * (size_t)D.nf * std::max(1, S.k)));

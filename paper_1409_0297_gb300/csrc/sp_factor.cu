@@ -532,7 +532,7 @@ __device__ __forceinline__ bool bar_wait(unsigned bar, unsigned parity, unsigned
 
 template <class T, int NT, int R>
 __global__ void __launch_bounds__(NT)
-    lu_panel_reg_kernel(T* fronts, int m, int k, int j0, int jb, int C, int* piv, int* perm,
+    lu_panel_reg_kernel(T* fronts, int m, int k, int j0, int jb, int C, int* piv, int* pmap, int* perm,
                         const double* scale, double ptol, int* status, unsigned long long wait_ns) {
   constexpr int W = NT / 32;
   const int q = C > 1 ? (int)(blockIdx.x % C) : 0;
@@ -695,11 +695,16 @@ __global__ void __launch_bounds__(NT)
     }
   }
   int* pvf = piv + f * k + j0;
+  int* mpf = pmap + (f * ((k + kNB - 1) / kNB) + j0 / kNB) * (2 * kNB);
   if (C > 1 && __syncthreads_or(!ok || stop)) {
     // later kernels of the factorisation still read this panel's interchanges
     if (tid == 0) atomicOr(status, 2);
     if (q == 0)
-      for (int c = tid; c < jb; c += NT) pvf[c] = j0 + c;
+      for (int c = tid; c < jb; c += NT) {
+        pvf[c] = j0 + c;
+        mpf[c] = c;
+        mpf[kNB + c] = -1;
+      }
   } else {
     // Replay of the interchanges: step j moves the pivot's slot to position j and the
     // slot there to the pivot's old position.  Only the slots 0 .. 31 (whose position
@@ -727,7 +732,11 @@ __global__ void __launch_bounds__(NT)
           pdst = p;
         }
       }
-      if (q == 0 && lane < jb) pvf[lane] = j0 + pdst;
+      if (q == 0 && lane < jb) {
+        pvf[lane] = j0 + pdst;
+        mpf[lane] = pslot;
+        mpf[kNB + lane] = fin ? -1 : pos;
+      }
       spos[lane] = pos;
       if (q == 0) {  // the row permutation of the eliminated block, kept up to date
         int* pm = perm + f * k + j0;
@@ -1072,79 +1081,140 @@ __global__ void __launch_bounds__(256) lu_panel_calu_kernel(float* fronts, int m
   }
 }
 
+// The interchanges of a panel as a map (per front and panel 2 x 32 ints, local rows):
+// map[i] = the row whose content goes to row i (the i-th pivot), map[32 + i] = the row that
+// takes row i's content, -1 when row i is a pivot itself.  Rows outside the map stay.  All
+// reads come before all writes, so a column takes one memory latency where the 32
+// exchanges in order took 32.  The register panel writes its map; this kernel makes it
+// from the pivot rows of the other panels (one warp per front).
+__global__ void panel_map_kernel(const int* piv, int* pmap, int k, int j0, int jb) {
+  const long f = blockIdx.x;
+  const int lane = threadIdx.x;
+  const int pv = lane < jb ? piv[f * k + j0 + lane] - j0 : lane;
+  int pos = lane, fin = 0, pslot = lane;
+  for (int j = 0; j < jb; ++j) {
+    const int p = __shfl_sync(0xffffffffu, pv, j);
+    const unsigned at = __ballot_sync(0xffffffffu, pos == p && !fin);
+    const int sb = at ? __ffs(at) - 1 : p;  // row at position p
+    const unsigned here = __ballot_sync(0xffffffffu, pos == j && !fin);
+    const int ia = __ffs(here) - 1;  // row at position j
+    if (lane == ia) pos = p;
+    if (lane == sb) {
+      pos = j;
+      fin = 1;
+    }
+    if (lane == j) pslot = sb;
+  }
+  int* mp = pmap + (f * ((k + kNB - 1) / kNB) + j0 / kNB) * (2 * kNB);
+  if (lane < jb) {
+    mp[lane] = pslot;
+    mp[kNB + lane] = fin ? -1 : pos;
+  }
+}
+
 // Interchanges of the panel's pivots and the row-block solve
 // A[j0:j0+jb, c] = L_pp^{-1} A[j0:j0+jb, c] on the columns c in [c_lo, c_hi)
 // outside the panel [j0, j0+jb): columns left of the panel get the interchanges
-// only, columns right of it the interchanges (when do_swap) and the solve.  One
-// thread per column.  The full-front form is c_lo = 0, c_hi = m, do_swap = 1.
+// only, columns right of it the interchanges (when do_swap) and the solve.
+// The full-front form is c_lo = 0, c_hi = m, do_swap = 1.
+// Four lanes per column (rows i = 4 r + lane % 4 in registers), eight columns per warp:
+// a solve is 144 FMA instructions and 32 shuffles deep where one thread per column took
+// 496 (in FP64, 64 cycles each), four times as many warps cover the SMs, and a column's
+// rows load as whole sectors.  3D 32^3 FP64: 29 us a launch with one thread per column.
+constexpr int kTrsmCols = 32;  // columns per CTA
 template <class T>
-__global__ void __launch_bounds__(256) lu_trsm_kernel(T* fronts, int m, int k, int j0, int jb,
-                                                      const int* piv, int c_lo, int c_hi,
-                                                      int do_swap) {
+__global__ void __launch_bounds__(4 * kTrsmCols) lu_trsm_kernel(T* fronts, int m, int k, int j0,
+                                                                int jb, const int* pmap, int c_lo,
+                                                                int c_hi, int do_swap) {
   T* A = fronts + (long)blockIdx.y * m * m;
   __shared__ T Lp[kNB][kNB + 1];
-  __shared__ int sp_[kNB];
-  for (int e = threadIdx.x; e < jb * jb; e += blockDim.x) {
-    int i = e % jb, l = e / jb;
-    Lp[i][l] = A[(j0 + i) + (long)(j0 + l) * m];
+  __shared__ int mp[2 * kNB];
+  for (int e = threadIdx.x; e < kNB * kNB; e += blockDim.x) {
+    const int i = e % kNB, l = e / kNB;
+    Lp[i][l] = (i < jb && l < i) ? A[(j0 + i) + (long)(j0 + l) * m] : (T)0;
   }
-  for (int e = threadIdx.x; e < jb; e += blockDim.x) sp_[e] = piv[(long)blockIdx.y * k + j0 + e];
+  if (do_swap && threadIdx.x < 2 * kNB)
+    mp[threadIdx.x] =
+        pmap[((long)blockIdx.y * ((k + kNB - 1) / kNB) + j0 / kNB) * (2 * kNB) + threadIdx.x];
   __syncthreads();
   const int nleft = max(0, min(j0, c_hi) - c_lo);
   const int rbeg = max(j0 + jb, c_lo);
-  const int cc = blockIdx.x * blockDim.x + threadIdx.x;
+  const int sub = threadIdx.x & 3;
+  const int cc = blockIdx.x * kTrsmCols + (threadIdx.x >> 2);
   const int c = cc < nleft ? c_lo + cc : rbeg + (cc - nleft);
-  if (c >= c_hi) return;
-  T* colg = A + (long)c * m;
-  if (do_swap)
-    for (int jj = 0; jj < jb; ++jj) {
-      int p = sp_[jj];
-      if (p != j0 + jj) {
-        T t = colg[j0 + jj];
-        colg[j0 + jj] = colg[p];
-        colg[p] = t;
-      }
+  const bool live = c < c_hi;
+  T* col = A + (long)c * m + j0;
+  constexpr int R = kNB / 4;
+  T x[R], y[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int i = 4 * r + sub;
+    const bool in = live && i < jb;
+    y[r] = in ? col[i] : (T)0;
+    x[r] = do_swap && in ? col[mp[i]] : y[r];
+  }
+  if (do_swap) {
+    __syncwarp();  // the four lanes of a column have read it
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = 4 * r + sub;
+      if (live && i < jb && mp[kNB + i] >= 0) col[mp[kNB + i]] = y[r];
     }
-  if (cc < nleft) return;
-  T x[kNB];
-  T* col = colg + j0;
+    __syncwarp();
+  }
 #pragma unroll
-  for (int i = 0; i < kNB; ++i)
-    if (i < jb) x[i] = col[i];
+  for (int l = 0; l < kNB - 1; ++l) {
+    const T xl = __shfl_sync(0xffffffffu, x[l >> 2], (threadIdx.x & 28) | (l & 3));
+    if (cc >= nleft) {
 #pragma unroll
-  for (int i = 1; i < kNB; ++i) {
-    if (i < jb) {
-      T acc = x[i];
-#pragma unroll
-      for (int l = 0; l < kNB; ++l)
-        if (l < i) acc -= Lp[i][l] * x[l];
-      x[i] = acc;
+      for (int r = l >> 2; r < R; ++r)
+        if (r > (l >> 2) || sub > (l & 3)) x[r] = fma(-Lp[4 * r + sub][l], xl, x[r]);
     }
   }
 #pragma unroll
-  for (int i = 0; i < kNB; ++i)
-    if (i < jb) col[i] = x[i];
+  for (int r = 0; r < R; ++r) {
+    const int i = 4 * r + sub;
+    if (live && i < jb) col[i] = x[r];
+  }
 }
 
-// Row interchanges piv[p0 .. p0+cnt) (in order) on the columns [a0, a1) and
-// [b0, b1) of every front; one thread per column.
+// Row interchanges of the panels covering [p0, p0 + cnt) (in order, p0 a multiple of 32)
+// on the columns [a0, a1) and [b0, b1) of every front: one warp per column, one panel's map
+// at a time (two loads and two stores per lane).  One thread per column and one exchange
+// after the other took up to 430 us a launch at 3D 64^3.
 template <class T>
-__global__ void lu_laswp_kernel(T* fronts, int m, int k, int p0, int cnt, const int* piv, int a0,
-                                int a1, int b0, int b1) {
+__global__ void __launch_bounds__(256) lu_laswp_kernel(T* fronts, int m, int k, int p0, int cnt,
+                                                       const int* pmap, int a0, int a1, int b0,
+                                                       int b1) {
   T* A = fronts + (long)blockIdx.y * m * m;
-  const int cc = blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int cc = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int na = a1 - a0;
   const int c = cc < na ? a0 + cc : b0 + (cc - na);
   if (c >= (cc < na ? a1 : b1)) return;
-  const int* pv = piv + (long)blockIdx.y * k;
   T* col = A + (long)c * m;
-  for (int j = p0; j < p0 + cnt; ++j) {
-    const int p = pv[j];
-    if (p != j) {
-      T t = col[j];
-      col[j] = col[p];
-      col[p] = t;
+  const int* mp = pmap + ((long)blockIdx.y * ((k + kNB - 1) / kNB) + p0 / kNB) * (2 * kNB);
+  int src = mp[lane], dst = mp[kNB + lane];
+  for (int j0 = p0; j0 < p0 + cnt; j0 += kNB) {
+    const int jb = min(kNB, p0 + cnt - j0);
+    T* cj = col + j0;
+    T x = 0, y = 0;
+    if (lane < jb) {
+      x = cj[src];
+      y = cj[lane];
     }
+    const int d = dst;
+    mp += 2 * kNB;
+    if (j0 + kNB < p0 + cnt) {
+      src = mp[lane];
+      dst = mp[kNB + lane];
+    }
+    __syncwarp();
+    if (lane < jb) {
+      cj[lane] = x;
+      if (d >= 0) cj[d] = y;
+    }
+    __syncwarp();
   }
 }
 
@@ -1944,7 +2014,7 @@ void launch_panel_reg(DevLevel& L, T* F, int j0, int jb, int C, double ptol, int
     cfg.attrs = at;
     cfg.numAttrs = 1;
   }
-  cudaLaunchKernelEx(&cfg, kern, F, L.m, L.k, j0, jb, C, L.piv, L.perm, (const double*)L.scale, ptol,
+  cudaLaunchKernelEx(&cfg, kern, F, L.m, L.k, j0, jb, C, L.piv, L.pmap, L.perm, (const double*)L.scale, ptol,
                      status, W.wait_ns);
 }
 
@@ -2038,16 +2108,15 @@ void panel_step(DevLevel& L, T* F, int j0, int jb, int c_lo, int c_hi, double pt
                          (const double*)L.scale, ptol, status, W.gpub, W.wait_ns);
     }
   }
+  if (!panel_in_registers<T>(L, W)) panel_map_kernel<<<L.nf, 32, 0, st>>>(L.piv, L.pmap, L.k, j0, jb);
   pp.done(pf * L.nf, 1, st);
   const int nleft = std::max(0, std::min(j0, c_hi) - c_lo);
   const int nright = std::max(0, c_hi - std::max(j0 + jb, c_lo));
   const int ncols = nleft + nright;
   if (ncols > 0) {
-    // one thread per column; narrow CTAs when few fronts would leave SMs idle
-    const int tb = ((long)((ncols + 255) / 256) * L.nf >= 152) ? 256 : 64;
-    dim3 gt((ncols + tb - 1) / tb, L.nf);
+    dim3 gt((ncols + kTrsmCols - 1) / kTrsmCols, L.nf);
     ProfScope pt(PROF_LU_TRSM, st);
-    lu_trsm_kernel<T><<<gt, tb, 0, st>>>(F, L.m, L.k, j0, jb, L.piv, c_lo, c_hi, 1);
+    lu_trsm_kernel<T><<<gt, 4 * kTrsmCols, 0, st>>>(F, L.m, L.k, j0, jb, L.pmap, c_lo, c_hi, 1);
     pt.done((double)nright * jb * (jb - 1) * L.nf, 1, st);
   }
 }
@@ -2167,8 +2236,8 @@ cudaError_t factor_level_t(int d, DevLevel& L, const DevLevel* child, const doub
       const int ncols = std::max(0, a1 - a0) + std::max(0, b1 - b0);
       if (ncols <= 0 || cnt <= 0) return;
       ProfScope pt(PROF_LU_TRSM, st);
-      dim3 g((ncols + 255) / 256, L.nf);
-      lu_laswp_kernel<T><<<g, 256, 0, st>>>(F, m, k, p0, cnt, L.piv, a0, std::max(a0, a1), b0,
+      dim3 g((ncols + 7) / 8, L.nf);
+      lu_laswp_kernel<T><<<g, 256, 0, st>>>(F, m, k, p0, cnt, L.pmap, a0, std::max(a0, a1), b0,
                                             std::max(b0, b1));
       pt.done(0, 1, st);
     };
@@ -2184,10 +2253,9 @@ cudaError_t factor_level_t(int d, DevLevel& L, const DevLevel* child, const doub
           const int jb = std::min(NB, r1 - j0);
           {
             const int ncol = c1 - c0;
-            const int tb = ((long)((ncol + 255) / 256) * L.nf >= 152) ? 256 : 64;
-            dim3 gt((ncol + tb - 1) / tb, L.nf);
+            dim3 gt((ncol + kTrsmCols - 1) / kTrsmCols, L.nf);
             ProfScope pt(PROF_LU_TRSM, st);
-            lu_trsm_kernel<T><<<gt, tb, 0, st>>>(F, m, k, j0, jb, L.piv, c0, c1, 0);
+            lu_trsm_kernel<T><<<gt, 4 * kTrsmCols, 0, st>>>(F, m, k, j0, jb, L.pmap, c0, c1, 0);
             pt.done((double)ncol * jb * (jb - 1) * L.nf, 1, st);
           }
           const int base = j0 + jb;

@@ -68,6 +68,7 @@ struct DevLevel {
   void* front = nullptr;    // nf x m x m of double (FP64) or float (FP32)
   int* perm = nullptr;      // nf x k row permutation of the eliminated block
   int* piv = nullptr;       // nf x k pivot rows (LAPACK style, 0-based within the front)
+  int* pmap = nullptr;      // nf x ceil(k / 32) x 64: each panel's interchanges as a map
   double* scale = nullptr;  // nf: max |entry| of the assembled front
   void* upd = nullptr;      // nf x (m - k) complex update vectors of the forward sweep
   void* y = nullptr;        // nf x k complex forward-sweep results
