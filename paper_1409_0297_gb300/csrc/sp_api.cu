@@ -836,9 +836,27 @@ static sp_status setup_impl(int d, int n, int b, int P, const double* shifts, sp
         for (int v : S.gidx) gg.push_back(v + (int)((long)p * N));
       SP_CK(upload(c.get(), &D.gidx, gg));
     }
-    SP_CK(upload(c.get(), &D.asm_row, S.asm_row));
-    SP_CK(upload(c.get(), &D.asm_tidx, S.asm_tidx));
-    SP_CK(upload(c.get(), &D.asm_cvar, S.asm_cvar));
+    {  // the assembly list in the order of the front's columns, rows ascending (two counting
+       // sorts), so that a warp of assemble_kernel writes neighbouring entries
+      const size_t na = S.asm_row.size();
+      std::vector<int> by(na), tmp(na), row(na), tidx(na), cvar(na);
+      for (size_t i = 0; i < na; ++i) by[i] = (int)i;
+      for (const std::vector<int>* key : {&S.asm_row, &S.asm_cvar}) {
+        std::vector<int> at(S.m + 1, 0);
+        for (int v : *key) ++at[v + 1];
+        for (int v = 0; v < S.m; ++v) at[v + 1] += at[v];
+        for (int i : by) tmp[at[(*key)[i]]++] = i;
+        by.swap(tmp);
+      }
+      for (size_t i = 0; i < na; ++i) {
+        row[i] = S.asm_row[by[i]];
+        tidx[i] = S.asm_tidx[by[i]];
+        cvar[i] = S.asm_cvar[by[i]];
+      }
+      SP_CK(upload(c.get(), &D.asm_row, row));
+      SP_CK(upload(c.get(), &D.asm_tidx, tidx));
+      SP_CK(upload(c.get(), &D.asm_cvar, cvar));
+    }
     SP_CK(upload(c.get(), &D.ea_map, S.ea_map));
     SP_CK(dalloc(c.get(), &D.front, fsz * (size_t)D.nf * S.m * S.m));
     SP_CK(dalloc(c.get(), &D.perm, sizeof(int) * (size_t)D.nf * std::max(1, S.k)));

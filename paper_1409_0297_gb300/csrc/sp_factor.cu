@@ -152,35 +152,41 @@ __global__ void f16_copy_kernel(const float* fronts, int m, int k, __half* out, 
   for (; r < rows; r += 32) hc[r] = __float2half_rn(col[r] * inv);
 }
 
-// max |entry| of every front: CTAs over (chunk, front), atomicMax on the bit
-// pattern (non-negative doubles order like their unsigned integer bits); scale
-// must be zeroed first.
+// max |entry| of every front: CTAs over (chunk, front).  Magnitudes order like their bit
+// patterns, so the maximum is an integer one (NaNs count as 0): as FP64 fmax it held the
+// pass at 1 TB/s in FP32 (3D 64^3 leaves, 1.1 GB: 1.05 ms).  scale must be zeroed first.
+__device__ __forceinline__ unsigned mag_word(float v) {
+  const unsigned u = __float_as_uint(v) & 0x7fffffffu;
+  return u > 0x7f800000u ? 0u : u;
+}
+__device__ __forceinline__ unsigned long long mag_word(double v) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  return u > 0x7ff0000000000000ull ? 0ull : u;
+}
+__device__ __forceinline__ double mag_value(unsigned u) { return (double)__uint_as_float(u); }
+__device__ __forceinline__ double mag_value(unsigned long long u) { return __longlong_as_double((long long)u); }
 template <class T>
-__global__ void front_scale_kernel(const T* fronts, long mm, double* scale) {
+__global__ void __launch_bounds__(256) front_scale_kernel(const T* fronts, long mm, double* scale) {
   const T* A = fronts + blockIdx.y * mm;
   // eight independent loads in flight per thread (a loop-carried max with one load per
   // trip is bound by memory latency, not bandwidth)
   constexpr int kU = 8;
+  using W = decltype(mag_word(T()));
   const long stride = (long)gridDim.x * blockDim.x;
-  double mxu[kU];
-#pragma unroll
-  for (int u = 0; u < kU; ++u) mxu[u] = 0;
+  W mx = 0;
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   for (; i + (kU - 1) * stride < mm; i += kU * stride) {
     T v[kU];
 #pragma unroll
     for (int u = 0; u < kU; ++u) v[u] = A[i + u * stride];
 #pragma unroll
-    for (int u = 0; u < kU; ++u) mxu[u] = fmax(mxu[u], fabs((double)v[u]));
+    for (int u = 0; u < kU; ++u) mx = max(mx, mag_word(v[u]));
   }
-  for (; i < mm; i += stride) mxu[0] = fmax(mxu[0], fabs((double)A[i]));
-  double mx = mxu[0];
-#pragma unroll
-  for (int u = 1; u < kU; ++u) mx = fmax(mx, mxu[u]);
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, o));
+  for (; i < mm; i += stride) mx = max(mx, mag_word(A[i]));
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o));
   if ((threadIdx.x & 31) == 0 && mx > 0)
     atomicMax(reinterpret_cast<unsigned long long*>(scale + blockIdx.y),
-              (unsigned long long)__double_as_longlong(mx));
+              (unsigned long long)__double_as_longlong(mag_value(mx)));
 }
 
 // Panel LU of a front too tall for the register panel below: G CTAs per front in one
@@ -1380,112 +1386,76 @@ __global__ void lu_perm_kernel(const int* piv, int* perm, int k, int nf) {
   }
 }
 
-// ---- explicit triangular inverses for levels with few fronts -------------------
-// Inverse of every 32 x 32 diagonal block of L11 (unit lower; upper == 0) or U11
-// (upper == 1) of every front, written to the matching diagonal block of X
-// (entry (i, j) at i + j ldx, front stride sX).  One CTA per (block, front);
-// thread c solves column c by substitution.
+// ---- explicit triangular inverses -------------------------------------------------
+// Inverses of every 32 x 32 diagonal block of L11 (unit lower) and U11 of every front, one
+// CTA per (block, front): threads 0-127 invert the L block, 128-255 the U block, four lanes
+// per column (rows 4 r + lane % 4 in registers) as in lu_trsm_kernel, U with the
+// reciprocals of its diagonal taken once.  Xl != null: written to the matching diagonal
+// blocks of Xl and Xu (entry (i, j) at i + j ldx, front stride sX).  Xl == null: in place,
+// the strict lower part from L^{-1}, the upper part with the diagonal from U^{-1}; the
+// sweeps then resolve a diagonal block with a matrix-vector product instead of 32
+// dependent steps.  With one thread per column (496 FMAs and 32 divisions in a row) an FP64
+// launch took 64 us however few its blocks were.
 template <class T>
-__global__ void trinv_diag32_kernel(const T* fronts, int m, T* X, int ldx, long sX, int k,
-                                    int upper) {
-  const int j0 = blockIdx.x * kNB;
-  const int jb = min(kNB, k - j0);
-  const T* A = fronts + (long)blockIdx.y * m * m;
-  T* Xf = X + (long)blockIdx.y * sX;
-  __shared__ T Bk[kNB][kNB + 1];
-  for (int e = threadIdx.x; e < jb * jb; e += blockDim.x) {
-    int i = e % jb, l = e / jb;
-    Bk[i][l] = A[(j0 + i) + (long)(j0 + l) * m];
-  }
-  __syncthreads();
-  const int c = threadIdx.x;
-  if (c >= jb) return;
-  T x[kNB];
-#pragma unroll
-  for (int i = 0; i < kNB; ++i) x[i] = (i == c) ? (T)1 : (T)0;
-  if (!upper) {
-#pragma unroll
-    for (int i = 0; i < kNB; ++i)
-      if (i < jb) {
-        T acc = x[i];
-#pragma unroll
-        for (int l = 0; l < kNB; ++l)
-          if (l < i) acc -= Bk[i][l] * x[l];
-        x[i] = acc;
-      }
-  } else {
-#pragma unroll
-    for (int i = kNB - 1; i >= 0; --i)
-      if (i < jb) {
-        T acc = x[i];
-#pragma unroll
-        for (int l = 0; l < kNB; ++l)
-          if (l > i && l < jb) acc -= Bk[i][l] * x[l];
-        x[i] = acc / Bk[i][i];
-      }
-  }
-  T* col = Xf + j0 + (long)(j0 + c) * ldx;
-#pragma unroll
-  for (int i = 0; i < kNB; ++i)
-    if (i < jb) col[i] = x[i];
-}
-
-// In-place inversion of the 32 x 32 diagonal blocks of L11 (unit lower) and U11
-// (upper) of every front: afterwards the block's strict lower part holds the
-// block of L11^{-1} and its upper part (with the diagonal) the block of U11^{-1}.
-// The sweeps then resolve a diagonal block with a 32 x 32 matrix-vector product
-// instead of 32 dependent steps and 32 divisions.  One CTA (32 threads) per
-// (block, front); thread c computes column c of both inverses.
-template <class T>
-__global__ void diag32_inplace_kernel(T* fronts, int m, int k) {
+__global__ void __launch_bounds__(256) diag32_kernel(T* fronts, int m, int k, T* Xl, T* Xu, int ldx,
+                                                     long sX) {
   const int j0 = blockIdx.x * kNB;
   const int jb = min(kNB, k - j0);
   T* A = fronts + (long)blockIdx.y * m * m;
   __shared__ T Bk[kNB][kNB + 1];
-  for (int e = threadIdx.x; e < jb * jb; e += blockDim.x) {
-    int i = e % jb, l = e / jb;
-    Bk[i][l] = A[(j0 + i) + (long)(j0 + l) * m];
+  __shared__ T dinv[kNB];
+  for (int e = threadIdx.x; e < kNB * kNB; e += 256) {
+    const int i = e % kNB, l = e / kNB;
+    Bk[i][l] = (i < jb && l < jb) ? A[(j0 + i) + (long)(j0 + l) * m] : (i == l ? (T)1 : (T)0);
   }
   __syncthreads();
-  const int c = threadIdx.x;
-  T xl[kNB], xu[kNB];
+  if (threadIdx.x < kNB) dinv[threadIdx.x] = (T)1 / Bk[threadIdx.x][threadIdx.x];
+  __syncthreads();
+  const bool upper = threadIdx.x >= 128;
+  const int sub = threadIdx.x & 3, c = (threadIdx.x & 127) >> 2, base = threadIdx.x & 28;
+  constexpr int R = kNB / 4;
+  T x[R];
 #pragma unroll
-  for (int i = 0; i < kNB; ++i) xl[i] = xu[i] = (i == c) ? (T)1 : (T)0;
+  for (int r = 0; r < R; ++r) x[r] = 4 * r + sub == c ? (T)1 : (T)0;
+  if (!upper) {
 #pragma unroll
-  for (int i = 0; i < kNB; ++i)
-    if (i < jb) {
-      T acc = xl[i];
+    for (int l = 0; l < kNB - 1; ++l) {
+      const T xl = __shfl_sync(0xffffffffu, x[l >> 2], base | (l & 3));
 #pragma unroll
-      for (int l = 0; l < kNB; ++l)
-        if (l < i) acc -= Bk[i][l] * xl[l];
-      xl[i] = acc;
+      for (int r = l >> 2; r < R; ++r)
+        if (r > (l >> 2) || sub > (l & 3)) x[r] = fma(-Bk[4 * r + sub][l], xl, x[r]);
     }
+  } else {
 #pragma unroll
-  for (int i = kNB - 1; i >= 0; --i)
-    if (i < jb) {
-      T acc = xu[i];
+    for (int l = kNB - 1; l >= 0; --l) {
+      if (sub == (l & 3)) x[l >> 2] *= dinv[l];
+      const T xl = __shfl_sync(0xffffffffu, x[l >> 2], base | (l & 3));
 #pragma unroll
-      for (int l = 0; l < kNB; ++l)
-        if (l > i && l < jb) acc -= Bk[i][l] * xu[l];
-      xu[i] = acc / Bk[i][i];
+      for (int r = 0; r <= (l >> 2); ++r)
+        if (r < (l >> 2) || sub < (l & 3)) x[r] = fma(-Bk[4 * r + sub][l], xl, x[r]);
     }
+  }
   if (c >= jb) return;
-  T* col = A + j0 + (long)(j0 + c) * m;
+  T* out = Xl == nullptr ? A + j0 + (long)(j0 + c) * m
+                         : (upper ? Xu : Xl) + (long)blockIdx.y * sX + j0 + (long)(j0 + c) * ldx;
 #pragma unroll
-  for (int i = 0; i < kNB; ++i)
-    if (i < jb) col[i] = (i > c) ? xl[i] : xu[i];
+  for (int r = 0; r < R; ++r) {
+    const int i = 4 * r + sub;
+    if (i < jb && (Xl != nullptr || (i > c) != upper)) out[i] = x[r];
+  }
 }
 
 // F11 <- strict lower part of Linv, upper part (with the diagonal) of Uinv, on
 // the diagonal blocks of size Bsz only (the off-diagonal blocks keep L11, U11).
-// X entry (r, c) at r + c Bsz (front stride sX); one thread per block entry.
+// X entry (r, c) at r + c Bsz (front stride sX); one thread per entry of the blocks, whose
+// existing part is side x side.
 template <class T>
 __global__ void trinv_store_kernel(T* fronts, int m, const T* Xl, const T* Xu, long sX, int k,
-                                   int Bsz) {
+                                   int Bsz, int side) {
   const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long bb = (long)Bsz * Bsz;
+  const long bb = (long)side * side;
   const long blk = e / bb, rem = e % bb;
-  const long r = blk * Bsz + rem % Bsz, c = blk * Bsz + rem / Bsz;
+  const long r = blk * Bsz + rem % side, c = blk * Bsz + rem / side;
   if (r >= k || c >= k) return;
   const long f = blockIdx.y;
   const long x = f * sX + r + c * Bsz;
@@ -1837,8 +1807,7 @@ void invert_triangles(DevLevel& L, T* scratch, int Bsz, cudaStream_t st) {
   cudaMemsetAsync(Xu, 0, sizeof(T) * sX * nf, st);
   const int nb = (k + kNB - 1) / kNB;
   dim3 gd(nb, nf);
-  trinv_diag32_kernel<T><<<gd, kNB, 0, st>>>(F, m, Xl, ldx, sX, k, 0);
-  trinv_diag32_kernel<T><<<gd, kNB, 0, st>>>(F, m, Xu, ldx, sX, k, 1);
+  diag32_kernel<T><<<gd, 256, 0, st>>>(F, m, k, Xl, Xu, ldx, sX);
   for (int s = kNB; s < k && s < Bsz; s *= 2) {
     // pairs p: A at [2ps, 2ps+s), C at [2ps+s, min(2ps+2s, k)); the pairs with a
     // full-size C go in one batched launch (fronts x pairs), a ragged last pair in
@@ -1875,9 +1844,12 @@ void invert_triangles(DevLevel& L, T* scratch, int Bsz, cudaStream_t st) {
                   L.gen_tile);
     }
   }
+  // fronts with fewer than Bsz eliminated rows have one k x k block (threads over the
+  // whole Bsz x Bsz block of 4096 fronts with k = 25 took 3.2 ms)
+  const int side = std::min(k, Bsz);
   const long nbk = (k + Bsz - 1) / Bsz;
-  dim3 g((unsigned)((nbk * Bsz * Bsz + 255) / 256), nf);
-  trinv_store_kernel<T><<<g, 256, 0, st>>>(F, m, Xl, Xu, sX, k, Bsz);
+  dim3 g((unsigned)((nbk * side * side + 255) / 256), nf);
+  trinv_store_kernel<T><<<g, 256, 0, st>>>(F, m, Xl, Xu, sX, k, Bsz, side);
 }
 
 template <class T>
@@ -2320,7 +2292,7 @@ cudaError_t factor_level_t(int d, DevLevel& L, const DevLevel* child, const doub
     bw = (2.0 / 3.0) * (double)Bz * Bz * L.k * L.nf;
   } else {
     dim3 gd((L.k + kNB - 1) / kNB, L.nf);
-    diag32_inplace_kernel<T><<<gd, kNB, 0, st>>>(F, L.m, L.k);
+    diag32_kernel<T><<<gd, 256, 0, st>>>(F, L.m, L.k, (T*)nullptr, (T*)nullptr, 0, 0L);
     bw = (2.0 / 3.0) * (double)kNB * kNB * L.k * L.nf;
   }
   pi.done(bw, 1, st);
