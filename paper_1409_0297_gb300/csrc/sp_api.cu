@@ -870,11 +870,13 @@ static sp_status setup_impl(int d, int n, int b, int P, const double* shifts, sp
     // sweeps spread over the GPU; in the FP32 form every level does (the block
     // inverses cost little in FP32 and the sweeps become matrix-vector products)
     D.inv = D.nf < 152 || prec == SP_PREC_FP32 || vsz * (size_t)(S.m + S.k) > 192 * 1024;
-    // block inverses: 2048-wide blocks where the fronts are huge (the sweeps of the 3D
-    // root become 48 instead of 189 launch pairs; measured 3D 128^3 TF32: sweeps
-    // 1.95 -> 1.51 s per solve for +0.1 s of inversion), 512 elsewhere (in 2D the
-    // larger inverses cost more than the launches they save)
-    D.ib = c->opts.inv_block > 0 ? c->opts.inv_block : (S.k >= 32768 ? 2048 : kInvBlockSize);
+    // block inverses: wider blocks shorten the sweeps' chain (a launch pair per block and
+    // direction) and cost inversion work ~ k ib^2, so they pay where k is large.  Factor +
+    // solve at ib = 512 / 1024 / 2048: 3D 64^3 TF32 (k = 23816, 26 iterations) 200.6 / 191.8
+    // / 189.9 ms, 3D 32^3 FP64 (k = 5768, 13 iterations) 69.5 / 68.5 / 70.4 ms, 2D 512^2 FP32
+    // Schroedinger (k = 2044, 11 iterations) 16.7 / 17.4 / 17.2 ms
+    D.ib = c->opts.inv_block > 0 ? c->opts.inv_block
+                                 : (S.k >= 16384 ? 2048 : (S.k >= 4096 ? 1024 : kInvBlockSize));
     D.pdl = c->opts.launch_overlap;
     if (D.inv && c->opts.sweeps != 1) {
       int C = 0, NT = 0;
