@@ -31,9 +31,9 @@ namespace {
 
 typedef __nv_bfloat16 bf16;
 
-constexpr int kTP = 128;          // points per CTA of the pointwise kernels
-constexpr int kRowsCta = 64;      // grid rows per CTA of the row transform
+constexpr int kRowsCta = 128;     // grid rows per CTA of the row transform
 constexpr int kRowPitch = kRowsCta + 4;
+constexpr int kRowChunk = 32;     // points of a row staged at a time
 constexpr int kWgChunk = 2048;    // points per CTA of the weight-gradient reduction
 constexpr int kWgSub = 64;
 constexpr int kLossChunks = 64;   // CTAs per sample of the loss reduction
@@ -53,15 +53,42 @@ __device__ __forceinline__ float gelu_d(float x) {
          x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
+// four consecutive values (p a multiple of 4)
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 ld4(const bf16* p) {
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void st4(float* p, const float* v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void st4(bf16* p, const float* v) {
+  const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
+  uint2 u;
+  u.x = *reinterpret_cast<const unsigned*>(&a);
+  u.y = *reinterpret_cast<const unsigned*>(&b);
+  *reinterpret_cast<uint2*>(p) = u;
+}
+
+// The kernels below keep the order in which every output adds its products (inputs, modes
+// and points ascending), so a launch shape never changes a bit of the network.
+
 // ------------------------------------------------------------------ pointwise linear
-// Y[b][o][p] = act(sum_i Wt(o, i) X[b][i][p] + bias[o]), optionally times
-// gelu'(aux[b][o][p]).  Wt(o, i) = W[o ldw + i] (trans = 0) or W[i ldw + o] (trans = 1).
-// gelu: pre (if not null) receives the value before the activation.
-template <class TX, class TY, class TA>
+// Y[b][o][p] = act(sum_i W[o ldw + i] X[b][i][p] + bias[o]); gelu: pre receives the value
+// before the activation.  P is a multiple of 4 (n a multiple of 64); aligned: X starts on a
+// 16-byte boundary (a caller's input may not).
+// A CTA keeps the weights and a 128-point tile in shared memory; a thread owns 8 outputs x 4
+// points, so 32 FMAs take 3 shared loads (one point per thread took 3 for 8, and the shared
+// pipe bound it: width 32 -> 128 with GELU, 16 x 256^2 points: 489 us).  What bounds it now:
+// the FMAs and erff.
+constexpr int kTP = 128;
+template <class TX, class TY>
 __global__ void __launch_bounds__(kTP)
     chan_linear_kernel(const TX* __restrict__ X, int ci, const bf16* __restrict__ W, int ldw,
-                       int trans, const bf16* __restrict__ bias, int co, long P, int gelu,
-                       TY* __restrict__ pre, TY* __restrict__ Y, const TA* __restrict__ aux) {
+                       const bf16* __restrict__ bias, int co, long P, int gelu,
+                       TY* __restrict__ pre, TY* __restrict__ Y, int aligned) {
   extern __shared__ float4 smf4[];
   float* sm = reinterpret_cast<float*>(smf4);
   const int co8 = (co + 7) & ~7;
@@ -69,196 +96,366 @@ __global__ void __launch_bounds__(kTP)
   float* bs = Ws + ci * co8;  // [co8]
   float* Xs = bs + co8;       // [ci][kTP]
   for (int idx = threadIdx.x; idx < ci * co8; idx += kTP) {
-    const int i = idx / co8, o = idx % co8;
-    float w = 0.f;
-    if (o < co) w = __bfloat162float(trans ? W[(long)i * ldw + o] : W[(long)o * ldw + i]);
-    Ws[idx] = w;
+    const int o = idx / ci, i = idx - o * ci;
+    Ws[i * co8 + o] = o < co ? __bfloat162float(W[(long)o * ldw + i]) : 0.f;
   }
-  for (int o = threadIdx.x; o < co8; o += kTP)
-    bs[o] = (bias != nullptr && o < co) ? __bfloat162float(bias[o]) : 0.f;
+  for (int o = threadIdx.x; o < co8; o += kTP) bs[o] = o < co ? __bfloat162float(bias[o]) : 0.f;
   const int b = blockIdx.y;
-  const long p = (long)blockIdx.x * kTP + threadIdx.x;
-  const bool live = p < P;
   const TX* Xb = X + (long)b * ci * P;
-  for (int i = 0; i < ci; ++i) Xs[i * kTP + threadIdx.x] = live ? ldf(Xb + (long)i * P + p) : 0.f;
-  __syncthreads();
-  if (!live) return;
-  for (int o0 = 0; o0 < co; o0 += 8) {
-    float acc[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[j] = bs[o0 + j];
-    for (int i = 0; i < ci; ++i) {
-      const float x = Xs[i * kTP + threadIdx.x];
-      const float4 w0 = *reinterpret_cast<const float4*>(Ws + i * co8 + o0);
-      const float4 w1 = *reinterpret_cast<const float4*>(Ws + i * co8 + o0 + 4);
-      acc[0] = fmaf(w0.x, x, acc[0]);
-      acc[1] = fmaf(w0.y, x, acc[1]);
-      acc[2] = fmaf(w0.z, x, acc[2]);
-      acc[3] = fmaf(w0.w, x, acc[3]);
-      acc[4] = fmaf(w1.x, x, acc[4]);
-      acc[5] = fmaf(w1.y, x, acc[5]);
-      acc[6] = fmaf(w1.z, x, acc[6]);
-      acc[7] = fmaf(w1.w, x, acc[7]);
+  const int pg = threadIdx.x & 31, og = threadIdx.x >> 5;
+  for (long p0 = (long)blockIdx.x * kTP; p0 < P; p0 += (long)gridDim.x * kTP) {
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < ci * (kTP / 4); idx += kTP) {
+      const int i = idx >> 5, q = (idx & 31) * 4;
+      const TX* src = Xb + (long)i * P + p0 + q;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (p0 + q < P) {
+        if (aligned) v = ld4(src);
+        else v = make_float4(ldf(src), ldf(src + 1), ldf(src + 2), ldf(src + 3));
+      }
+      *reinterpret_cast<float4*>(Xs + i * kTP + q) = v;
     }
+    __syncthreads();
+    const long p = p0 + 4 * pg;
+    for (int o0 = og * 8; o0 < co8; o0 += 32) {
+      float acc[8][4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (o0 + j < co) {
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[j][q] = bs[o0 + j];
+#pragma unroll 4
+      for (int i = 0; i < ci; ++i) {
+        const float4 x = *reinterpret_cast<const float4*>(Xs + i * kTP + 4 * pg);
+        const float4 w0 = *reinterpret_cast<const float4*>(Ws + i * co8 + o0);
+        const float4 w1 = *reinterpret_cast<const float4*>(Ws + i * co8 + o0 + 4);
+        const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+        const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[j][q] = fmaf(wv[j], xv[q], acc[j][q]);
+      }
+      if (p >= P) continue;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (o0 + j >= co) break;
         const long idx = ((long)b * co + o0 + j) * P + p;
-        float v = acc[j];
         if (gelu) {
-          if (pre != nullptr) stf(pre + idx, v);
-          v = gelu_f(v);
+          if (pre != nullptr) st4(pre + idx, acc[j]);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[j][q] = gelu_f(acc[j][q]);
         }
-        if (aux != nullptr) v *= gelu_d(ldf(aux + idx));
-        stf(Y + idx, v);
+        st4(Y + idx, acc[j]);
       }
     }
   }
+}
+
+// The same for few outputs (the projection's last layer, CO <= 8): the inputs stream through
+// registers, four points per thread, and nothing but the weights is staged.  Bound by
+// reading X once (128 -> 2, 16 x 256^2 points, 268 MB: 330 us through the tile above, whose
+// outputs are padded to 8).
+template <class TX, int CO>
+__global__ void __launch_bounds__(128)
+    chan_narrow_kernel(const TX* __restrict__ X, int ci, const bf16* __restrict__ W, int ldw,
+                       const bf16* __restrict__ bias, int co, long P, float* __restrict__ Y) {
+  __shared__ float Ws[128 * CO];
+  for (int idx = threadIdx.x; idx < ci * CO; idx += 128) {
+    const int i = idx / CO, o = idx % CO;
+    Ws[idx] = o < co ? __bfloat162float(W[(long)o * ldw + i]) : 0.f;
+  }
+  __syncthreads();
+  const int b = blockIdx.y;
+  const long p = 4 * ((long)blockIdx.x * 128 + threadIdx.x);
+  if (p >= P) return;
+  float acc[CO][4];
+#pragma unroll
+  for (int o = 0; o < CO; ++o)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[o][q] = o < co ? __bfloat162float(bias[o]) : 0.f;
+  const TX* Xb = X + (long)b * ci * P + p;
+#pragma unroll 8
+  for (int i = 0; i < ci; ++i) {
+    const float4 x = ld4(Xb + (long)i * P);
+    const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int o = 0; o < CO; ++o)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[o][q] = fmaf(Ws[i * CO + o], xv[q], acc[o][q]);
+  }
+#pragma unroll
+  for (int o = 0; o < CO; ++o)
+    if (o < co) st4(Y + ((long)b * co + o) * P + p, acc[o]);
 }
 
 // ------------------------------------------------------------------ weight gradients
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // part[(b nchunk + chunk)][o ci + i] = sum over the chunk's points of dY[b][o][p] X[b][i][p],
-// part[..][co ci + o] = sum dY[b][o][p].  Each thread owns a 4 x 4 block of (o, i).
-// With Q2 != nullptr the rows are not read from dY but formed on the fly as the
-// projection's hidden-layer gradient de[h][p] = (sum_o Q2[o][h] dY[o][p]) gelu'(E[h][p])
-// (dY then has c2 channels, co = H), so de never goes to memory.
-template <class TX, class TE>
-__global__ void __launch_bounds__(256)
-    chan_wgrad_kernel(const float* __restrict__ dY, int co, const TX* __restrict__ X, int ci,
-                      long P, float* __restrict__ part, const TE* __restrict__ E,
-                      const bf16* __restrict__ Q2, int c2) {
+// part[..][co ci + o] = sum dY[b][o][p].  One CTA per chunk; thread t < own adds the points of
+// a 4 x 4 set of (o, i) in order (o = ob + r co4 / 4, i = ib + c ci4 / 4, so that a warp's
+// reads of a tile spread over the banks), one more warp the bias sums.  The chunk streams
+// through kWgStages tiles of kWgSub points in shared memory, channel-major as it lies in
+// device memory (cp.async, X still in its storage type).  With plain loads of one tile at a
+// time the reduction waited for memory (235 us per 32 x 32 layer at 16 x 256^2 points, whose
+// FMAs take 27).  aligned = 0 (a caller's X off the 16-byte grid) copies with plain loads.
+constexpr int kWgStages = 3;
+template <class TX>
+__global__ void __launch_bounds__(288)
+    chan_wgrad_kernel(const float* __restrict__ dY, int co, const TX* __restrict__ X, int ci, long P,
+                      float* __restrict__ part, int own, int aligned) {
   extern __shared__ float4 smf4[];
-  float* sm = reinterpret_cast<float*>(smf4);
+  constexpr int pY = kWgSub + 4, pX = kWgSub + 16 / (int)sizeof(TX);  // row pitches (16-byte rows)
   const int co4 = (co + 3) & ~3, ci4 = (ci + 3) & ~3;
-  const int pco = co4 + 4, pci = ci4 + 4;
-  float* sY = sm;                  // [kWgSub][pco]
-  float* sX = sY + kWgSub * pco;   // [kWgSub][pci]
-  float* sQ = sX + kWgSub * pci;   // [c2][co] (de mode)
-  if (Q2 != nullptr)
-    for (int idx = threadIdx.x; idx < c2 * co; idx += 256) sQ[idx] = __bfloat162float(Q2[idx]);
-  const int nib = ci4 / 4, nblk = (co4 / 4) * nib;
-  const int t = threadIdx.x;
-  const int ob = t / nib, ib = t % nib;
-  const bool owner = t < nblk;
-  float acc[16];
-  float accb[4];
-#pragma unroll
-  for (int j = 0; j < 16; ++j) acc[j] = 0.f;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) accb[j] = 0.f;
+  const size_t ybytes = (size_t)co4 * pY * sizeof(float), xbytes = (size_t)ci4 * pX * sizeof(TX);
+  unsigned char* sm = reinterpret_cast<unsigned char*>(smf4);
+  auto tY = [&](int st) { return reinterpret_cast<float*>(sm + st * (ybytes + xbytes)); };
+  auto tX = [&](int st) { return reinterpret_cast<TX*>(sm + st * (ybytes + xbytes) + ybytes); };
+  const int t = threadIdx.x, nth = blockDim.x;
+  const int nob = co4 / 4, nib = ci4 / 4;
+  const int ob = t / nib, ib = t - ob * nib;
+  const bool owner = t < nob * nib;
+  const int bt = t - own;  // bias channel of the extra warp's lanes
   const int b = blockIdx.y;
   const long c0 = (long)blockIdx.x * kWgChunk;
-  const long c1 = c0 + kWgChunk < P ? c0 + kWgChunk : P;
+  const long c1 = c0 + kWgChunk < P ? c0 + kWgChunk : P;  // P and kWgChunk are multiples of kWgSub
   const float* Yb = dY + (long)b * co * P;
   const TX* Xb = X + (long)b * ci * P;
-  __syncthreads();
-  for (long s0 = c0; s0 < c1; s0 += kWgSub) {
-    __syncthreads();
-    if (Q2 == nullptr) {
-      for (int idx = t; idx < co4 * kWgSub; idx += 256) {
-        const int o = idx / kWgSub, q = idx % kWgSub;
-        const long p = s0 + q;
-        sY[q * pco + o] = (o < co && p < c1) ? Yb[(long)o * P + p] : 0.f;
+  const int ntile = (int)((c1 - c0) / kWgSub);
+  // rows that pad the channels to a multiple of four stay zero
+  for (int st = 0; st < kWgStages; ++st) {
+    for (int e = t; e < (co4 - co) * pY; e += nth) tY(st)[co * pY + e] = 0.f;
+    for (int e = t; e < (ci4 - ci) * pX; e += nth) stf(tX(st) + ci * pX + e, 0.f);
+  }
+  auto fetch = [&](int tile) {
+    if (tile < ntile) {
+      const long p = c0 + (long)tile * kWgSub;
+      float* y = tY(tile % kWgStages);
+      TX* x = tX(tile % kWgStages);
+      constexpr int vY = 4, vX = 16 / (int)sizeof(TX);
+      for (int e = t; e < co * (kWgSub / vY); e += nth) {
+        const int o = e / (kWgSub / vY), q = vY * (e % (kWgSub / vY));
+        cp_async16(y + o * pY + q, Yb + (long)o * P + p + q);
       }
-    } else {
-      const float* Db = dY + (long)b * c2 * P;
-      const TE* Eb = E + (long)b * co * P;
-      for (int idx = t; idx < co4 * kWgSub; idx += 256) {
-        const int h = idx / kWgSub, q = idx % kWgSub;
-        const long p = s0 + q;
-        float v = 0.f;
-        if (h < co && p < c1) {
-          for (int o = 0; o < c2; ++o) v = fmaf(sQ[o * co + h], Db[(long)o * P + p], v);
-          v *= gelu_d(ldf(Eb + (long)h * P + p));
+      for (int e = t; e < ci * (kWgSub / vX); e += nth) {
+        const int i = e / (kWgSub / vX), q = vX * (e % (kWgSub / vX));
+        const TX* src = Xb + (long)i * P + p + q;
+        if (aligned) {
+          cp_async16(x + i * pX + q, src);
+        } else {
+#pragma unroll
+          for (int u = 0; u < vX; ++u) x[i * pX + q + u] = src[u];
         }
-        sY[q * pco + h] = v;
       }
     }
-    for (int idx = t; idx < ci4 * kWgSub; idx += 256) {
-      const int i = idx / kWgSub, q = idx % kWgSub;
-      const long p = s0 + q;
-      sX[q * pci + i] = (i < ci && p < c1) ? ldf(Xb + (long)i * P + p) : 0.f;
-    }
-    __syncthreads();
+    cp_commit();
+  };
+  float acc[16];
+  float accb = 0.f;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) acc[j] = 0.f;
+  for (int st = 0; st < kWgStages - 1; ++st) fetch(st);
+  for (int tile = 0; tile < ntile; ++tile) {
+    cp_wait<kWgStages - 2>();
+    __syncthreads();  // tile arrived; everyone is done with the stage that is refilled now
+    fetch(tile + kWgStages - 1);
+    const float* y = tY(tile % kWgStages);
+    const TX* x = tX(tile % kWgStages);
     if (owner) {
-      for (int q = 0; q < kWgSub; ++q) {
-        const float4 y = *reinterpret_cast<const float4*>(sY + q * pco + 4 * ob);
-        const float4 x = *reinterpret_cast<const float4*>(sX + q * pci + 4 * ib);
-        const float yv[4] = {y.x, y.y, y.z, y.w}, xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll 2
+      for (int q = 0; q < kWgSub; q += 4) {
+        float yv[4][4], xv[4][4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[r * 4 + c] = fmaf(yv[r], xv[c], acc[r * 4 + c]);
-          accb[r] += yv[r];
+          const float4 v = *reinterpret_cast<const float4*>(y + (ob + r * nob) * pY + q);
+          yv[r][0] = v.x, yv[r][1] = v.y, yv[r][2] = v.z, yv[r][3] = v.w;
+          const float4 w = ld4(x + (ib + r * nib) * pX + q);
+          xv[r][0] = w.x, xv[r][1] = w.y, xv[r][2] = w.z, xv[r][3] = w.w;
         }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[r * 4 + c] = fmaf(yv[r][u], xv[c][u], acc[r * 4 + c]);
+      }
+    } else if (bt >= 0 && bt < co) {
+#pragma unroll 4
+      for (int q = 0; q < kWgSub; q += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(y + bt * pY + q);
+        accb += v.x;
+        accb += v.y;
+        accb += v.z;
+        accb += v.w;
       }
     }
   }
+  cp_wait<0>();
+  float* out = part + ((long)b * gridDim.x + blockIdx.x) * (long)(co * ci + co);
   if (owner) {
-    float* out = part + ((long)b * gridDim.x + blockIdx.x) * (long)(co * ci + co);
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      const int o = 4 * ob + r;
+      const int o = ob + r * nob;
       if (o >= co) continue;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const int i = 4 * ib + c;
+        const int i = ib + c * nib;
         if (i < ci) out[o * ci + i] = acc[r * 4 + c];
       }
-      if (ib == 0) out[co * ci + o] = accb[r];
     }
   }
+  if (bt >= 0 && bt < co) out[co * ci + bt] = accb;
 }
 
-// Projection backward to the last layer's output: for every point,
-// de_h = (sum_o Q2[o][h] dy_o) gelu'(e_h) and dv_i = sum_h Q1[h][i] de_h (H <= 128,
-// W <= 32, c2 <= 8); de stays in registers.
+// Projection backward, both products of its hidden-layer gradient
+// de[h][p] = (sum_o Q2[o][h] dY[o][p]) gelu'(E[h][p]): the partial sums of dQ1 (rows h, as
+// chan_wgrad_kernel with the last layer's output v) and dv_i = sum_h Q1[h][i] de_h.  A tile of
+// de is formed once in shared memory and never goes to device memory (H <= 128, W <= 32,
+// c2 <= 8).  What bounds it: erff and expf of gelu'; formed twice, once for each product, the
+// two kernels took 1.70 ms at 16 x 256^2 points.
 template <class TA>
-__global__ void __launch_bounds__(kTP)
-    proj_bwd_kernel(const float* __restrict__ dy, int c2, const TA* __restrict__ e, int H,
-                    const bf16* __restrict__ Q2, const bf16* __restrict__ Q1, int W, long P,
-                    float* __restrict__ dv) {
-  __shared__ __align__(16) float Q1s[128 * 32];  // [h][i], row pitch 32
-  __shared__ float Q2s[8 * 128];                 // [o][h], row pitch 128
-  for (int idx = threadIdx.x; idx < 128 * 32; idx += kTP) {
+__global__ void __launch_bounds__(256)
+    proj_bwd_kernel(const float* __restrict__ dY, int c2, const TA* __restrict__ E, int H,
+                    const bf16* __restrict__ Q2, const bf16* __restrict__ Q1, const TA* __restrict__ V,
+                    int W, long P, float* __restrict__ dv, float* __restrict__ part) {
+  extern __shared__ float4 smf4[];
+  constexpr int pH = 132, pW = 36;  // row pitches: 16-byte rows, spread over the banks
+  float* sD = reinterpret_cast<float*>(smf4);  // [kWgSub][pH] de
+  float* sV = sD + kWgSub * pH;                // [kWgSub][pW] v
+  float* Q1s = sV + kWgSub * pW;               // [128][32]
+  float* Q2s = Q1s + 128 * 32;                 // [8][128]
+  const int t = threadIdx.x;
+  for (int idx = t; idx < 128 * 32; idx += 256) {
     const int h = idx >> 5, i = idx & 31;
     Q1s[idx] = (h < H && i < W) ? __bfloat162float(Q1[h * W + i]) : 0.f;
   }
-  for (int idx = threadIdx.x; idx < 8 * 128; idx += kTP) {
+  for (int idx = t; idx < 8 * 128; idx += 256) {
     const int o = idx >> 7, h = idx & 127;
     Q2s[idx] = (o < c2 && h < H) ? __bfloat162float(Q2[o * H + h]) : 0.f;
   }
-  __syncthreads();
+  const int ob = t >> 3, ib = t & 7;         // dQ1: rows 4 ob, columns 4 ib
+  const int q1 = t & 63, hg = t >> 6;        // de: point, rows 16 k + 4 hg + r
+  const int q2 = t & 31, i4 = 4 * (t >> 5);  // dv: points q2, q2 + 32, first of four channels
+  float acc[16];
+  float accb = 0.f;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) acc[j] = 0.f;
   const int b = blockIdx.y;
-  const long p = (long)blockIdx.x * kTP + threadIdx.x;
-  if (p >= P) return;
+  const long c0 = (long)blockIdx.x * kWgChunk;
+  const long c1 = c0 + kWgChunk < P ? c0 + kWgChunk : P;  // P and kWgChunk are multiples of kWgSub
+  const float* Db = dY + (long)b * c2 * P;
+  const TA* Eb = E + (long)b * H * P;
+  const TA* Vb = V + (long)b * W * P;
+  // the next tile's E, v and dY values travel while the current one is used
+  TA ev[32], vv[8];
   float d[8];
+  auto fetch = [&](long s0) {
+    const long p = s0 + q1;
 #pragma unroll
-  for (int o = 0; o < 8; ++o) d[o] = o < c2 ? dy[((long)b * c2 + o) * P + p] : 0.f;
-  float acc[32];
+    for (int o = 0; o < 8; ++o) d[o] = o < c2 ? Db[(long)o * P + p] : 0.f;
 #pragma unroll
-  for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-  const int W4 = (W + 3) >> 2;
-  const TA* eb = e + (long)b * H * P + p;
-  for (int h = 0; h < H; ++h) {
-    float a = 0.f;
+    for (int u = 0; u < 32; ++u) {
+      const int h = 16 * (u >> 2) + 4 * hg + (u & 3);
+      if (h < H) ev[u] = Eb[(long)h * P + p];
+    }
 #pragma unroll
-    for (int o = 0; o < 8; ++o) a = fmaf(Q2s[o * 128 + h], d[o], a);
-    const float de = a * gelu_d(ldf(eb + (long)h * P));
-    const float4* q = reinterpret_cast<const float4*>(Q1s + h * 32);
+    for (int u = 0; u < 8; ++u) {
+      const int i = 16 * (u >> 2) + 4 * hg + (u & 3);
+      if (i < W) vv[u] = Vb[(long)i * P + p];
+    }
+  };
+  fetch(c0);
+  for (long s0 = c0; s0 < c1; s0 += kWgSub) {
+    __syncthreads();
 #pragma unroll
-    for (int i4 = 0; i4 < 8; ++i4)
-      if (i4 < W4) {
-        const float4 w = q[i4];
-        acc[4 * i4] = fmaf(w.x, de, acc[4 * i4]);
-        acc[4 * i4 + 1] = fmaf(w.y, de, acc[4 * i4 + 1]);
-        acc[4 * i4 + 2] = fmaf(w.z, de, acc[4 * i4 + 2]);
-        acc[4 * i4 + 3] = fmaf(w.w, de, acc[4 * i4 + 3]);
+    for (int k = 0; k < 8; ++k) {
+      const int h = 16 * k + 4 * hg;
+      float v[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        v[r] = 0.f;
+        if (h + r < H) {
+          float a = 0.f;
+#pragma unroll
+          for (int o = 0; o < 8; ++o)
+            if (o < c2) a = fmaf(Q2s[o * 128 + h + r], d[o], a);
+          v[r] = a * gelu_d(ldf(&ev[4 * k + r]));
+        }
       }
-  }
+      *reinterpret_cast<float4*>(sD + q1 * pH + h) = make_float4(v[0], v[1], v[2], v[3]);
+    }
 #pragma unroll
-  for (int i = 0; i < 32; ++i)
-    if (i < W) dv[((long)b * W + i) * P + p] = acc[i];
+    for (int k = 0; k < 2; ++k) {
+      const int i = 16 * k + 4 * hg;
+      float v[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) v[r] = i + r < W ? ldf(&vv[4 * k + r]) : 0.f;
+      *reinterpret_cast<float4*>(sV + q1 * pW + i) = make_float4(v[0], v[1], v[2], v[3]);
+    }
+    if (s0 + kWgSub < c1) fetch(s0 + kWgSub);
+    __syncthreads();
+    float dvr[4][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) dvr[j][0] = dvr[j][1] = 0.f;
+    // four rows h at a time (the rows past H hold zeros), one 16-byte load per point
+#pragma unroll 2
+    for (int h = 0; h < H; h += 4) {
+      const float4 a = *reinterpret_cast<const float4*>(sD + q2 * pH + h);
+      const float4 c = *reinterpret_cast<const float4*>(sD + (q2 + 32) * pH + h);
+      const float av[4] = {a.x, a.y, a.z, a.w}, cv[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 w = *reinterpret_cast<const float4*>(Q1s + (h + u) * 32 + i4);
+        const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          dvr[j][0] = fmaf(wv[j], av[u], dvr[j][0]);
+          dvr[j][1] = fmaf(wv[j], cv[u], dvr[j][1]);
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (i4 + j < W) {
+        float* out = dv + ((long)b * W + i4 + j) * P + s0 + q2;
+        out[0] = dvr[j][0];
+        out[32] = dvr[j][1];
+      }
+#pragma unroll 4
+    for (int q = 0; q < kWgSub; ++q) {
+      const float4 y = *reinterpret_cast<const float4*>(sD + q * pH + 4 * ob);
+      const float4 x = *reinterpret_cast<const float4*>(sV + q * pW + 4 * ib);
+      const float yv[4] = {y.x, y.y, y.z, y.w}, xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r * 4 + c] = fmaf(yv[r], xv[c], acc[r * 4 + c]);
+    }
+    if (t < H)
+#pragma unroll 16
+      for (int q = 0; q < kWgSub; ++q) accb += sD[q * pH + t];
+  }
+  float* out = part + ((long)b * gridDim.x + blockIdx.x) * (long)(H * W + H);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int h = 4 * ob + r;
+    if (h >= H) continue;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int i = 4 * ib + c;
+      if (i < W) out[h * W + i] = acc[r * 4 + c];
+    }
+  }
+  if (t < H) out[H * W + t] = accb;
 }
 
 // grad[j] = sum over the nparts partials (fixed order) of part[k][j], j < len
@@ -273,54 +470,78 @@ __global__ void sum_parts_kernel(const float* __restrict__ part, int nparts, int
 
 // ------------------------------------------------------------------ truncated DFT
 // Rows: A[row][kx] = sum_j0 X[row][j0] e^{-2 pi i kx j0 / n}, row = (b C + c) n + j1.
-// Thread (kx, row group of 4) with the rows staged transposed, x[j0][row].
+// 128 rows per CTA, 32 points of them staged at a time (transposed, x[j0][row]); a thread
+// owns two modes of eight rows: 32 FMAs for three 16-byte shared loads (one mode of four
+// rows: 8 for two, 125 us at 16 x 32 x 256 rows of 256).
 template <class TX>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(128, sizeof(TX) == 4 ? 3 : 4)
     dft_rows_fwd_kernel(const TX* __restrict__ X, long rows, int n, int M,
                         const float2* __restrict__ twr, float2* __restrict__ A) {
-  extern __shared__ float4 smf4[];
-  float* xs = reinterpret_cast<float*>(smf4);                 // [n][kRowPitch]
-  float2* tw = reinterpret_cast<float2*>(xs + n * kRowPitch);  // [n][16]
+  __shared__ __align__(16) float xs[kRowChunk * kRowPitch];
+  __shared__ __align__(16) float2 tw[kRowChunk * 16];
   const long r0 = (long)blockIdx.x * kRowsCta;
-  const int t = threadIdx.x;
-  for (int idx = t; idx < n * 16; idx += 256) tw[idx] = twr[idx];
-  for (int idx = t; idx < n * (kRowsCta / 4); idx += 256) {
-    const int j0 = idx % n, g = idx / n;
-    const long r = r0 + 4 * g;
-    float4 v;
-    v.x = r + 0 < rows ? ldf(X + (r + 0) * n + j0) : 0.f;
-    v.y = r + 1 < rows ? ldf(X + (r + 1) * n + j0) : 0.f;
-    v.z = r + 2 < rows ? ldf(X + (r + 2) * n + j0) : 0.f;
-    v.w = r + 3 < rows ? ldf(X + (r + 3) * n + j0) : 0.f;
-    *reinterpret_cast<float4*>(xs + j0 * kRowPitch + 4 * g) = v;
-  }
-  __syncthreads();
-  const int kx = t & 15, rg = t >> 4;
-  if (kx >= M) return;
-  float ar[4] = {0.f, 0.f, 0.f, 0.f}, ai[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int j0 = 0; j0 < n; ++j0) {
-    const float4 x = *reinterpret_cast<const float4*>(xs + j0 * kRowPitch + 4 * rg);
-    const float2 w = tw[j0 * 16 + kx];
-    ar[0] = fmaf(x.x, w.x, ar[0]);
-    ai[0] = fmaf(x.x, w.y, ai[0]);
-    ar[1] = fmaf(x.y, w.x, ar[1]);
-    ai[1] = fmaf(x.y, w.y, ai[1]);
-    ar[2] = fmaf(x.z, w.x, ar[2]);
-    ai[2] = fmaf(x.z, w.y, ai[2]);
-    ar[3] = fmaf(x.w, w.x, ar[3]);
-    ai[3] = fmaf(x.w, w.y, ai[3]);
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int kp = t & 7, rg = t >> 3;  // modes 2 kp, 2 kp + 1 of rows 8 rg ..
+  float ar[2][8], ai[2][8];
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) ar[u][q] = ai[u][q] = 0.f;
+  // the next chunk's values travel while the current one is multiplied
+  TX pre[kRowsCta / 4];
+  auto fetch = [&](int c0) {
+#pragma unroll
+    for (int u = 0; u < kRowsCta / 4; ++u) {
+      const long r = r0 + 16 * (u >> 2) + 4 * warp + (u & 3);
+      if (r < rows) pre[u] = X[r * n + c0 + lane];
+    }
+  };
+  fetch(0);
+  for (int c0 = 0; c0 < n; c0 += kRowChunk) {
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < kRowsCta / 16; ++v) {
+      float4 x;
+      const long r = r0 + 16 * v + 4 * warp;
+      x.x = r + 0 < rows ? ldf(&pre[4 * v]) : 0.f;
+      x.y = r + 1 < rows ? ldf(&pre[4 * v + 1]) : 0.f;
+      x.z = r + 2 < rows ? ldf(&pre[4 * v + 2]) : 0.f;
+      x.w = r + 3 < rows ? ldf(&pre[4 * v + 3]) : 0.f;
+      *reinterpret_cast<float4*>(xs + lane * kRowPitch + 16 * v + 4 * warp) = x;
+    }
+    for (int idx = t; idx < kRowChunk * 16; idx += 128) tw[idx] = twr[c0 * 16 + idx];
+    if (c0 + kRowChunk < n) fetch(c0 + kRowChunk);
+    __syncthreads();
+#pragma unroll 4
+    for (int j = 0; j < kRowChunk; ++j) {
+      const float4 x0 = *reinterpret_cast<const float4*>(xs + j * kRowPitch + 8 * rg);
+      const float4 x1 = *reinterpret_cast<const float4*>(xs + j * kRowPitch + 8 * rg + 4);
+      const float4 w = *reinterpret_cast<const float4*>(tw + j * 16 + 2 * kp);
+      const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        ar[0][q] = fmaf(xv[q], w.x, ar[0][q]);
+        ai[0][q] = fmaf(xv[q], w.y, ai[0][q]);
+        ar[1][q] = fmaf(xv[q], w.z, ar[1][q]);
+        ai[1][q] = fmaf(xv[q], w.w, ai[1][q]);
+      }
+    }
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const long r = r0 + 4 * rg + q;
-    if (r < rows) A[r * M + kx] = make_float2(ar[q], ai[q]);
+  for (int q = 0; q < 8; ++q) {
+    const long r = r0 + 8 * rg + q;
+    if (r >= rows) continue;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (2 * kp + u < M) A[r * M + 2 * kp + u] = make_float2(ar[u][q], ai[u][q]);
   }
 }
 
 __device__ __forceinline__ int ky_of(int kq, int n, int M) { return kq < M ? kq : n - 2 * M + kq; }
 
 // Columns: V[bc][ky'][kx] = s_kx sum_j1 A[bc][j1][kx] e^{-2 pi i ky j1 / n}
-// (s_0 = s0, s_kx = s1 for kx >= 1); one CTA per (b, c).
+// (s_0 = s0, s_kx = s1 for kx >= 1); one CTA per (b, c), a thread its two modes
+// ky' = g, g + 16 of a kx together (one load of A for both).
 __global__ void __launch_bounds__(256)
     dft_cols_fwd_kernel(const float2* __restrict__ A, int n, int M, const float2* __restrict__ twb,
                         float s0, float s1, float2* __restrict__ V) {
@@ -333,63 +554,85 @@ __global__ void __launch_bounds__(256)
   for (int idx = t; idx < n; idx += 256) tb[idx] = twb[idx];
   __syncthreads();
   const int kx = t & 15, g = t >> 4;
-  if (kx >= M) return;
   const int K2 = 2 * M;
+  if (kx >= M || g >= K2) return;
   const float s = kx == 0 ? s0 : s1;
-  for (int kq = g; kq < K2; kq += 16) {
-    const int ky = ky_of(kq, n, M);
-    float re = 0.f, im = 0.f;
-    int e = 0;
-    for (int j1 = 0; j1 < n; ++j1) {
-      const float2 a = As[j1 * M + kx], w = tb[e];
-      re = fmaf(a.x, w.x, fmaf(-a.y, w.y, re));
-      im = fmaf(a.x, w.y, fmaf(a.y, w.x, im));
-      e += ky;
-      if (e >= n) e -= n;
-    }
-    V[(bc * K2 + kq) * M + kx] = make_float2(s * re, s * im);
+  const int kb = g + 16;
+  const int ka = ky_of(g, n, M), kc = kb < K2 ? ky_of(kb, n, M) : 0;
+  float re[2] = {0.f, 0.f}, im[2] = {0.f, 0.f};
+  int e0 = 0, e1 = 0;
+#pragma unroll 4
+  for (int j1 = 0; j1 < n; ++j1) {
+    const float2 a = As[j1 * M + kx], w = tb[e0], v = tb[e1];
+    re[0] = fmaf(a.x, w.x, fmaf(-a.y, w.y, re[0]));
+    im[0] = fmaf(a.x, w.y, fmaf(a.y, w.x, im[0]));
+    re[1] = fmaf(a.x, v.x, fmaf(-a.y, v.y, re[1]));
+    im[1] = fmaf(a.x, v.y, fmaf(a.y, v.x, im[1]));
+    e0 += ka;
+    if (e0 >= n) e0 -= n;
+    e1 += kc;
+    if (e1 >= n) e1 -= n;
   }
+  V[(bc * K2 + g) * M + kx] = make_float2(s * re[0], s * im[0]);
+  if (kb < K2) V[(bc * K2 + kb) * M + kx] = make_float2(s * re[1], s * im[1]);
 }
 
 // Columns, inverse: Bc[bc][j1][kx] = sum_ky' Y[bc][ky'][kx] e^{+2 pi i ky j1 / n}.
-// Thread (kx, g) owns the n / 16 rows j1 = g, g + 16, ...; the twiddle index of a mode
-// advances by 16 ky (mod n) from one of its rows to the next.  n % 16 == 0.
+// Thread (kx, g) owns the rows j1 = g, g + 16, ... of its CTA's share of the rows
+// (blockIdx.y, RT rows a thread) for NC channels, which share every twiddle load; the
+// twiddle index of a mode advances by 16 ky (mod n) from one of its rows to the next.
+// n % 64 == 0.  NC = 2, RT = n / 16 for a training batch (74 us a call with one channel),
+// NC = 1 and the rows over four CTAs for a single sample (35 us with one CTA per channel).
+template <int NC, int RT>
 __global__ void __launch_bounds__(256)
-    dft_cols_inv_kernel(const float2* __restrict__ Y, int n, int M, const float2* __restrict__ twb,
-                        float2* __restrict__ Bc) {
+    dft_cols_inv_kernel(const float2* __restrict__ Y, int n, int M, int nbc,
+                        const float2* __restrict__ twb, float2* __restrict__ Bc) {
   extern __shared__ float4 smf4[];
   const int K2 = 2 * M;
-  float2* Ys = reinterpret_cast<float2*>(smf4);  // [2M][M]
-  float2* tb = Ys + K2 * M;                       // [n]
-  const long bc = blockIdx.x;
+  float2* Ys = reinterpret_cast<float2*>(smf4);  // [NC][2M][M]
+  float2* tb = Ys + NC * K2 * M;                  // [n]
+  const long bc = (long)blockIdx.x * NC;
   const int t = threadIdx.x;
-  for (int idx = t; idx < K2 * M; idx += 256) Ys[idx] = Y[bc * K2 * M + idx];
+  const int have = min(NC, (int)(nbc - bc));
+  for (int idx = t; idx < have * K2 * M; idx += 256) Ys[idx] = Y[bc * K2 * M + idx];
   for (int idx = t; idx < n; idx += 256) tb[idx] = twb[idx];
   __syncthreads();
   const int kx = t & 15, g = t >> 4;
   if (kx >= M) return;
-  const int R = n >> 4;  // rows per thread, <= 32
-  float re[32], im[32];
+  const int R = n >> 4;                      // rows per (kx, g) over all CTAs
+  const int first = blockIdx.y * RT;         // rows g + 16 (first + r), r < RT
+  const int last = min(R, first + RT) - first;
+  float re[NC][RT], im[NC][RT];
 #pragma unroll
-  for (int r = 0; r < 32; ++r) re[r] = im[r] = 0.f;
+  for (int c = 0; c < NC; ++c)
+#pragma unroll
+    for (int r = 0; r < RT; ++r) re[c][r] = im[c][r] = 0.f;
   for (int kq = 0; kq < K2; ++kq) {
     const int ky = ky_of(kq, n, M);
-    const float2 y = Ys[kq * M + kx];
-    int e = (int)(((long)ky * g) % n);
+    float2 y[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) y[c] = c < have ? Ys[(c * K2 + kq) * M + kx] : make_float2(0.f, 0.f);
+    int e = (int)(((long)ky * (g + 16 * first)) % n);
     const int step = (int)(((long)ky * 16) % n);
 #pragma unroll
-    for (int r = 0; r < 32; ++r)
-      if (r < R) {
+    for (int r = 0; r < RT; ++r)
+      if (r < last) {
         const float2 w = tb[e];  // e^{+i theta} = conj(w)
-        re[r] = fmaf(y.x, w.x, fmaf(y.y, w.y, re[r]));
-        im[r] = fmaf(y.y, w.x, fmaf(-y.x, w.y, im[r]));
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          re[c][r] = fmaf(y[c].x, w.x, fmaf(y[c].y, w.y, re[c][r]));
+          im[c][r] = fmaf(y[c].y, w.x, fmaf(-y[c].x, w.y, im[c][r]));
+        }
         e += step;
         if (e >= n) e -= n;
       }
   }
 #pragma unroll
-  for (int r = 0; r < 32; ++r)
-    if (r < R) Bc[(bc * n + g + 16 * r) * M + kx] = make_float2(re[r], im[r]);
+  for (int c = 0; c < NC; ++c)
+#pragma unroll
+    for (int r = 0; r < RT; ++r)
+      if (c < have && r < last)
+        Bc[((bc + c) * n + g + 16 * (first + r)) * M + kx] = make_float2(re[c][r], im[c][r]);
 }
 
 // Mode mixing: Y[b][o][k] = sum_i V[b][i][k] R[k][i][o]; one CTA per mode k.
@@ -462,73 +705,90 @@ __global__ void __launch_bounds__(256)
 
 // Layer output: out[b][o][j1][j0] = sum_i Wt(o, i) X[b][i][j1][j0] + bias[o]
 //   + sum_kx w_kx Re(Bc[b][o][j1][kx] e^{+2 pi i kx j0 / n}),  w_0 = w0, w_kx = w1;
-// with gelu, pre <- the value and out <- gelu(value).  One CTA per grid row (b, j1);
-// a thread keeps its point's C inputs and M twiddles in registers and reads the
-// weight row and the row's spectral coefficients as float4 broadcasts.  C <= 32, M <= 16.
-template <class TX, class TY>
-__global__ void __launch_bounds__(256)
+// with gelu, pre <- the value and out <- gelu(value).  C <= 32, M <= 16.
+// One product of depth C + 2 M per grid row: a CTA of n threads keeps the scaled twiddles of
+// all points and one row's inputs in shared memory (2 x 32 x n floats) and walks `rows` grid
+// rows; a thread owns 8 outputs x 4 points (32 FMAs for 3 shared loads; with one point per
+// thread a load fed 4 and a single chain of 64 FMAs: 354 us at 16 x 256^2 with GELU).
+template <class TX, class TY, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 3 : 1)
     combine_kernel(const TX* __restrict__ X, int C, const bf16* __restrict__ W, int trans,
                    const bf16* __restrict__ bias, const float2* __restrict__ Bc, int n, int M,
                    const float2* __restrict__ twr, float w0, float w1, int gelu,
-                   TY* __restrict__ pre, TY* __restrict__ out) {
-  __shared__ __align__(16) float Ws[32 * 32];   // [o][i], row pitch 32
-  __shared__ float bs[32];
-  __shared__ __align__(16) float2 Bs[32 * 16];  // [o][kx], row pitch 16
-  const int j1 = blockIdx.x, b = blockIdx.y, t = threadIdx.x;
+                   TY* __restrict__ pre, TY* __restrict__ out, int rows) {
+  extern __shared__ float4 smf4[];
+  float* xs = reinterpret_cast<float*>(smf4);  // [32][n]
+  float* ts = xs + 32 * n;                     // [32][n]: rows 2 kx (cos), 2 kx + 1 (-sin), scaled
+  __shared__ __align__(16) float Ws[32 * 32];  // [i][o]
+  __shared__ __align__(16) float Bs[32 * 32];  // [2 kx + (0: re, 1: im)][o]
+  __shared__ __align__(16) float bs[32];
+  const int b = blockIdx.y, t = threadIdx.x;
   for (int idx = t; idx < 32 * 32; idx += blockDim.x) {
-    const int o = idx >> 5, i = idx & 31;
+    const int i = idx >> 5, o = idx & 31;
     float w = 0.f;
     if (o < C && i < C) w = __bfloat162float(trans ? W[i * C + o] : W[o * C + i]);
     Ws[idx] = w;
   }
   for (int o = t; o < 32; o += blockDim.x)
     bs[o] = (bias != nullptr && o < C) ? __bfloat162float(bias[o]) : 0.f;
-  for (int idx = t; idx < 32 * 16; idx += blockDim.x) {
-    const int o = idx >> 4, kx = idx & 15;
-    Bs[idx] = (o < C && kx < M) ? Bc[(((long)b * C + o) * n + j1) * M + kx] : make_float2(0.f, 0.f);
+  for (int idx = t; idx < 16 * n; idx += blockDim.x) {
+    const int j0 = idx >> 4, kx = idx & 15;
+    const float2 w = kx < M ? twr[idx] : make_float2(0.f, 0.f);
+    const float s = kx == 0 ? w0 : w1;
+    ts[(2 * kx) * n + j0] = s * w.x;
+    ts[(2 * kx + 1) * n + j0] = s * w.y;
   }
-  __syncthreads();
   const long P = (long)n * n;
-  const int C4 = (C + 3) >> 2, M2 = (M + 1) >> 1;
-  for (int j0 = t; j0 < n; j0 += blockDim.x) {
-    const long p = (long)j1 * n + j0;
-    float x[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) x[i] = i < C ? ldf(X + ((long)b * C + i) * P + p) : 0.f;
-    float2 tw[16];
-#pragma unroll
-    for (int kx = 0; kx < 16; ++kx) {
-      float2 w = kx < M ? twr[j0 * 16 + kx] : make_float2(0.f, 0.f);
-      const float s = kx == 0 ? w0 : w1;
-      tw[kx] = make_float2(s * w.x, s * w.y);
+  const int ng = n >> 2;  // point groups of four
+  const int og = t / ng, j0 = 4 * (t - og * ng), o0 = 8 * og;
+  const int j1e = min(n, (int)(blockIdx.x + 1) * rows);
+  for (int j1 = blockIdx.x * rows; j1 < j1e; ++j1) {
+    __syncthreads();
+    for (int idx = t; idx < C * ng; idx += blockDim.x) {
+      const int i = idx / ng, q = 4 * (idx - i * ng);
+      *reinterpret_cast<float4*>(xs + i * n + q) = ld4(X + ((long)b * C + i) * P + (long)j1 * n + q);
     }
-    for (int o = 0; o < C; ++o) {
-      float acc = bs[o];
-      const float4* wr = reinterpret_cast<const float4*>(Ws + o * 32);
+    for (int idx = t; idx < 32 * 16; idx += blockDim.x) {
+      const int o = idx >> 4, kx = idx & 15;
+      const float2 v = (o < C && kx < M) ? Bc[(((long)b * C + o) * n + j1) * M + kx] : make_float2(0.f, 0.f);
+      Bs[(2 * kx) * 32 + o] = v.x;
+      Bs[(2 * kx + 1) * 32 + o] = v.y;
+    }
+    __syncthreads();
+    float acc[8][4];
 #pragma unroll
-      for (int i4 = 0; i4 < 8; ++i4)
-        if (i4 < C4) {
-          const float4 w = wr[i4];
-          acc = fmaf(w.x, x[4 * i4], acc);
-          acc = fmaf(w.y, x[4 * i4 + 1], acc);
-          acc = fmaf(w.z, x[4 * i4 + 2], acc);
-          acc = fmaf(w.w, x[4 * i4 + 3], acc);
-        }
-      // Re(B e^{+i theta}) with tw = s e^{-i theta}
-      const float4* br = reinterpret_cast<const float4*>(Bs + o * 16);
+    for (int j = 0; j < 8; ++j)
 #pragma unroll
-      for (int k2 = 0; k2 < 8; ++k2)
-        if (k2 < M2) {
-          const float4 bb = br[k2];
-          acc = fmaf(bb.x, tw[2 * k2].x, fmaf(bb.y, tw[2 * k2].y, acc));
-          acc = fmaf(bb.z, tw[2 * k2 + 1].x, fmaf(bb.w, tw[2 * k2 + 1].y, acc));
-        }
-      const long idx = ((long)b * C + o) * P + p;
+      for (int q = 0; q < 4; ++q) acc[j][q] = bs[o0 + j];
+    auto step = [&](const float* a, const float* v) {
+      const float4 a0 = *reinterpret_cast<const float4*>(a + o0);
+      const float4 a1 = *reinterpret_cast<const float4*>(a + o0 + 4);
+      const float4 x = *reinterpret_cast<const float4*>(v + j0);
+      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[j][q] = fmaf(av[j], xv[q], acc[j][q]);
+    };
+#pragma unroll 2
+    for (int i = 0; i < C; ++i) step(Ws + i * 32, xs + i * n);
+    // Re(B e^{+i theta}) with the twiddles s e^{-i theta}: the imaginary product first
+#pragma unroll 1
+    for (int kx = 0; kx < M; ++kx) {
+      step(Bs + (2 * kx + 1) * 32, ts + (2 * kx + 1) * n);
+      step(Bs + (2 * kx) * 32, ts + (2 * kx) * n);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (o0 + j >= C) break;
+      const long idx = ((long)b * C + o0 + j) * P + (long)j1 * n + j0;
       if (gelu) {
-        if (pre != nullptr) stf(pre + idx, acc);
-        acc = gelu_f(acc);
+        if (pre != nullptr) st4(pre + idx, acc[j]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[j][q] = gelu_f(acc[j][q]);
       }
-      stf(out + idx, acc);
+      st4(out + idx, acc[j]);
     }
   }
 }
@@ -576,19 +836,26 @@ __global__ void __launch_bounds__(256)
 // loss = mean_b S1_b / S2_b; scale[b] = 2 / (B S2_b) (the gradient factor); rel[b] = sqrt(S1/S2)
 __global__ void loss_finish_kernel(const double2* __restrict__ part, int B, int nchunk,
                                    double* __restrict__ loss, float* __restrict__ scale) {
-  if (threadIdx.x != 0) return;
-  double L = 0.0;
-  for (int b = 0; b < B; ++b) {
+  // one thread per sample adds its chunks in order, then one adds the samples
+  __shared__ double rs[256];
+  const int b = threadIdx.x;
+  if (b < B) {
     double s1 = 0.0, s2 = 0.0;
+#pragma unroll 16
     for (int c = 0; c < nchunk; ++c) {
-      s1 += part[(long)b * nchunk + c].x;
-      s2 += part[(long)b * nchunk + c].y;
+      const double2 v = part[(long)b * nchunk + c];
+      s1 += v.x;
+      s2 += v.y;
     }
-    const double r = s2 > 0.0 ? s1 / s2 : 0.0;
-    L += r;
+    rs[b] = s2 > 0.0 ? s1 / s2 : 0.0;
     scale[b] = s2 > 0.0 ? (float)(2.0 / (B * s2)) : 0.f;
   }
-  *loss = L / B;
+  __syncthreads();
+  if (b == 0) {
+    double L = 0.0;
+    for (int i = 0; i < B; ++i) L += rs[i];
+    *loss = L / B;
+  }
 }
 
 __global__ void loss_grad_kernel(const float* __restrict__ y, const float* __restrict__ t, long len,
@@ -645,13 +912,21 @@ __global__ void __launch_bounds__(256)
 }
 
 __global__ void scale_kernel(const double* __restrict__ part, int nb, long N, double2* __restrict__ c) {
-  if (threadIdx.x != 0) return;
-  double s = 0.0, sr = 0.0, si = 0.0;
-  for (int i = 0; i < nb; ++i) {
-    s += part[3 * i];
-    sr += part[3 * i + 1];
-    si += part[3 * i + 2];
+  // the partial sums staged at once, each of the three sums added in order by a thread of
+  // its own (as one thread's chain of loads: 43 us)
+  __shared__ double ps[3 * kNormBlocks];
+  __shared__ double sum[3];
+  for (int i = threadIdx.x; i < 3 * nb; i += blockDim.x) ps[i] = part[i];
+  __syncthreads();
+  if (threadIdx.x % 32 == 0 && threadIdx.x < 96) {
+    const int j = threadIdx.x / 32;
+    double a = 0.0;
+    for (int i = 0; i < nb; ++i) a += ps[3 * i + j];
+    sum[j] = a;
   }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const double s = sum[0], sr = sum[1], si = sum[2];
   const double sigma = sqrt(s / (double)N);
   const double phi = (sr == 0.0 && si == 0.0) ? 0.0 : 0.5 * atan2(si, sr);
   *c = make_double2(sigma * cos(phi), sigma * sin(phi));
@@ -801,59 +1076,51 @@ sp_status cuda_st(cudaError_t e) {
     if (e_ != cudaSuccess) return cuda_st(e_); \
   } while (0)
 
-constexpr size_t kLinSmemMax = (128 * kTP + 128 * 128 + 128) * sizeof(float);
-constexpr size_t kWgSmemMax = ((size_t)kWgSub * (132 + 132) + 8 * 128) * sizeof(float);
-constexpr size_t kRowsSmemMax = 512 * kRowPitch * sizeof(float) + 512 * 16 * sizeof(float2);
+constexpr size_t kProjSmem = ((size_t)kWgSub * (132 + 36) + 128 * 32 + 8 * 128) * sizeof(float);
+constexpr size_t kWgSmemMax = 200 * 1024;  // staged tiles of a weight-gradient CTA
 constexpr size_t kColsSmemMax = (512 * 16 + 512) * sizeof(float2);
+constexpr size_t kCombineSmemMax = 64 * 512 * sizeof(float);
 
 template <class TA>
 cudaError_t set_attrs(int mixB, int W) {
   cudaError_t e;
   const size_t mix = (size_t)(W * W + 2 * mixB * W) * sizeof(float2);
-  if ((e = cudaFuncSetAttribute(chan_linear_kernel<float, TA, TA>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLinSmemMax))) return e;
-  if ((e = cudaFuncSetAttribute(chan_linear_kernel<TA, TA, TA>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLinSmemMax))) return e;
-  if ((e = cudaFuncSetAttribute(chan_linear_kernel<TA, float, TA>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLinSmemMax))) return e;
-  if ((e = cudaFuncSetAttribute(chan_wgrad_kernel<TA, float>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmemMax))) return e;
-  if ((e = cudaFuncSetAttribute(chan_wgrad_kernel<TA, TA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)kWgSmemMax))) return e;
-  if ((e = cudaFuncSetAttribute(chan_wgrad_kernel<float, float>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmemMax))) return e;
-  if ((e = cudaFuncSetAttribute(dft_rows_fwd_kernel<TA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)kRowsSmemMax))) return e;
-  if ((e = cudaFuncSetAttribute(dft_rows_fwd_kernel<float>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmemMax))) return e;
-  if ((e = cudaFuncSetAttribute(dft_cols_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)kColsSmemMax))) return e;
-  if ((e = cudaFuncSetAttribute(dft_cols_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)kColsSmemMax))) return e;
-  if ((e = cudaFuncSetAttribute(spec_mix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mix))) return e;
-  return cudaFuncSetAttribute(spec_mix_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mix);
+  const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if ((e = cudaFuncSetAttribute(chan_wgrad_kernel<TA>, at, (int)kWgSmemMax))) return e;
+  if ((e = cudaFuncSetAttribute(chan_wgrad_kernel<float>, at, (int)kWgSmemMax))) return e;
+  if ((e = cudaFuncSetAttribute(proj_bwd_kernel<TA>, at, (int)kProjSmem))) return e;
+  if ((e = cudaFuncSetAttribute(combine_kernel<TA, TA, 256>, at, (int)kCombineSmemMax))) return e;
+  if ((e = cudaFuncSetAttribute(combine_kernel<TA, TA, 512>, at, (int)kCombineSmemMax))) return e;
+  if ((e = cudaFuncSetAttribute(combine_kernel<float, float, 256>, at, (int)kCombineSmemMax))) return e;
+  if ((e = cudaFuncSetAttribute(combine_kernel<float, float, 512>, at, (int)kCombineSmemMax))) return e;
+  if ((e = cudaFuncSetAttribute(dft_cols_fwd_kernel, at, (int)kColsSmemMax))) return e;
+  if ((e = cudaFuncSetAttribute(spec_mix_kernel, at, (int)mix))) return e;
+  return cudaFuncSetAttribute(spec_mix_bwd_kernel, at, (int)mix);
 }
 
-template <class TX, class TY, class TA>
-void linear(sp_fno* f, int B, const TX* X, int ci, const bf16* W, int ldw, int trans,
-            const bf16* bias, int co, int gelu, TY* pre, TY* Y, const TA* aux) {
+// a tiled pointwise layer (ci <= 32); ~8 CTAs per SM, each keeping its weights over its tiles
+template <class TX, class TY>
+void linear(sp_fno* f, int B, const TX* X, int ci, const bf16* W, const bf16* bias, int co, int gelu,
+            TY* pre, TY* Y) {
   const int co8 = (co + 7) & ~7;
   const size_t smem = (size_t)(ci * co8 + co8 + ci * kTP) * sizeof(float);
-  dim3 grid((unsigned)((f->P + kTP - 1) / kTP), (unsigned)B);
-  chan_linear_kernel<TX, TY, TA><<<grid, kTP, smem, f->st>>>(X, ci, W, ldw, trans, bias, co, f->P,
-                                                             gelu, pre, Y, aux);
+  const long tiles = (f->P + kTP - 1) / kTP;
+  dim3 grid((unsigned)std::min<long>(tiles, std::max<long>(1, 1216 / B)), (unsigned)B);
+  chan_linear_kernel<TX, TY><<<grid, kTP, smem, f->st>>>(X, ci, W, ci, bias, co, f->P, gelu, pre, Y,
+                                                         ((size_t)X & 15) == 0 ? 1 : 0);
 }
 
 // gradient of a pointwise layer's weight [co][ci] and bias [co] (adjacent in the
 // parameter vector at off)
-template <class TX, class TE = float>
-void wgrad(sp_fno* f, int B, const float* dY, int co, const TX* X, int ci, long long off,
-           const TE* E = nullptr, const bf16* Q2 = nullptr, int c2 = 0) {
+template <class TX>
+void wgrad(sp_fno* f, int B, const float* dY, int co, const TX* X, int ci, long long off) {
   const int nchunk = (int)((f->P + kWgChunk - 1) / kWgChunk);
   const int co4 = (co + 3) & ~3, ci4 = (ci + 3) & ~3;
-  const size_t smem = ((size_t)kWgSub * (co4 + 4 + ci4 + 4) + (size_t)c2 * co) * sizeof(float);
-  chan_wgrad_kernel<TX, TE><<<dim3((unsigned)nchunk, (unsigned)B), 256, smem, f->st>>>(
-      dY, co, X, ci, f->P, f->part, E, Q2, c2);
+  const int own = ((co4 / 4) * (ci4 / 4) + 31) & ~31;
+  const size_t smem = kWgStages * ((size_t)co4 * (kWgSub + 4) * sizeof(float) +
+                                   (size_t)ci4 * (kWgSub * sizeof(TX) + 16));
+  chan_wgrad_kernel<TX><<<dim3((unsigned)nchunk, (unsigned)B), own + 32, smem, f->st>>>(
+      dY, co, X, ci, f->P, f->part, own, ((size_t)X & 15) == 0 ? 1 : 0);
   const int len = co * ci + co;
   sum_parts_kernel<<<(len + 255) / 256, 256, 0, f->st>>>(f->part, B * nchunk, len, f->g + off);
 }
@@ -862,17 +1129,35 @@ template <class TX>
 void dft_forward(sp_fno* f, int B, const TX* X, float s0, float s1, float2* V) {
   const int n = f->D.n, M = f->D.modes, C = f->D.width;
   const long rows = (long)B * C * n;
-  const size_t rs = (size_t)n * kRowPitch * sizeof(float) + (size_t)n * 16 * sizeof(float2);
-  dft_rows_fwd_kernel<TX><<<(unsigned)((rows + kRowsCta - 1) / kRowsCta), 256, rs, f->st>>>(
+  dft_rows_fwd_kernel<TX><<<(unsigned)((rows + kRowsCta - 1) / kRowsCta), 128, 0, f->st>>>(
       X, rows, n, M, f->twr, f->A);
   const size_t cs = (size_t)(n * M + n) * sizeof(float2);
   dft_cols_fwd_kernel<<<(unsigned)(B * C), 256, cs, f->st>>>(f->A, n, M, f->twb, s0, s1, V);
 }
 
 void dft_cols_inverse(sp_fno* f, int B, const float2* Y) {
-  const int n = f->D.n, M = f->D.modes, C = f->D.width;
-  const size_t cs = (size_t)(2 * M * M + n) * sizeof(float2);
-  dft_cols_inv_kernel<<<(unsigned)(B * C), 256, cs, f->st>>>(Y, n, M, f->twb, f->Bc);
+  const int n = f->D.n, M = f->D.modes, C = f->D.width, R = n / 16;
+  const int nbc = B * C;
+  if (nbc >= 256) {  // enough channels to fill the GPU: pairs share the twiddle loads
+    const size_t cs = (size_t)(2 * 2 * M * M + n) * sizeof(float2);
+    dft_cols_inv_kernel<2, 16><<<dim3((unsigned)((nbc + 1) / 2), (unsigned)((R + 15) / 16)), 256, cs,
+                                 f->st>>>(Y, n, M, nbc, f->twb, f->Bc);
+  } else {
+    const size_t cs = (size_t)(2 * M * M + n) * sizeof(float2);
+    dft_cols_inv_kernel<1, 4><<<dim3((unsigned)nbc, (unsigned)((R + 3) / 4)), 256, cs, f->st>>>(
+        Y, n, M, nbc, f->twb, f->Bc);
+  }
+}
+
+// the layer output kernel: n threads, ~6 CTAs per SM walking the grid rows of a sample
+template <class TX, class TY>
+void combine(sp_fno* f, int B, const TX* X, const bf16* W, int trans, const bf16* bias, float w0,
+             float w1, int gelu, TY* pre, TY* out) {
+  const int n = f->D.n;
+  const int rows = std::max(1, (int)((long)B * n / 912));
+  auto kern = n <= 256 ? combine_kernel<TX, TY, 256> : combine_kernel<TX, TY, 512>;
+  kern<<<dim3((unsigned)((n + rows - 1) / rows), (unsigned)B), n, (size_t)64 * n * sizeof(float), f->st>>>(
+      X, f->D.width, W, trans, bias, f->Bc, n, f->D.modes, f->twr, w0, w1, gelu, pre, out, rows);
 }
 
 template <class TA>
@@ -880,8 +1165,8 @@ cudaError_t forward_t(sp_fno* f, int B, const float* x) {
   const sp_fno_dims& D = f->D;
   const int W = D.width, L = D.layers, n = D.n;
   const bf16* wb = f->wb;
-  linear<float, TA, TA>(f, B, x, D.c_in, wb + f->offP, D.c_in, 0, wb + f->offP + (long long)W * D.c_in,
-                        W, 0, nullptr, (TA*)f->vv[0], (const TA*)nullptr);
+  linear<float, TA>(f, B, x, D.c_in, wb + f->offP, wb + f->offP + (long long)W * D.c_in, W, 0, nullptr,
+                    (TA*)f->vv[0]);
   const float inv2 = 1.f / ((float)n * (float)n);
   for (int l = 0; l < L; ++l) {
     dft_forward<TA>(f, B, (const TA*)f->vv[l], 1.f, 1.f, f->Vh[l]);
@@ -890,16 +1175,18 @@ cudaError_t forward_t(sp_fno* f, int B, const float* x) {
     dft_cols_inverse(f, B, f->Yh);
     const bool act = l < L - 1;
     const bf16* Wl = wb + f->offW[l];
-    combine_kernel<TA, TA><<<dim3((unsigned)n, (unsigned)B), 256, 0, f->st>>>(
-        (const TA*)f->vv[l], W, Wl, 0, Wl + W * W, f->Bc, n, D.modes, f->twr, inv2, 2.f * inv2,
-        act ? 1 : 0, act ? (TA*)f->hh[l] : (TA*)nullptr, (TA*)f->vv[l + 1]);
+    combine<TA, TA>(f, B, (const TA*)f->vv[l], Wl, 0, Wl + W * W, inv2, 2.f * inv2, act ? 1 : 0,
+                    act ? (TA*)f->hh[l] : (TA*)nullptr, (TA*)f->vv[l + 1]);
   }
   const int H = D.hidden;
-  linear<TA, TA, TA>(f, B, (const TA*)f->vv[L], W, wb + f->offQ1, W, 0, wb + f->offQ1 + (long long)H * W,
-                     H, 1, (TA*)f->e, (TA*)f->ge, (const TA*)nullptr);
-  linear<TA, float, TA>(f, B, (const TA*)f->ge, H, wb + f->offQ2, H, 0,
-                        wb + f->offQ2 + (long long)D.c_out * H, D.c_out, 0, (float*)nullptr, f->y,
-                        (const TA*)nullptr);
+  linear<TA, TA>(f, B, (const TA*)f->vv[L], W, wb + f->offQ1, wb + f->offQ1 + (long long)H * W, H, 1,
+                 (TA*)f->e, (TA*)f->ge);
+  const bf16 *q2 = wb + f->offQ2, *c2 = q2 + (long long)D.c_out * H;
+  const dim3 gn((unsigned)((f->P / 4 + 127) / 128), (unsigned)B);
+  if (D.c_out <= 2)
+    chan_narrow_kernel<TA, 2><<<gn, 128, 0, f->st>>>((const TA*)f->ge, H, q2, H, c2, D.c_out, f->P, f->y);
+  else
+    chan_narrow_kernel<TA, 8><<<gn, 128, 0, f->st>>>((const TA*)f->ge, H, q2, H, c2, D.c_out, f->P, f->y);
   return cudaGetLastError();
 }
 
@@ -910,15 +1197,18 @@ cudaError_t backward_t(sp_fno* f, int B, const float* x, const float* t) {
   const bf16* wb = f->wb;
   const long len = (long)co * f->P;
   loss_partial_kernel<<<dim3(kLossChunks, (unsigned)B), 256, 0, f->st>>>(f->y, t, len, f->lpart);
-  loss_finish_kernel<<<1, 32, 0, f->st>>>(f->lpart, B, kLossChunks, f->dloss, f->lscale);
+  loss_finish_kernel<<<1, 256, 0, f->st>>>(f->lpart, B, kLossChunks, f->dloss, f->lscale);
   loss_grad_kernel<<<grid_for(len * B, 256), 256, 0, f->st>>>(f->y, t, len, B, f->lscale, f->dy);
-  // projection: dQ2 from (dy, gelu(e)); dQ1 and dv from de = (Q2^T dy) gelu'(e), formed
-  // on the fly in both kernels
+  // projection: dQ2 from (dy, gelu(e)); dQ1 and dv from de = (Q2^T dy) gelu'(e) in one kernel
   wgrad<TA>(f, B, f->dy, co, (const TA*)f->ge, H, f->offQ2);
-  wgrad<TA, TA>(f, B, f->dy, H, (const TA*)f->vv[L], W, f->offQ1, (const TA*)f->e, wb + f->offQ2, co);
   int cur = 0;
-  proj_bwd_kernel<TA><<<dim3((unsigned)((f->P + kTP - 1) / kTP), (unsigned)B), kTP, 0, f->st>>>(
-      f->dy, co, (const TA*)f->e, H, wb + f->offQ2, wb + f->offQ1, W, f->P, f->dv[cur]);
+  {
+    const int nchunk = (int)((f->P + kWgChunk - 1) / kWgChunk), len = H * W + H;
+    proj_bwd_kernel<TA><<<dim3((unsigned)nchunk, (unsigned)B), 256, kProjSmem, f->st>>>(
+        f->dy, co, (const TA*)f->e, H, wb + f->offQ2, wb + f->offQ1, (const TA*)f->vv[L], W, f->P,
+        f->dv[cur], f->part);
+    sum_parts_kernel<<<(len + 255) / 256, 256, 0, f->st>>>(f->part, B * nchunk, len, f->g + f->offQ1);
+  }
   const float inv2 = 1.f / ((float)n * (float)n);
   const long act_len = (long)B * W * f->P;
   for (int l = L - 1; l >= 0; --l) {
@@ -936,9 +1226,7 @@ cudaError_t backward_t(sp_fno* f, int B, const float* x, const float* t) {
                                                   f->g + f->offR[l]);
     dft_cols_inverse(f, B, f->dVh);
     const int nxt = cur ^ 1;
-    combine_kernel<float, float><<<dim3((unsigned)n, (unsigned)B), 256, 0, f->st>>>(
-        dhp, W, wb + f->offW[l], 1, nullptr, f->Bc, n, D.modes, f->twr, 1.f, 1.f, 0, (float*)nullptr,
-        f->dv[nxt]);
+    combine<float, float>(f, B, dhp, wb + f->offW[l], 1, nullptr, 1.f, 1.f, 0, (float*)nullptr, f->dv[nxt]);
     cur = nxt;
   }
   wgrad<float>(f, B, f->dv[cur], W, x, D.c_in, f->offP);  // lift
@@ -1150,7 +1438,7 @@ sp_status sp_fno_features(sp_fno* f, const double* q_dev, double q_scale, const 
   if (!f || !q_dev || !g_dev || !x_dev || !scale_dev || f->D.c_in != 3) return SP_ERR_ARG;
   const long N = f->P;
   norm_partial_kernel<<<kNormBlocks, 256, 0, f->st>>>((const double2*)g_dev, N, f->npart);
-  scale_kernel<<<1, 32, 0, f->st>>>(f->npart, kNormBlocks, N, (double2*)scale_dev);
+  scale_kernel<<<1, 256, 0, f->st>>>(f->npart, kNormBlocks, N, (double2*)scale_dev);
   features_kernel<<<grid_for(N, 256), 256, 0, f->st>>>(q_dev, q_scale, (const double2*)g_dev,
                                                        (const double2*)scale_dev, N, x_dev);
   return cuda_st(cudaGetLastError());
@@ -1161,7 +1449,7 @@ sp_status sp_fno_features_prior(sp_fno* f, const double* q_dev, double q_scale, 
   if (!f || !q_dev || !g_dev || !z_dev || !x_dev || !scale_dev || f->D.c_in != 5) return SP_ERR_ARG;
   const long N = f->P;
   norm_partial_kernel<<<kNormBlocks, 256, 0, f->st>>>((const double2*)g_dev, N, f->npart);
-  scale_kernel<<<1, 32, 0, f->st>>>(f->npart, kNormBlocks, N, (double2*)scale_dev);
+  scale_kernel<<<1, 256, 0, f->st>>>(f->npart, kNormBlocks, N, (double2*)scale_dev);
   features_kernel<<<grid_for(N, 256), 256, 0, f->st>>>(q_dev, q_scale, (const double2*)g_dev,
                                                        (const double2*)scale_dev, N, x_dev);
   features_prior_kernel<<<grid_for(N, 256), 256, 0, f->st>>>((const double2*)z_dev,
