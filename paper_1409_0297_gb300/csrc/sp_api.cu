@@ -977,7 +977,7 @@ static sp_status setup_impl(int d, int n, int b, int P, const double* shifts, sp
   SP_CK(dalloc(c.get(), &c->t, sizeof(double2) * N * IM));
   SP_CK(dalloc(c.get(), &c->fbuf, sizeof(double2) * NP));
   SP_CK(dalloc(c.get(), &c->ubuf, sizeof(double2) * N * IM));
-  c->K.nblk = (int)std::min<long>(304, std::max<long>(1, (N + 1023) / 1024));
+  c->K.nblk = (int)std::min<long>(304, (N + 255) / 256);
   SP_CK(dalloc(c.get(), &c->K.partial, sizeof(double2) * (size_t)c->K.nblk * 1024 * IM));
   SP_CK(dalloc(c.get(), &c->K.h, sizeof(double2) * 1024));
   SP_CK(cudaMallocHost(&c->host_sc, 8 * sizeof(double) * IM));

@@ -4,33 +4,30 @@
 //   G x = F^{-1} diag(1/(4 pi^2 |k|^2 - s)) F x       (Eq. G)
 //   A x = x + G (q x)                                   (Section 2.2)
 //
-// The n^d transform is done axis by axis.  Each CTA owns W complete 1D lines of
-// length n of one axis, stages them in shared memory (coalesced: along axis 0 the
-// lines are contiguous, along the other axes W neighbouring lines give W
-// consecutive elements per row), runs radix-2 butterflies in shared memory and
-// writes the lines back.  Fused pointwise work:
+// The n^d transform is done axis by axis; a CTA owns W neighbouring lines of one axis.  A
+// line is transformed by self-sorting (Stockham) steps: with l the product of the radices
+// before a step of radix r, butterfly b takes x[b + k n / r] (k < r), multiplies by
+// w_{l r}^{(b mod l) k}, transforms and writes y[(b - b mod l) r + b mod l + k l].  A thread
+// keeps its butterflies in registers; the first step reads device memory, the last writes
+// it, and between steps the line passes through shared memory once, so a line of 64 points
+// (three steps of radix 4) costs two exchanges and no bit reversal, and its first step no
+// twiddles.  Fused pointwise work:
 //   first pass   x -> q x              (PRE_Q)
-//   last axis    forward, * D/N, inverse in one pass (MID), so the spectrum never
-//                leaves shared memory between the forward and inverse transform
+//   last axis    forward, * D/N, inverse in one pass (MID): the inverse takes the radices in
+//                reverse, so its first step wants exactly the elements that the last forward
+//                step left in the thread's registers
 //   final pass   out = x + result      (POST_ADD)
-// Forward transforms are decimation-in-time (bit-reversed load), inverse ones
-// decimation-in-frequency (bit-reversed store), so no extra permutation pass is
-// needed.  n = R M with M a power of two and R = 1 or 3: for R = 3 the line is
-// split by j mod 3 into three M-point lines (element j = 3 j' + r goes to
-// sub-line r at the bit-reversed position of j'), the three M-point transforms
-// run side by side, and one radix-3 step combines them in place,
-//   X[k1 + M k2] = sum_r w_n^(r k1) w_3^(r k2) Y_r[k1],
-// which leaves the spectrum in natural order (sub-line k2 holds X[k1 + M k2]);
-// the inverse runs the conjugate steps in the opposite order.
-#include <cstdio>
+// n = 2^p or 3 2^p; the radix 3 is the last forward step.
+// What bounds it: the FP64 pipe (28 instructions per radix-4 butterfly, two lanes per SM
+// cycle) on large grids, the chain of three launches on small ones.
+#include <algorithm>
+#include <type_traits>
 
 #include "sp_internal.h"
 
 namespace sp {
 
 namespace {
-
-constexpr int kThreads = 256;
 
 template <class VT> struct Real;
 template <> struct Real<double2> { using T = double; };
@@ -47,6 +44,8 @@ __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_doub
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 
+constexpr int kMaxSteps = 16;
+
 template <class VT>
 struct PassArgs {
   using T = typename Real<VT>::T;
@@ -59,102 +58,18 @@ struct PassArgs {
   long S;               // stride between consecutive elements of a line
   long nlines;          // number of lines of this axis, all vectors
   long vlines, vstride; // lines per vector, entries per vector (vectors stacked)
-  int n, W, pad;
-  int R, M, logM;       // n = R M, R in {1, 3}, M = 2^logM
+  int n, W, U;          // U threads per line
+  int ld;               // entries between two lines in shared memory
+  int steps;
+  int rad[kMaxSteps];   // radices of the forward transform; the inverse runs them in reverse
   int mode;             // 0 forward, 1 inverse, 2 middle (forward, scale, inverse)
   int qper;             // q and Dn per vector: vector v reads those of v % qper (vstride apart)
 };
 
-// position in the staged row of element i of a line in permuted (DIT input /
-// DIF output) order
-template <int R, class VT>
-__device__ __forceinline__ int perm_pos(const PassArgs<VT>& a, int i) {
-  const int r = i % R, j = i / R;
-  return r * a.M + (a.logM ? (int)(__brev((unsigned)j) >> (32 - a.logM)) : 0);
-}
-// w_n^t for 0 <= t < n (w_n^(t + n/2) = -w_n^t)
-template <class VT>
-__device__ __forceinline__ VT tw_at(const PassArgs<VT>& a, int t) {
-  const int h = a.n >> 1;
-  if (t < h) return a.tw[t];
-  VT v = a.tw[t - h];
-  v.x = -v.x;
-  v.y = -v.y;
-  return v;
-}
+// shared-memory position of element i of a line: one entry of padding per eight keeps the
+// strided writes of a step (stride r) off each other's banks
+__device__ __forceinline__ int spos(int i) { return i + (i >> 3); }
 
-// address of element i of line t within its vector (q and the symbol are shared
-// by every vector), and the offset of that vector
-template <class VT>
-__device__ __forceinline__ long line_addr(const PassArgs<VT>& a, long t, int i) {
-  const long tl = t % a.vlines;
-  long lo = tl % a.S, hi = tl / a.S;
-  return lo + hi * a.S * a.n + (long)i * a.S;
-}
-template <class VT>
-__device__ __forceinline__ long vec_off(const PassArgs<VT>& a, long t) {
-  return (t / a.vlines) * a.vstride;
-}
-
-// radix-2 stages of the W R sub-lines of length M (sub-line r of row w at
-// offset r M); the M-point twiddle w_M^t is w_n^(R t)
-template <int R, class VT>
-__device__ __forceinline__ void dit_stages(VT* sm, const PassArgs<VT>& a, bool conj_tw) {
-  const int M = a.M, half_m = M >> 1, ld = a.n + a.pad;
-  const int work = a.W * R * half_m;
-  for (int s = 1; s <= a.logM; ++s) {
-    const int half = 1 << (s - 1);
-    for (int it = threadIdx.x; it < work; it += blockDim.x) {
-      int u = it / half_m, p = it - u * half_m;
-      int w = u / R, r = u - w * R;
-      int jj = p & (half - 1);
-      int i0 = ((p >> (s - 1)) << s) + jj;
-      int i1 = i0 + half;
-      VT t = a.tw[(jj << (a.logM - s)) * R];
-      if (conj_tw) t.y = -t.y;
-      VT* row = sm + w * ld + r * M;
-      VT x0 = row[i0], v = cmul(row[i1], t);
-      row[i0] = cadd(x0, v);
-      row[i1] = csub(x0, v);
-    }
-    __syncthreads();
-  }
-}
-
-template <int R, class VT>
-__device__ __forceinline__ void dif_stages(VT* sm, const PassArgs<VT>& a, bool conj_tw) {
-  const int M = a.M, half_m = M >> 1, ld = a.n + a.pad;
-  const int work = a.W * R * half_m;
-  for (int s = a.logM; s >= 1; --s) {
-    const int half = 1 << (s - 1);
-    for (int it = threadIdx.x; it < work; it += blockDim.x) {
-      int u = it / half_m, p = it - u * half_m;
-      int w = u / R, r = u - w * R;
-      int jj = p & (half - 1);
-      int i0 = ((p >> (s - 1)) << s) + jj;
-      int i1 = i0 + half;
-      VT t = a.tw[(jj << (a.logM - s)) * R];
-      if (conj_tw) t.y = -t.y;
-      VT* row = sm + w * ld + r * M;
-      VT x0 = row[i0], v = row[i1];
-      row[i0] = cadd(x0, v);
-      row[i1] = cmul(csub(x0, v), t);
-    }
-    __syncthreads();
-  }
-}
-
-// The same transforms with the radix-2 stages taken two at a time (radix 4): three
-// twiddle products and one barrier per pair of stages instead of four and two.
-//   DIT stages s, s+1 (h = 2^(s-1)): with t1 = w_{2h}^j, t2 = w_{4h}^j,
-//     u0 = x0, u1 = t1 x1, u2 = t2 x2, u3 = t1 t2 x3 (x_q at base + j + q h),
-//     y0 = (u0 + u1) + (u2 + u3), y2 = (u0 + u1) - (u2 + u3),
-//     y1 = (u0 - u1) - i (u2 - u3), y3 = (u0 - u1) + i (u2 - u3);
-//   DIF stages s, s-1 (q = 2^(s-2)) of the conjugate (inverse) transform: with
-//     t1 = conj w_{4q}^j, t2 = conj w_{2q}^j, s0 = x0 + x2, s1 = x0 - x2, s2 = x1 + x3,
-//     s3 = x1 - x3 (x_r at base + j + r q): y0 = s0 + s2, y1 = (s0 - s2) t2,
-//     y2 = (s1 + i s3) t1, y3 = (s1 - i s3) t1 t2.
-// An odd stage count leaves one radix-2 stage (first for DIT, last for DIF).
 template <class VT>
 __device__ __forceinline__ VT mul_i(VT v) {  // i v
   VT r;
@@ -162,225 +77,193 @@ __device__ __forceinline__ VT mul_i(VT v) {  // i v
   r.y = v.x;
   return r;
 }
-template <int R, class VT>
-__device__ __forceinline__ void dit_stages4(VT* sm, const PassArgs<VT>& a) {
-  const int M = a.M, ld = a.n + a.pad;
-  int s = 1;
-  if (a.logM & 1) {  // one radix-2 stage first (twiddle 1)
-    const int work = a.W * R * (M >> 1);
-    for (int it = threadIdx.x; it < work; it += blockDim.x) {
-      const int u = it / (M >> 1), p = it - u * (M >> 1);
-      const int w = u / R, r = u - w * R;
-      VT* row = sm + w * ld + r * M;
-      const int i0 = 2 * p;
-      const VT x0 = row[i0], x1 = row[i0 + 1];
-      row[i0] = cadd(x0, x1);
-      row[i0 + 1] = csub(x0, x1);
-    }
-    __syncthreads();
-    s = 2;
-  }
-  const int quarter = M >> 2;
-  const int work = a.W * R * quarter;
-  for (; s + 1 <= a.logM; s += 2) {
-    const int h = 1 << (s - 1);
-    for (int it = threadIdx.x; it < work; it += blockDim.x) {
-      const int u = it / quarter, p = it - u * quarter;
-      const int w = u / R, r = u - w * R;
-      const int j = p & (h - 1);
-      const int base = ((p >> (s - 1)) << (s + 1)) + j;
-      VT* row = sm + w * ld + r * M;
-      const VT t1 = a.tw[(j << (a.logM - s)) * R];
-      const VT t2 = a.tw[(j << (a.logM - s - 1)) * R];
-      const VT t3 = tw_at(a, (3 * j << (a.logM - s - 1)) * R);
-      const VT u0 = row[base], u1 = cmul(row[base + h], t1);
-      const VT u2 = cmul(row[base + 2 * h], t2), u3 = cmul(row[base + 3 * h], t3);
-      const VT s0 = cadd(u0, u1), s1 = csub(u0, u1), s2 = cadd(u2, u3), s3 = mul_i(csub(u2, u3));
-      row[base] = cadd(s0, s2);
-      row[base + 2 * h] = csub(s0, s2);
-      row[base + h] = csub(s1, s3);
-      row[base + 3 * h] = cadd(s1, s3);
-    }
-    __syncthreads();
-  }
-}
-template <int R, class VT>
-__device__ __forceinline__ void dif_stages4_conj(VT* sm, const PassArgs<VT>& a) {
-  const int M = a.M, ld = a.n + a.pad;
-  const int quarter = M >> 2;
-  const int work4 = a.W * R * quarter;
-  int s = a.logM;
-  for (; s >= 2; s -= 2) {
-    const int q = 1 << (s - 2);
-    for (int it = threadIdx.x; it < work4; it += blockDim.x) {
-      const int u = it / quarter, p = it - u * quarter;
-      const int w = u / R, r = u - w * R;
-      const int j = p & (q - 1);
-      const int base = ((p >> (s - 2)) << s) + j;
-      VT* row = sm + w * ld + r * M;
-      VT t1 = a.tw[(j << (a.logM - s)) * R];
-      VT t2 = a.tw[(j << (a.logM - s + 1)) * R];
-      VT t3 = tw_at(a, (3 * j << (a.logM - s)) * R);
-      t1.y = -t1.y;
-      t2.y = -t2.y;
-      t3.y = -t3.y;
-      const VT x0 = row[base], x1 = row[base + q], x2 = row[base + 2 * q], x3 = row[base + 3 * q];
-      const VT s0 = cadd(x0, x2), s1 = csub(x0, x2), s2 = cadd(x1, x3), s3 = mul_i(csub(x1, x3));
-      row[base] = cadd(s0, s2);
-      row[base + q] = cmul(csub(s0, s2), t2);
-      row[base + 2 * q] = cmul(cadd(s1, s3), t1);
-      row[base + 3 * q] = cmul(csub(s1, s3), t3);
-    }
-    __syncthreads();
-  }
-  if (s == 1) {  // one radix-2 stage last (twiddle 1)
-    const int work = a.W * R * (M >> 1);
-    for (int it = threadIdx.x; it < work; it += blockDim.x) {
-      const int u = it / (M >> 1), p = it - u * (M >> 1);
-      const int w = u / R, r = u - w * R;
-      VT* row = sm + w * ld + r * M;
-      const int i0 = 2 * p;
-      const VT x0 = row[i0], x1 = row[i0 + 1];
-      row[i0] = cadd(x0, x1);
-      row[i0 + 1] = csub(x0, x1);
-    }
-    __syncthreads();
-  }
-}
-
-// radix-3 step over the three sub-lines of every row (R = 3 only).  Forward:
-// X[k1 + M k2] = sum_r w_3^(r k2) (w_n^(r k1) Y_r[k1]); inverse (conjugate):
-// Z_r[k1] = w_n^(-r k1) sum_k2 w_3^(-r k2) X[k1 + M k2].
 template <class VT>
-__device__ __forceinline__ void radix3_step(VT* sm, const PassArgs<VT>& a, bool inverse) {
-  using T = typename Real<VT>::T;
-  const int M = a.M, ld = a.n + a.pad;
-  const T h3 = (T)0.86602540378443864676372317075294;  // sin(2 pi / 3)
-  for (int it = threadIdx.x; it < a.W * M; it += blockDim.x) {
-    const int w = it / M, k1 = it - w * M;
-    VT* row = sm + w * ld;
-    VT w1 = tw_at(a, k1), w2 = tw_at(a, 2 * k1);
-    if (!inverse) {
-      const VT a0 = row[k1], b1 = cmul(row[M + k1], w1), b2 = cmul(row[2 * M + k1], w2);
-      const VT t1 = cadd(b1, b2), t2 = csub(b1, b2);
-      VT mm = a0;
-      mm.x -= (T)0.5 * t1.x;
-      mm.y -= (T)0.5 * t1.y;
-      VT rot;  // -i sin(2 pi / 3) t2
-      rot.x = h3 * t2.y;
-      rot.y = -h3 * t2.x;
-      row[k1] = cadd(a0, t1);
-      row[M + k1] = cadd(mm, rot);
-      row[2 * M + k1] = csub(mm, rot);
-    } else {
-      const VT x0 = row[k1], x1 = row[M + k1], x2 = row[2 * M + k1];
-      const VT u1 = cadd(x1, x2), u2 = csub(x1, x2);
-      VT mm = x0;
-      mm.x -= (T)0.5 * u1.x;
-      mm.y -= (T)0.5 * u1.y;
-      VT rot;  // +i sin(2 pi / 3) u2
-      rot.x = -h3 * u2.y;
-      rot.y = h3 * u2.x;
-      w1.y = -w1.y;
-      w2.y = -w2.y;
-      row[k1] = cadd(x0, u1);
-      row[M + k1] = cmul(cadd(mm, rot), w1);
-      row[2 * M + k1] = cmul(csub(mm, rot), w2);
-    }
-  }
-  __syncthreads();
+__device__ __forceinline__ VT mul_mi(VT v) {  // -i v
+  VT r;
+  r.x = v.y;
+  r.y = -v.x;
+  return r;
 }
 
-template <class VT, int R>
-__global__ void __launch_bounds__(kThreads) fft_pass_kernel(PassArgs<VT> a) {
+// in-register transform of r values, sign -1 (forward) or +1 (INV) in the exponent
+template <int r, bool INV, class VT>
+__device__ __forceinline__ void dft_reg(VT* v) {
   using T = typename Real<VT>::T;
-  extern __shared__ unsigned char smraw[];
-  VT* sm = reinterpret_cast<VT*>(smraw);
-  const int n = a.n, ld = n + a.pad, W = a.W;
-  const long t0 = (long)blockIdx.x * W;
-  const int total = W * n;
-  const bool axis0 = (a.S == 1);
-  const bool bitrev_load = (a.mode != 1);  // forward transforms are DIT
-  // ---- load (coalesced), optional q multiply, bit-reversed placement for DIT
-  for (int e = threadIdx.x; e < total; e += blockDim.x) {
-    int w, i;
-    if (axis0) {
-      w = e / n;
-      i = e - w * n;
-    } else {
-      i = e / W;
-      w = e - i * W;
-    }
-    long t = t0 + w;
-    if (t >= a.nlines) continue;
-    long g = line_addr(a, t, i);
-    VT v = a.in[vec_off(a, t) + g];
-    if (a.q) {
-      T qq = a.q[(a.qper > 1 ? (t / a.vlines) % a.qper * a.vstride : 0) + g];
-      v.x *= qq;
-      v.y *= qq;
-    }
-    int pos = bitrev_load ? perm_pos<R>(a, i) : i;
-    sm[w * ld + pos] = v;
-  }
-  __syncthreads();
-  if (a.mode == 0) {
-    dit_stages4<R>(sm, a);
-    if (R == 3) radix3_step(sm, a, false);
-  } else if (a.mode == 1) {
-    if (R == 3) radix3_step(sm, a, true);
-    dif_stages4_conj<R>(sm, a);
+  if constexpr (r == 2) {
+    const VT t = v[0];
+    v[0] = cadd(t, v[1]);
+    v[1] = csub(t, v[1]);
+  } else if constexpr (r == 3) {
+    const T h3 = (T)0.86602540378443864676372317075294;  // sin(2 pi / 3)
+    const VT t1 = cadd(v[1], v[2]), t2 = csub(v[1], v[2]);
+    VT m = v[0];
+    m.x -= (T)0.5 * t1.x;
+    m.y -= (T)0.5 * t1.y;
+    VT rot = INV ? mul_i(t2) : mul_mi(t2);
+    rot.x *= h3;
+    rot.y *= h3;
+    v[0] = cadd(v[0], t1);
+    v[1] = cadd(m, rot);
+    v[2] = csub(m, rot);
   } else {
-    dit_stages4<R>(sm, a);
-    if (R == 3) radix3_step(sm, a, false);
-    for (int e = threadIdx.x; e < total; e += blockDim.x) {
-      int w, i;
-      if (axis0) {
-        w = e / n;
-        i = e - w * n;
-      } else {
-        i = e / W;
-        w = e - i * W;
-      }
-      long t = t0 + w;
-      if (t >= a.nlines) continue;
-      T dn = a.Dn[(a.qper > 1 ? (t / a.vlines) % a.qper * a.vstride : 0) + line_addr(a, t, i)];
-      VT* p = &sm[w * ld + i];
-      p->x *= dn;
-      p->y *= dn;
-    }
-    __syncthreads();
-    if (R == 3) radix3_step(sm, a, true);
-    dif_stages4_conj<R>(sm, a);
-  }
-  const bool bitrev_store = (a.mode != 0);  // inverse transforms are DIF
-  for (int e = threadIdx.x; e < total; e += blockDim.x) {
-    int w, i;
-    if (axis0) {
-      w = e / n;
-      i = e - w * n;
-    } else {
-      i = e / W;
-      w = e - i * W;
-    }
-    long t = t0 + w;
-    if (t >= a.nlines) continue;
-    long g = vec_off(a, t) + line_addr(a, t, i);
-    int pos = bitrev_store ? perm_pos<R>(a, i) : i;
-    VT v = sm[w * ld + pos];
-    if (a.addx) v = cadd(v, a.addx[g]);
-    a.out[g] = v;
+    const VT s0 = cadd(v[0], v[2]), s1 = csub(v[0], v[2]), s2 = cadd(v[1], v[3]);
+    const VT d = csub(v[1], v[3]);
+    const VT s3 = INV ? mul_i(d) : mul_mi(d);
+    v[0] = cadd(s0, s2);
+    v[1] = cadd(s1, s3);
+    v[2] = csub(s0, s2);
+    v[3] = csub(s1, s3);
   }
 }
 
-int lines_per_cta(int n, long nlines, int esize) {
-  // enough lines for >= 256 butterflies per stage, at most 64 KB of lines, and
-  // at least ~2 CTAs per SM on 152 SMs when the grid allows it
-  int W = 1;
-  while (W * n < 2 * kThreads && W < 64) W <<= 1;
-  while (W > 1 && (long)W * n * esize > 64 * 1024) W >>= 1;
-  while (W > 1 && nlines / W < 304) W >>= 1;
-  return W;
+// w_n^t (INV: its conjugate) for 0 <= t < n (w_n^(t + n/2) = -w_n^t)
+template <bool INV, class VT>
+__device__ __forceinline__ VT tw_at(const PassArgs<VT>& a, int t) {
+  const int h = a.n >> 1;
+  const bool up = t >= h;
+  VT v = a.tw[up ? t - h : t];
+  if (up) {
+    v.x = -v.x;
+    v.y = -v.y;
+  }
+  if (INV) v.y = -v.y;
+  return v;
+}
+
+// values a thread holds: one butterfly of radix 4, two of radix 2, two of radix 3
+constexpr int kVal = 6;
+template <int r>
+constexpr int kPer = r == 4 ? 1 : 2;
+
+// One step of radix r at l for the butterflies b = bb + j U of a line: from the values in v
+// (loaded: already there) or from the line in shared memory, to registers.
+template <int r, bool INV, class VT>
+__device__ __forceinline__ void step_reg(const PassArgs<VT>& a, const VT* line, int bb, bool loaded,
+                                         int l, VT* v) {
+  const int nb = a.n / r;
+#pragma unroll
+  for (int j = 0; j < kPer<r>; ++j) {
+    const int b = bb + j * a.U;
+    if (b >= nb) continue;
+    VT* x = v + j * r;
+    if (!loaded) {
+#pragma unroll
+      for (int k = 0; k < r; ++k) x[k] = line[spos(b + k * nb)];
+    }
+    if (l > 1) {
+      const int t = (b % l) * (nb / l);  // w_{l r}^1 = w_n^(n / (l r))
+#pragma unroll
+      for (int k = 1; k < r; ++k) x[k] = cmul(x[k], tw_at<INV>(a, t * k));
+    }
+    dft_reg<r, INV>(x);
+  }
+}
+template <int r, class VT>
+__device__ __forceinline__ void put_line(const PassArgs<VT>& a, VT* line, int bb, int l, const VT* v) {
+  const int nb = a.n / r;
+#pragma unroll
+  for (int j = 0; j < kPer<r>; ++j) {
+    const int b = bb + j * a.U;
+    if (b >= nb) continue;
+    const int m = b % l, o = (b - m) * r + m;
+#pragma unroll
+    for (int k = 0; k < r; ++k) line[spos(o + k * l)] = v[j * r + k];
+  }
+}
+
+// The transform of one line: on entry the first step's inputs are in v, on return the last
+// step's outputs (element b + k n / r of butterfly b), radices rad[0 .. steps) or, INV, in
+// reverse.
+template <bool INV, class VT>
+__device__ __forceinline__ void transform(const PassArgs<VT>& a, VT* line, int bb, bool live, VT* v) {
+  int l = 1;
+  for (int s = 0; s < a.steps; ++s) {
+    const int r = a.rad[INV ? a.steps - 1 - s : s];
+    const bool first = s == 0, last = s == a.steps - 1;
+    if (live) {
+      if (r == 4) step_reg<4, INV>(a, line, bb, first, l, v);
+      else if (r == 2) step_reg<2, INV>(a, line, bb, first, l, v);
+      else step_reg<3, INV>(a, line, bb, first, l, v);
+    }
+    if (!last) {
+      __syncthreads();  // the line has been read
+      if (live) {
+        if (r == 4) put_line<4>(a, line, bb, l, v);
+        else if (r == 2) put_line<2>(a, line, bb, l, v);
+        else put_line<3>(a, line, bb, l, v);
+      }
+      __syncthreads();
+    }
+    l *= r;
+  }
+}
+
+// fn(value, element index) for the values of a step of radix r read or written at
+// b + k n / r
+template <class VT, class Fn>
+__device__ __forceinline__ void each_value(const PassArgs<VT>& a, int r, int bb, VT* v, Fn fn) {
+  const int nb = a.n / r;
+  auto go = [&](auto rr) {
+    constexpr int R = decltype(rr)::value;
+#pragma unroll
+    for (int j = 0; j < kPer<R>; ++j) {
+      const int b = bb + j * a.U;
+      if (b >= nb) continue;
+#pragma unroll
+      for (int k = 0; k < R; ++k) fn(v[j * R + k], b + k * nb);
+    }
+  };
+  if (r == 4) go(std::integral_constant<int, 4>{});
+  else if (r == 2) go(std::integral_constant<int, 2>{});
+  else go(std::integral_constant<int, 3>{});
+}
+
+template <class VT>
+__global__ void __launch_bounds__(1024) fft_pass_kernel(PassArgs<VT> a) {
+  using T = typename Real<VT>::T;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const bool axis0 = a.S == 1;
+  // lines side by side along axis 0, element-interleaved along the others (coalesced)
+  const int tid = threadIdx.x;
+  const int w = axis0 ? tid / a.U : tid % a.W, bb = axis0 ? tid - w * a.U : tid / a.W;
+  const long t = (long)blockIdx.x * a.W + w;
+  const bool live = w < a.W && bb < a.U && t < a.nlines;
+  VT* line = reinterpret_cast<VT*>(smraw) + (long)w * a.ld;
+  const long vec = t / a.vlines, tl = t - vec * a.vlines;
+  const long hi = tl / a.S, base = (tl - hi * a.S) + hi * a.S * a.n;  // within the vector
+  const long voff = vec * a.vstride;
+  const long qoff = (a.qper > 1 ? vec % a.qper * a.vstride : 0) + base;
+  const VT* in = a.in + voff + base;
+  VT v[kVal];
+  const int rf = a.mode == 1 ? a.rad[a.steps - 1] : a.rad[0];                 // radix read first
+  const int rl = a.mode == 0 ? a.rad[a.steps - 1] : a.rad[0];                 // radix written last
+  if (live) {
+    each_value(a, rf, bb, v, [&](VT& x, int i) { x = in[(long)i * a.S]; });
+    if (a.q)
+      each_value(a, rf, bb, v, [&](VT& x, int i) {
+        const T qq = a.q[qoff + (long)i * a.S];
+        x.x *= qq;
+        x.y *= qq;
+      });
+  }
+  if (a.mode != 1) transform<false>(a, line, bb, live, v);
+  if (a.mode == 2) {
+    if (live)
+      each_value(a, a.rad[a.steps - 1], bb, v, [&](VT& x, int i) {
+        const T dn = a.Dn[qoff + (long)i * a.S];
+        x.x *= dn;
+        x.y *= dn;
+      });
+  }
+  if (a.mode != 0) transform<true>(a, line, bb, live, v);
+  if (live) {
+    VT* out = a.out + voff + base;
+    if (a.addx) {
+      const VT* add = a.addx + voff + base;
+      each_value(a, rl, bb, v, [&](VT& x, int i) { x = cadd(x, add[(long)i * a.S]); });
+    }
+    each_value(a, rl, bb, v, [&](VT& x, int i) { out[(long)i * a.S] = x; });
+  }
 }
 
 template <class VT>
@@ -397,10 +280,12 @@ cudaError_t run_pass(int d, int n, const VT* tw, const typename Real<VT>::T* Dn,
   a.addx = addx;
   a.tw = tw;
   a.n = n;
-  a.R = (n % 3 == 0) ? 3 : 1;
-  a.M = n / a.R;
-  a.logM = 0;
-  while ((1 << a.logM) < a.M) ++a.logM;
+  {  // radices: 4 as often as they go, a 2, a 3
+    int m = n % 3 == 0 ? n / 3 : n;
+    for (; m >= 4; m /= 4) a.rad[a.steps++] = 4;
+    if (m == 2) a.rad[a.steps++] = 2;
+    if (n % 3 == 0) a.rad[a.steps++] = 3;
+  }
   long S = 1;
   for (int i = 0; i < axis; ++i) S *= n;
   a.S = S;
@@ -409,25 +294,26 @@ cudaError_t run_pass(int d, int n, const VT* tw, const typename Real<VT>::T* Dn,
   a.vlines = N / n;
   a.vstride = N;
   a.nlines = a.vlines * nvec;
-  a.W = lines_per_cta(n, a.nlines, (int)sizeof(VT));
-  // axis > 0 lines are grouped W at a time inside one S-block: W must divide S
-  if (axis > 0)
-    while (a.W > 1 && (S % a.W)) a.W >>= 1;
-  a.pad = 1;
-  size_t smem = (size_t)a.W * (n + a.pad) * sizeof(VT);
-  long grid = (a.nlines + a.W - 1) / a.W;
+  a.U = (n + 3) / 4;
+  if (a.U > 1024) return cudaErrorInvalidValue;
+  // lines per CTA: eight (whole 128-byte lines across an axis > 0) while there are six CTAs
+  // per SM, down to two (whole sectors) and to a full warp
+  int least = axis > 0 ? 2 : 1;
+  while (least * a.U < 32) least *= 2;
+  a.W = std::max(8, least);
+  while (a.W > least && a.nlines / a.W < 912) a.W /= 2;
+  while (a.W > 1 && (a.W * a.U > 1024 || (axis > 0 && S % a.W))) a.W /= 2;
+  a.ld = (n + n / 8 + 1) | 1;
+  const size_t smem = (size_t)a.W * a.ld * sizeof(VT);
+  const unsigned grid = (unsigned)((a.nlines + a.W - 1) / a.W);
   static bool attr_set = false;
   if (!attr_set) {
-    cudaFuncSetAttribute(fft_pass_kernel<VT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(fft_pass_kernel<VT, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(fft_pass_kernel<VT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr_set = true;
   }
   const double es = sizeof(VT);
   ProfScope ps(PROF_FFT, st);
-  if (a.R == 3)
-    fft_pass_kernel<VT, 3><<<(unsigned)grid, kThreads, smem, st>>>(a);
-  else
-    fft_pass_kernel<VT, 1><<<(unsigned)grid, kThreads, smem, st>>>(a);
+  fft_pass_kernel<VT><<<grid, (unsigned)((a.W * a.U + 31) / 32 * 32), smem, st>>>(a);
   ps.done((double)N * nvec * (2 * es + (q ? es / 2 : 0.0) + (mode == 2 ? es / 2 : 0.0) +
                              (addx ? es : 0.0)),
           1, st);

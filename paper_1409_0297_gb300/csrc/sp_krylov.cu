@@ -19,63 +19,74 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-__device__ __forceinline__ void chunk_of(long N, long* c0, long* c1) {
-  long per = (N + gridDim.x - 1) / gridDim.x;
-  *c0 = (long)blockIdx.x * per;
-  *c1 = min(N, *c0 + per);
-}
+// A CTA takes the elements i = 256 (blockIdx.x + g gridDim.x) + thread: with whole units of
+// 256 dealt out in turn, the SMs' shares of the FP64 work differ by one unit (contiguous
+// shares over 256 CTAs left the 152 SMs 19 % apart at N = 262144).
+__device__ __forceinline__ long first_of() { return (long)blockIdx.x * kThr + threadIdx.x; }
+__device__ __forceinline__ long stride_of() { return (long)gridDim.x * kThr; }
 
 // The Krylov basis V is read with the evict-first hint (it is larger than L2 at
 // 512^2 and streams through it every iteration), so the preconditioner's data stays.
 // partial[j * nblk + blk] = sum over the CTA's chunk of conj(V_j) w.  Each thread
 // walks its elements of the chunk with w[i] in registers and accumulates eight
 // vectors at a time (independent FMA chains; w is re-read once per eight
-// vectors, V once); the sums are reduced over the CTA in shared memory in a fixed
-// order.
-__device__ void chunk_dots(const double2* V, long ldv, int nv, const double2* w, long c0, long c1,
+// vectors, V once).  The 16 sums of a warp are reduced together, each exchange halving the
+// values a lane still holds (15 additions and one more instead of 80: with four elements
+// per thread the 80 were as much FP64 work as the products), then over the CTA in shared
+// memory in a fixed order.
+__device__ void chunk_dots(const double2* V, long ldv, int nv, const double2* w, long N,
                            double2* partial) {
   constexpr int kJ = 8;
-  __shared__ double2 red[kJ][kThr / 32];
+  __shared__ double red[2 * kJ][kThr / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int j0 = 0; j0 < nv; j0 += kJ) {
     const int nj = min(kJ, nv - j0);
-    double sr[kJ], si[kJ];
+    double sum[2 * kJ];  // real parts, imaginary parts
 #pragma unroll
-    for (int q = 0; q < kJ; ++q) sr[q] = si[q] = 0.0;
-    for (long i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
+    for (int q = 0; q < 2 * kJ; ++q) sum[q] = 0.0;
+    for (long i = first_of(); i < N; i += stride_of()) {
       const double2 wi = w[i];
 #pragma unroll
       for (int q = 0; q < kJ; ++q) {
         if (q < nj) {
           const double2 v = __ldcs(V + (long)(j0 + q) * ldv + i);  // conj(v) w; evict-first
-          sr[q] = fma(v.x, wi.x, fma(v.y, wi.y, sr[q]));
-          si[q] = fma(v.x, wi.y, fma(-v.y, wi.x, si[q]));
+          sum[q] = fma(v.x, wi.x, fma(v.y, wi.y, sum[q]));
+          sum[kJ + q] = fma(v.x, wi.y, fma(-v.y, wi.x, sum[kJ + q]));
         }
       }
     }
 #pragma unroll
-    for (int q = 0; q < kJ; ++q) {
-      const double a = warp_sum(sr[q]), b = warp_sum(si[q]);
-      if (lane == 0) red[q][warp] = make_double2(a, b);
+    for (int o = 16, m = kJ; m > 0; o >>= 1, m >>= 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int q = 0; q < kJ; ++q)
+        if (q < m) {
+          const double give = up ? sum[q] : sum[q + m], keep = up ? sum[q + m] : sum[q];
+          sum[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
     }
+    sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], 1);
+    if (!(lane & 1)) red[lane >> 1][warp] = sum[0];  // lanes 2 i, 2 i + 1 hold sum i
     __syncthreads();
-    if (threadIdx.x < nj) {
-      double a = 0, b = 0;
-      for (int x = 0; x < nw; ++x) {
-        a += red[threadIdx.x][x].x;
-        b += red[threadIdx.x][x].y;
+    if (threadIdx.x < 2 * kJ) {
+      double a = 0;
+      for (int x = 0; x < nw; ++x) a += red[threadIdx.x][x];
+      const int q = threadIdx.x & (kJ - 1);
+      if (q < nj) {
+        double2* p = partial + (long)(j0 + q) * gridDim.x + blockIdx.x;
+        (threadIdx.x < kJ ? p->x : p->y) = a;
       }
-      partial[(long)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = make_double2(a, b);
     }
     __syncthreads();
   }
 }
 
 // w_i -= sum_j V_j[i] hs_j over the chunk, four independent partial sums (FP64 FMA
-// latency); hs in shared memory
-__device__ void chunk_update(const double2* V, long ldv, int nv, double2* w, long c0, long c1,
-                             const double2* hs) {
-  for (long i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
+// latency); hs in shared memory.  Returns the thread's sum of |w_i|^2.
+__device__ double chunk_update(const double2* V, long ldv, int nv, double2* w, long N,
+                               const double2* hs) {
+  double nrm = 0;
+  for (long i = first_of(); i < N; i += stride_of()) {
     double ax[4] = {0, 0, 0, 0}, ay[4] = {0, 0, 0, 0};
     int j = 0;
     for (; j + 4 <= nv; j += 4) {
@@ -92,18 +103,16 @@ __device__ void chunk_update(const double2* V, long ldv, int nv, double2* w, lon
       ay[0] = fma(v.x, hj.y, fma(v.y, hj.x, ay[0]));
     }
     const double2 wi = w[i];
-    w[i] = make_double2(wi.x - ((ax[0] + ax[1]) + (ax[2] + ax[3])),
-                        wi.y - ((ay[0] + ay[1]) + (ay[2] + ay[3])));
+    const double2 r = make_double2(wi.x - ((ax[0] + ax[1]) + (ax[2] + ax[3])),
+                                   wi.y - ((ay[0] + ay[1]) + (ay[2] + ay[3])));
+    w[i] = r;
+    nrm = fma(r.x, r.x, fma(r.y, r.y, nrm));
   }
+  return nrm;
 }
 
-// partial[blockIdx.x] = (sum over the chunk of |w_i|^2, 0)
-__device__ void chunk_norm2(const double2* w, long c0, long c1, double2* partial) {
-  double s = 0;
-  for (long i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
-    double2 v = w[i];
-    s = fma(v.x, v.x, fma(v.y, v.y, s));
-  }
+// partial[blockIdx.x] = (the threads' sums s added over the CTA, 0)
+__device__ void cta_norm2(double s, double2* partial) {
   __shared__ double red[kThr / 32];
   s = warp_sum(s);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -113,6 +122,16 @@ __device__ void chunk_norm2(const double2* w, long c0, long c1, double2* partial
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
     partial[blockIdx.x] = make_double2(t, 0);
   }
+}
+
+// partial[blockIdx.x] = (sum over the chunk of |w_i|^2, 0)
+__device__ void chunk_norm2(const double2* w, long N, double2* partial) {
+  double s = 0;
+  for (long i = first_of(); i < N; i += stride_of()) {
+    double2 v = w[i];
+    s = fma(v.x, v.x, fma(v.y, v.y, s));
+  }
+  cta_norm2(s, partial);
 }
 
 // sum_b partial[j * nblk + b] in a fixed order; called by one whole warp
@@ -130,22 +149,43 @@ __device__ double2 warp_reduce_partial(const double2* partial, int nblk, int j) 
 __device__ __forceinline__ double cabs2(double2 a) { return hypot(a.x, a.y); }
 
 // Column j of the Hessenberg matrix, earlier rotations, a new rotation, the
-// residual estimate |gamma_{j+1}|.  Single thread.
+// residual estimate |gamma_{j+1}|.  One warp: the column's entries and the rotations are
+// staged in shared memory (as one thread's chain of loads and stores in device memory the
+// j rotations took ~0.3 us each), lane 0 applies the rotations in order.
 __device__ void givens_col(double2* H, int ldh, int j, const double2* h1, const double2* h2,
                            double nrm, double* cs, double2* sn, double2* gam, double* est) {
+  constexpr int kStage = 256;  // rotations staged at a time
+  __shared__ double2 sc[kStage + 1], ss[kStage];
+  __shared__ double sr[kStage];
+  const int lane = threadIdx.x & 31;
   double2* col = H + (long)j * ldh;
-  for (int i = 0; i <= j; ++i) col[i] = make_double2(h1[i].x + h2[i].x, h1[i].y + h2[i].y);
-  col[j + 1] = make_double2(nrm, 0.0);
-  for (int i = 0; i < j; ++i) {
-    double c = cs[i];
-    double2 s = sn[i], a = col[i], b = col[i + 1];
-    // [c, s; -conj(s), c] (a, b)
-    double2 t0 = make_double2(c * a.x + (s.x * b.x - s.y * b.y), c * a.y + (s.x * b.y + s.y * b.x));
-    double2 t1 = make_double2(-(s.x * a.x + s.y * a.y) + c * b.x, -(s.x * a.y - s.y * a.x) + c * b.y);
-    col[i] = t0;
-    col[i + 1] = t1;
+  double2 a = make_double2(0, 0);  // lane 0: the entry the next rotation starts from
+  for (int i0 = 0; i0 <= j; i0 += kStage) {
+    const int cnt = min(kStage, j - i0);  // rotations i0 .. i0 + cnt - 1, entries up to i0 + cnt
+    __syncwarp();
+    for (int i = lane; i <= cnt; i += 32)
+      sc[i] = make_double2(h1[i0 + i].x + h2[i0 + i].x, h1[i0 + i].y + h2[i0 + i].y);
+    for (int i = lane; i < cnt; i += 32) {
+      sr[i] = cs[i0 + i];
+      ss[i] = sn[i0 + i];
+    }
+    __syncwarp();
+    if (lane == 0) {
+      if (i0 == 0) a = sc[0];
+      for (int i = 0; i < cnt; ++i) {
+        const double c = sr[i];
+        const double2 s = ss[i], b = sc[i + 1];
+        // [c, s; -conj(s), c] (a, b)
+        sc[i] = make_double2(c * a.x + (s.x * b.x - s.y * b.y), c * a.y + (s.x * b.y + s.y * b.x));
+        a = make_double2(-(s.x * a.x + s.y * a.y) + c * b.x, -(s.x * a.y - s.y * a.x) + c * b.y);
+      }
+    }
+    __syncwarp();
+    for (int i = lane; i < cnt; i += 32) col[i0 + i] = sc[i];
+    if (cnt < kStage) break;
   }
-  double2 a = col[j], b = col[j + 1];
+  if (lane != 0) return;
+  double2 b = make_double2(nrm, 0.0);
   double c;
   double2 s;
   double aa = cabs2(a), bb = cabs2(b);
@@ -212,9 +252,7 @@ __device__ __forceinline__ void combine_at(const double2* Z, long ldz, int k, co
 
 __global__ void __launch_bounds__(kThr) dots_kernel(const double2* V, long ldv, int nv,
                                                     const double2* w, long N, double2* partial) {
-  long c0, c1;
-  chunk_of(N, &c0, &c1);
-  chunk_dots(V, ldv, nv, w, c0, c1, partial);
+  chunk_dots(V, ldv, nv, w, N, partial);
 }
 
 __global__ void __launch_bounds__(kThr) update_dots_kernel(const double2* V, long ldv, int nv,
@@ -223,12 +261,10 @@ __global__ void __launch_bounds__(kThr) update_dots_kernel(const double2* V, lon
   __shared__ double2 hs[1024];
   for (int j = threadIdx.x; j < nv; j += blockDim.x) hs[j] = h[j];
   __syncthreads();
-  long c0, c1;
-  chunk_of(N, &c0, &c1);
-  chunk_update(V, ldv, nv, w, c0, c1, hs);
+  chunk_update(V, ldv, nv, w, N, hs);
   if (partial) {
     __syncthreads();
-    chunk_dots(V, ldv, nv, w, c0, c1, partial);
+    chunk_dots(V, ldv, nv, w, N, partial);
   }
 }
 
@@ -241,9 +277,7 @@ __global__ void reduce_partials_kernel(const double2* partial, int nblk, int nv,
 }
 
 __global__ void __launch_bounds__(kThr) norm2_kernel(const double2* w, long N, double2* partial) {
-  long c0, c1;
-  chunk_of(N, &c0, &c1);
-  chunk_norm2(w, c0, c1, partial);
+  chunk_norm2(w, N, partial);
 }
 
 __global__ void sqrt_kernel(const double2* s, double* out) { out[0] = sqrt(s[0].x); }
@@ -279,7 +313,6 @@ __global__ void start_kernel(const double2* r, long N, const double* nrm, double
 __global__ void givens_kernel(double2* H, int ldh, int j, const double2* h1, const double2* h2,
                               const double* nrm, double* cs, double2* sn, double2* gam,
                               double* est) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   givens_col(H, ldh, j, h1, h2, nrm[0], cs, sn, gam, est);
 }
 
@@ -333,13 +366,11 @@ __global__ void kb_copy_kernel(KBatch b, double2* vec, int to_z) {
 __global__ void __launch_bounds__(kThr) kb_dots_kernel(KBatch b) {
   const int i = blockIdx.y;
   if (!inst_cont(b, i)) return;
-  long c0, c1;
-  chunk_of(b.N, &c0, &c1);
-  chunk_dots(b.V + i * b.sV, b.N, b.head[i].j + 1, b.w + i * b.N, c0, c1, b.partial + i * b.sP);
+  chunk_dots(b.V + i * b.sV, b.N, b.head[i].j + 1, b.w + i * b.N, b.N, b.partial + i * b.sP);
 }
 
-// w_i -= V_i h_i (h = h1 if second = 0, else h2); then, if second = 0, h2 = V_i^H w_i
-// partials
+// w_i -= V_i h_i (h = h1 if second = 0, else h2); then the partials of h2 = V_i^H w_i
+// (second = 0) or of |w_i|^2 (second = 1, added in chunk_norm2's order)
 __global__ void __launch_bounds__(kThr) kb_update_dots_kernel(KBatch b, int second) {
   const int i = blockIdx.y;
   if (!inst_cont(b, i)) return;
@@ -348,14 +379,14 @@ __global__ void __launch_bounds__(kThr) kb_update_dots_kernel(KBatch b, int seco
   __shared__ double2 hs[1024];
   for (int j = threadIdx.x; j < nv; j += blockDim.x) hs[j] = h[j];
   __syncthreads();
-  long c0, c1;
-  chunk_of(b.N, &c0, &c1);
   const double2* V = b.V + i * b.sV;
   double2* w = b.w + i * b.N;
-  chunk_update(V, b.N, nv, w, c0, c1, hs);
-  if (!second) {
+  const double s = chunk_update(V, b.N, nv, w, b.N, hs);
+  if (second) {
+    cta_norm2(s, b.partial + i * b.sP);
+  } else {
     __syncthreads();
-    chunk_dots(V, b.N, nv, w, c0, c1, b.partial + i * b.sP);
+    chunk_dots(V, b.N, nv, w, b.N, b.partial + i * b.sP);
   }
 }
 
@@ -369,27 +400,27 @@ __global__ void kb_reduce_kernel(KBatch b, int which) {
   if ((threadIdx.x & 31) == 0) (which ? b.h2 : b.h1)[i * b.sh + j] = s;
 }
 
-// partials of |x_i|^2 (x with instance stride N); active = 1: only instances in a step
-__global__ void __launch_bounds__(kThr) kb_norm2_kernel(KBatch b, const double2* x, int active) {
+// partials of |x_i|^2 (x with instance stride N)
+__global__ void __launch_bounds__(kThr) kb_norm2_kernel(KBatch b, const double2* x) {
   const int i = blockIdx.y;
-  if (active && !inst_cont(b, i)) return;
-  long c0, c1;
-  chunk_of(b.N, &c0, &c1);
-  chunk_norm2(x + i * b.N, c0, c1, b.partial + i * b.sP);
+  chunk_norm2(x + i * b.N, b.N, b.partial + i * b.sP);
 }
 
 // nrm_i[slot] = sqrt(sum of the partials); one warp per instance
-__global__ void kb_norm_finish_kernel(KBatch b, int slot, int active) {
+__global__ void kb_norm_finish_kernel(KBatch b, int slot) {
   const int i = blockIdx.x;
-  if (active && !inst_cont(b, i)) return;
   const double2 s = warp_reduce_partial(b.partial + i * b.sP, b.nblk, 0);
   if (threadIdx.x == 0) b.nrm[i * 4 + slot] = sqrt(s.x);
 }
 
+// the norm from its partial sums, then the Hessenberg column; one warp per instance
 __global__ void kb_givens_kernel(KBatch b) {
   const int i = blockIdx.x;
-  if (threadIdx.x != 0 || !inst_cont(b, i)) return;
-  givens_col(b.H + i * b.sH, b.ldh, b.head[i].j, b.h1 + i * b.sh, b.h2 + i * b.sh, b.nrm[i * 4],
+  if (!inst_cont(b, i)) return;
+  const double2 s = warp_reduce_partial(b.partial + i * b.sP, b.nblk, 0);
+  const double nrm = sqrt(__shfl_sync(0xffffffffu, s.x, 0));
+  if (threadIdx.x == 0) b.nrm[i * 4] = nrm;
+  givens_col(b.H + i * b.sH, b.ldh, b.head[i].j, b.h1 + i * b.sh, b.h2 + i * b.sh, nrm,
              b.cs + i * b.sG, b.sn + i * b.sG, b.gam + i * b.sG, b.est + i * 4);
 }
 
@@ -580,15 +611,13 @@ cudaError_t kb_arnoldi(const KBatch& b, int I, int nv_max, cudaStream_t st) {
   kb_update_dots_kernel<<<gd, kThr, 0, st>>>(b, 0);
   kb_reduce_kernel<<<gr, 256, 0, st>>>(b, 1);
   kb_update_dots_kernel<<<gd, kThr, 0, st>>>(b, 1);
-  kb_norm2_kernel<<<gd, kThr, 0, st>>>(b, b.w, 1);
-  kb_norm_finish_kernel<<<I, 32, 0, st>>>(b, 0, 1);
   kb_givens_kernel<<<I, 32, 0, st>>>(b);
   return cudaGetLastError();
 }
 
 cudaError_t kb_norm(const KBatch& b, int I, const double2* x, int slot, cudaStream_t st) {
-  kb_norm2_kernel<<<dim3(b.nblk, I), kThr, 0, st>>>(b, x, 0);
-  kb_norm_finish_kernel<<<I, 32, 0, st>>>(b, slot, 0);
+  kb_norm2_kernel<<<dim3(b.nblk, I), kThr, 0, st>>>(b, x);
+  kb_norm_finish_kernel<<<I, 32, 0, st>>>(b, slot);
   return cudaGetLastError();
 }
 
@@ -626,6 +655,13 @@ cudaError_t kb_copy_nrm(const KBatch& b, int I, int from, int to, cudaStream_t s
 namespace sp {
 
 namespace {
+
+// contiguous share of the N elements of a CTA
+__device__ __forceinline__ void chunk_of(long N, long* c0, long* c1) {
+  const long per = (N + gridDim.x - 1) / gridDim.x;
+  *c0 = (long)blockIdx.x * per;
+  *c1 = min(N, *c0 + per);
+}
 
 __device__ __forceinline__ void chunk_dots32(const float2* V, long ldv, int nv, const float2* w,
                                              long c0, long c1, double2* partial) {
