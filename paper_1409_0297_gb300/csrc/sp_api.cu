@@ -878,7 +878,10 @@ static sp_status setup_impl(int d, int n, int b, int P, const double* shifts, sp
     D.ib = c->opts.inv_block > 0 ? c->opts.inv_block
                                  : (S.k >= 16384 ? 2048 : (S.k >= 4096 ? 1024 : kInvBlockSize));
     D.pdl = c->opts.launch_overlap;
-    if (D.inv && c->opts.sweeps != 1) {
+    // fused sweeps pay on fronts with enough rows for a CTA: applying the preconditioner,
+    // leaves of 289 (169) rows 0.411 against 0.430 (0.279 against 0.308) ms with launch chains,
+    // leaves of 49 and 69 rows (four 192^2 problems) 0.308 against 0.266 ms
+    if (D.inv && (c->opts.sweeps == 2 || (c->opts.sweeps == 0 && S.m >= 128))) {
       int C = 0, NT = 0;
       if (sweep_fused_config(prec, D.nf, S.m, S.k, num_sms, max_cluster, c->opts.sweeps == 2, &C,
                              &NT)) {
