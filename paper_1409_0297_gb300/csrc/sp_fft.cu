@@ -135,25 +135,36 @@ constexpr int kVal = 6;
 template <int r>
 constexpr int kPer = r == 4 ? 1 : 2;
 
-// One step of radix r at l for the butterflies b = bb + j U of a line: from the values in v
-// (loaded: already there) or from the line in shared memory, to registers.
+// The twiddles of a step of radix r at l, w_{l r}^{(b mod l) k} for k = 1 .. r - 1 of each
+// butterfly, loaded ahead of the exchange that the step waits for.
 template <int r, bool INV, class VT>
-__device__ __forceinline__ void step_reg(const PassArgs<VT>& a, const VT* line, int bb, bool loaded,
-                                         int l, VT* v) {
+__device__ __forceinline__ void load_tw(const PassArgs<VT>& a, int bb, int l, VT* tw) {
+  const int nb = a.n / r;
+#pragma unroll
+  for (int j = 0; j < kPer<r>; ++j) {
+    const int b = bb + j * a.U;
+    const int t = b < nb ? (b % l) * (nb / l) : 0;  // w_{l r}^1 = w_n^(n / (l r))
+#pragma unroll
+    for (int k = 1; k < r; ++k) tw[j * (r - 1) + k - 1] = tw_at<INV>(a, t * k);
+  }
+}
+
+// One step of radix r at l for the butterflies b = bb + j U of a line: from the values in v
+// (first: already there, no twiddles) or from the line in shared memory, to registers.
+template <int r, bool INV, class VT>
+__device__ __forceinline__ void step_reg(const PassArgs<VT>& a, const VT* line, int bb, bool first,
+                                         const VT* tw, VT* v) {
   const int nb = a.n / r;
 #pragma unroll
   for (int j = 0; j < kPer<r>; ++j) {
     const int b = bb + j * a.U;
     if (b >= nb) continue;
     VT* x = v + j * r;
-    if (!loaded) {
+    if (!first) {
 #pragma unroll
       for (int k = 0; k < r; ++k) x[k] = line[spos(b + k * nb)];
-    }
-    if (l > 1) {
-      const int t = (b % l) * (nb / l);  // w_{l r}^1 = w_n^(n / (l r))
 #pragma unroll
-      for (int k = 1; k < r; ++k) x[k] = cmul(x[k], tw_at<INV>(a, t * k));
+      for (int k = 1; k < r; ++k) x[k] = cmul(x[k], tw[j * (r - 1) + k - 1]);
     }
     dft_reg<r, INV>(x);
   }
@@ -176,16 +187,23 @@ __device__ __forceinline__ void put_line(const PassArgs<VT>& a, VT* line, int bb
 // reverse.
 template <bool INV, class VT>
 __device__ __forceinline__ void transform(const PassArgs<VT>& a, VT* line, int bb, bool live, VT* v) {
+  VT tw[4];  // kPer (r - 1) twiddles of the next step
   int l = 1;
   for (int s = 0; s < a.steps; ++s) {
     const int r = a.rad[INV ? a.steps - 1 - s : s];
     const bool first = s == 0, last = s == a.steps - 1;
     if (live) {
-      if (r == 4) step_reg<4, INV>(a, line, bb, first, l, v);
-      else if (r == 2) step_reg<2, INV>(a, line, bb, first, l, v);
-      else step_reg<3, INV>(a, line, bb, first, l, v);
+      if (r == 4) step_reg<4, INV>(a, line, bb, first, tw, v);
+      else if (r == 2) step_reg<2, INV>(a, line, bb, first, tw, v);
+      else step_reg<3, INV>(a, line, bb, first, tw, v);
     }
     if (!last) {
+      const int nx = a.rad[INV ? a.steps - 2 - s : s + 1], ln = l * r;
+      if (live) {
+        if (nx == 4) load_tw<4, INV>(a, bb, ln, tw);
+        else if (nx == 2) load_tw<2, INV>(a, bb, ln, tw);
+        else load_tw<3, INV>(a, bb, ln, tw);
+      }
       __syncthreads();  // the line has been read
       if (live) {
         if (r == 4) put_line<4>(a, line, bb, l, v);
