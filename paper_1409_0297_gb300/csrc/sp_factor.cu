@@ -1293,30 +1293,48 @@ __global__ void __launch_bounds__(256) gemm_sub_kernel(int M, int N, int K, cons
   }
 }
 
-// Batched C = beta C + alpha A B (column-major, any K) with triangle-aware K
+// One batched product C = beta C + alpha A B (column-major, any K) with triangle-aware K
 // ranges: tri_a = 1 when A is lower triangular (A[r, l] = 0 for l > r), 2 when
 // upper (A[r, l] = 0 for l < r); tri_b = 1 when B is lower (B[l, c] = 0 for
 // l < c), 2 when upper (B[l, c] = 0 for l > c).  Zero tiles are skipped, entries
 // inside a computed tile must hold their zeros.  beta is 0 or 1.
+// batch index = outer * nb2 + inner with strides (sA, sB, sC) and (sA2, sB2, sC2)
+template <class T>
+struct GemmSide {
+  int M = 0, N = 0, K = 0;
+  const T* A = nullptr;
+  int lda = 0;
+  long sA = 0, sA2 = 0;
+  const T* B = nullptr;
+  int ldb = 0;
+  long sB = 0, sB2 = 0;
+  T* C = nullptr;
+  int ldc = 0;
+  long sC = 0, sC2 = 0;
+  int tri_a = 0, tri_b = 0;
+};
+
+// A launch takes one product or two independent ones of a batch (blockIdx.z: the inverses
+// of L and U, whose chains of small products then cost one launch each instead of two).
 template <class T, int TILE>
-__global__ void __launch_bounds__(256) gemm_gen_kernel(int M, int N, int K, T alpha, int beta_one,
-                                                       const T* A, int lda, long sA, const T* B,
-                                                       int ldb, long sB, T* C, int ldc, long sC,
-                                                       int tilesM, int tri_a, int tri_b, int nb2,
-                                                       long sA2, long sB2, long sC2) {
+__global__ void __launch_bounds__(256) gemm_gen_kernel(GemmSide<T> g0, GemmSide<T> g1, T alpha,
+                                                       int beta_one, int nb2) {
   constexpr int R = TILE / 16;  // outputs per thread along each dimension
-  // batch index = outer * nb2 + inner with strides (sA, sB, sC) and (sA2, sB2, sC2)
+  const GemmSide<T> g = blockIdx.z ? g1 : g0;
+  const int M = g.M, N = g.N, lda = g.lda, ldb = g.ldb, ldc = g.ldc;
+  const int tilesM = (M + TILE - 1) / TILE, tilesN = (N + TILE - 1) / TILE;
+  if ((int)blockIdx.x >= tilesM * tilesN) return;
   const long bo = blockIdx.y / nb2, bi = blockIdx.y % nb2;
-  A += bo * sA + bi * sA2;
-  B += bo * sB + bi * sB2;
-  C += bo * sC + bi * sC2;
+  const T* A = g.A + bo * g.sA + bi * g.sA2;
+  const T* B = g.B + bo * g.sB + bi * g.sB2;
+  T* C = g.C + bo * g.sC + bi * g.sC2;
   const int tr = blockIdx.x % tilesM, tc = blockIdx.x / tilesM;
   const int r0 = tr * TILE, c0 = tc * TILE;
-  int klo = 0, khi = K;
-  if (tri_a == 1) khi = min(khi, r0 + TILE);
-  if (tri_a == 2) klo = max(klo, r0);
-  if (tri_b == 1) klo = max(klo, c0);
-  if (tri_b == 2) khi = min(khi, c0 + TILE);
+  int klo = 0, khi = g.K;
+  if (g.tri_a == 1) khi = min(khi, r0 + TILE);
+  if (g.tri_a == 2) klo = max(klo, r0);
+  if (g.tri_b == 1) klo = max(klo, c0);
+  if (g.tri_b == 2) khi = min(khi, c0 + TILE);
   __shared__ T As[kNB][TILE];
   __shared__ T Bs[kNB][TILE + 1];
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
@@ -1570,24 +1588,26 @@ __device__ __forceinline__ double add_digits(double acc, const float* S, int es,
 // alpha = -1 (neg = the sign bit) or 1.
 template <bool ONE>
 __global__ void __launch_bounds__(256, ONE ? 2 : 1)
-    gemm_f64_kernel(int M, int N, int K, unsigned neg, int beta_one, const double* A, int lda,
-                    long sA, const double* B, int ldb, long sB, double* C, int ldc, long sC,
-                    int tilesM, int tri_a, int tri_b, int nb2, long sA2, long sB2, long sC2) {
+    gemm_f64_kernel(GemmSide<double> g0, GemmSide<double> g1, unsigned neg, int beta_one, int nb2) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __half* Ad = reinterpret_cast<__half*>(smraw);
   __half* Bd = Ad + kDig * kDigPlane;
   __shared__ int eA[4][kDigT], eB[kDigT];
   __shared__ int s_plain;
+  const GemmSide<double> g = blockIdx.z ? g1 : g0;
+  const int M = g.M, N = g.N, lda = g.lda, ldb = g.ldb, ldc = g.ldc;
+  const int tilesM = (M + kDigT - 1) / kDigT, tilesN = (N + kDigT - 1) / kDigT;
+  if ((int)blockIdx.x >= tilesM * tilesN) return;
   const long bo = blockIdx.y / nb2, bi = blockIdx.y % nb2;
-  A += bo * sA + bi * sA2;
-  B += bo * sB + bi * sB2;
-  C += bo * sC + bi * sC2;
+  const double* A = g.A + bo * g.sA + bi * g.sA2;
+  const double* B = g.B + bo * g.sB + bi * g.sB2;
+  double* C = g.C + bo * g.sC + bi * g.sC2;
   const int r0 = (blockIdx.x % tilesM) * kDigT, c0 = (blockIdx.x / tilesM) * kDigT;
-  int klo = 0, khi = K;
-  if (tri_a == 1) khi = min(khi, r0 + kDigT);
-  if (tri_a == 2) klo = max(klo, r0);
-  if (tri_b == 1) klo = max(klo, c0);
-  if (tri_b == 2) khi = min(khi, c0 + kDigT);
+  int klo = 0, khi = g.K;
+  if (g.tri_a == 1) khi = min(khi, r0 + kDigT);
+  if (g.tri_a == 2) klo = max(klo, r0);
+  if (g.tri_b == 1) klo = max(klo, c0);
+  if (g.tri_b == 2) khi = min(khi, c0 + kDigT);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // this thread's outputs: half s, n-tile t, register i: row rw + 8 (i / 2), column
   // cw + 16 s + 8 t + (i & 1)
@@ -1718,25 +1738,21 @@ __global__ void __launch_bounds__(256, ONE ? 2 : 1)
   }
 }
 
-void gemm_f64(int M, int N, int K, bool minus, bool beta_one, const double* A, int lda, long sA,
-              const double* B, int ldb, long sB, double* C, int ldc, long sC, int batch, int tri_a,
-              int tri_b, cudaStream_t st, int nb2 = 1, long sA2 = 0, long sB2 = 0, long sC2 = 0) {
-  const int tilesM = (M + kDigT - 1) / kDigT, tilesN = (N + kDigT - 1) / kDigT;
+void gemm_f64(const GemmSide<double>& g0, const GemmSide<double>* g1, bool minus, bool beta_one,
+              int batch, int nb2, cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(gemm_f64_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDigSmem);
     cudaFuncSetAttribute(gemm_f64_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDigSmem);
     attr = true;
   }
-  dim3 g((unsigned)(tilesM * tilesN), (unsigned)(batch * nb2));
-  const unsigned neg = minus ? 0x80000000u : 0u;
-  if (K <= 32 && beta_one)
-    gemm_f64_kernel<true><<<g, 256, kDigSmem, st>>>(M, N, K, neg, 1, A, lda, sA, B, ldb, sB, C, ldc, sC,
-                                                    tilesM, tri_a, tri_b, nb2, sA2, sB2, sC2);
-  else
-    gemm_f64_kernel<false><<<g, 256, kDigSmem, st>>>(M, N, K, neg, beta_one ? 1 : 0, A, lda, sA, B, ldb,
-                                                     sB, C, ldc, sC, tilesM, tri_a, tri_b, nb2, sA2, sB2,
-                                                     sC2);
+  auto tiles = [](const GemmSide<double>& g) {
+    return ((g.M + kDigT - 1) / kDigT) * ((g.N + kDigT - 1) / kDigT);
+  };
+  dim3 gr((unsigned)(g1 ? std::max(tiles(g0), tiles(*g1)) : tiles(g0)), (unsigned)(batch * nb2), g1 ? 2 : 1);
+  const bool one = g0.K <= 32 && (!g1 || g1->K <= 32) && beta_one;
+  auto kern = one ? gemm_f64_kernel<true> : gemm_f64_kernel<false>;
+  kern<<<gr, 256, kDigSmem, st>>>(g0, g1 ? *g1 : g0, minus ? 0x80000000u : 0u, beta_one ? 1 : 0, nb2);
 }
 
 template <class T>
@@ -1744,7 +1760,8 @@ void gemm_sub(int M, int N, int K, const T* A, int lda, long sA, const T* B, int
               T* C, int ldc, long sC, int batch, cudaStream_t st, int tile = 0) {
   if (M <= 0 || N <= 0 || K <= 0) return;
   if constexpr (sizeof(T) == sizeof(double)) {
-    gemm_f64(M, N, K, true, true, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, 0, 0, st);
+    GemmSide<T> g{M, N, K, A, lda, sA, 0, B, ldb, sB, 0, C, ldc, sC, 0, 0, 0};
+    gemm_f64(g, nullptr, true, true, batch, 1, st);
   } else {
     // padded work of 64- and 32-wide tiles relative to M N
     const double w64 = (double)((M + 63) / 64 * 64) * ((N + 63) / 64 * 64);
@@ -1759,24 +1776,21 @@ void gemm_sub(int M, int N, int K, const T* A, int lda, long sA, const T* B, int
   }
 }
 
+// one product (g1 null) or two, alpha = -1 (minus) or 1
 template <class T>
-void gemm_gen(int M, int N, int K, T alpha, bool beta_one, const T* A, int lda, long sA,
-              const T* B, int ldb, long sB, T* C, int ldc, long sC, int batch, int tri_a,
-              int tri_b, cudaStream_t st, int nb2 = 1, long sA2 = 0, long sB2 = 0, long sC2 = 0,
-              int tile = 0) {
-  if (M <= 0 || N <= 0 || K <= 0 || batch <= 0 || nb2 <= 0) return;
-  if constexpr (sizeof(T) == sizeof(double)) {  // every caller's alpha is 1 or -1
-    gemm_f64(M, N, K, alpha < 0, beta_one, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, tri_a, tri_b, st,
-             nb2, sA2, sB2, sC2);
+void gemm_gen(const GemmSide<T>& g0, const GemmSide<T>* g1, bool minus, bool beta_one, int batch,
+              int nb2, int tile, cudaStream_t st) {
+  if (g0.M <= 0 || g0.N <= 0 || g0.K <= 0 || batch <= 0 || nb2 <= 0) return;
+  if constexpr (sizeof(T) == sizeof(double)) {
+    gemm_f64(g0, g1, minus, beta_one, batch, nb2, st);
   } else {
+    auto tiles = [&](const GemmSide<T>& g, int t) { return (long)((g.M + t - 1) / t) * ((g.N + t - 1) / t); };
     // a small problem takes 32 x 32 tiles: four times the CTAs
-    const long big = (long)((M + kTile - 1) / kTile) * ((N + kTile - 1) / kTile) * batch * nb2;
-    const int t = tile == 32 || (tile == 0 && big < 304) ? 32 : kTile;
-    const int tilesM = (M + t - 1) / t, tilesN = (N + t - 1) / t;
-    dim3 g(tilesM * tilesN, batch * nb2);
+    const int t = tile == 32 || (tile == 0 && tiles(g0, kTile) * batch * nb2 < 304) ? 32 : kTile;
+    dim3 gr((unsigned)(g1 ? std::max(tiles(g0, t), tiles(*g1, t)) : tiles(g0, t)), (unsigned)(batch * nb2),
+            g1 ? 2 : 1);
     auto kern = t == 32 ? gemm_gen_kernel<T, 32> : gemm_gen_kernel<T, kTile>;
-    kern<<<g, 256, 0, st>>>(M, N, K, alpha, beta_one ? 1 : 0, A, lda, sA, B, ldb, sB, C, ldc, sC, tilesM,
-                            tri_a, tri_b, nb2, sA2, sB2, sC2);
+    kern<<<gr, 256, 0, st>>>(g0, g1 ? *g1 : g0, minus ? (T)-1 : (T)1, beta_one ? 1 : 0, nb2);
   }
 }
 
@@ -1787,12 +1801,13 @@ void gemm_gen(int M, int N, int K, T alpha, bool beta_one, const T* A, int lda, 
 // Recursive doubling on the diagonal blocks (32, 64, 128, ... up to Bsz):
 //   [A 0; B C]^{-1} = [A^{-1} 0; -C^{-1} (B A^{-1}), C^{-1}]
 //   [A B; 0 C]^{-1} = [A^{-1}, -(A^{-1} B) C^{-1}; 0 C^{-1}]
-// with the two products of each merge as batched GEMMs over fronts and pairs.
+// with the two products of each merge as batched GEMMs over fronts, pairs and the two
+// triangles.
 // Storage: the inverses Xl, Xu keep entry (i, j) of a diagonal block at
 // i + j Bsz (a column-major array with leading dimension Bsz whose columns
 // overlap: the diagonal blocks never collide, and a pair's diagonal step is
-// 2 s (1 + Bsz) everywhere), k (Bsz + 1) entries per front; the work array W
-// holds pair p's product at rows [2ps, 2ps+s) of a k x Bsz/2 block per front.
+// 2 s (1 + Bsz) everywhere), k (Bsz + 1) entries per front; the work arrays Wl, Wu
+// hold pair p's product at rows [2ps, 2ps+s) of a k x Bsz/2 block per front.
 template <class T>
 void invert_triangles(DevLevel& L, T* scratch, int Bsz, cudaStream_t st) {
   const int k = L.k, m = L.m, nf = L.nf;
@@ -1802,7 +1817,8 @@ void invert_triangles(DevLevel& L, T* scratch, int Bsz, cudaStream_t st) {
   T* F = (T*)L.front;
   T* Xl = scratch;
   T* Xu = scratch + sX * nf;
-  T* W = scratch + 2 * sX * nf;
+  T* Wl = scratch + 2 * sX * nf;
+  T* Wu = Wl + sW * nf;
   cudaMemsetAsync(Xl, 0, sizeof(T) * sX * nf, st);
   cudaMemsetAsync(Xu, 0, sizeof(T) * sX * nf, st);
   const int nb = (k + kNB - 1) / kNB;
@@ -1830,18 +1846,18 @@ void invert_triangles(DevLevel& L, T* scratch, int Bsz, cudaStream_t st) {
       }
       if (cnt <= 0) continue;
       const int a0 = p0 * 2 * s, c0 = a0 + s;
-      // lower: W = B Ainv (B = L[c0.., a0..], Ainv lower), Xl[c0.., a0..] = -Cinv W
-      gemm_gen<T>(sc, s, s, (T)1, false, F + c0 + (long)a0 * m, m, mm, Xl + a0 + (long)a0 * ldx,
-                  ldx, sX, W + a0, k, sW, nf, 0, 1, st, cnt, ps_m, ps_x, ps_w, L.gen_tile);
-      gemm_gen<T>(sc, s, sc, (T)-1, false, Xl + c0 + (long)c0 * ldx, ldx, sX, W + a0, k, sW,
-                  Xl + c0 + (long)a0 * ldx, ldx, sX, nf, 1, 0, st, cnt, ps_x, ps_w, ps_x,
-                  L.gen_tile);
-      // upper: W = Ainv B (B = U[a0.., c0..], Ainv upper), Xu[a0.., c0..] = -W Cinv
-      gemm_gen<T>(s, sc, s, (T)1, false, Xu + a0 + (long)a0 * ldx, ldx, sX, F + a0 + (long)c0 * m,
-                  m, mm, W + a0, k, sW, nf, 2, 0, st, cnt, ps_x, ps_m, ps_w, L.gen_tile);
-      gemm_gen<T>(s, sc, sc, (T)-1, false, W + a0, k, sW, Xu + c0 + (long)c0 * ldx, ldx, sX,
-                  Xu + a0 + (long)c0 * ldx, ldx, sX, nf, 0, 2, st, cnt, ps_w, ps_x, ps_x,
-                  L.gen_tile);
+      // lower: Wl = B Ainv (B = L[c0.., a0..], Ainv lower), Xl[c0.., a0..] = -Cinv Wl;
+      // upper: Wu = Ainv B (B = U[a0.., c0..], Ainv upper), Xu[a0.., c0..] = -Wu Cinv
+      const GemmSide<T> l1{sc, s, s, F + c0 + (long)a0 * m, m, mm, ps_m, Xl + a0 + (long)a0 * ldx, ldx, sX,
+                           ps_x, Wl + a0, k, sW, ps_w, 0, 1};
+      const GemmSide<T> u1{s, sc, s, Xu + a0 + (long)a0 * ldx, ldx, sX, ps_x, F + a0 + (long)c0 * m, m, mm,
+                           ps_m, Wu + a0, k, sW, ps_w, 2, 0};
+      gemm_gen<T>(l1, &u1, false, false, nf, cnt, L.gen_tile, st);
+      const GemmSide<T> l2{sc, s, sc, Xl + c0 + (long)c0 * ldx, ldx, sX, ps_x, Wl + a0, k, sW, ps_w,
+                           Xl + c0 + (long)a0 * ldx, ldx, sX, ps_x, 1, 0};
+      const GemmSide<T> u2{s, sc, sc, Wu + a0, k, sW, ps_w, Xu + c0 + (long)c0 * ldx, ldx, sX, ps_x,
+                           Xu + a0 + (long)c0 * ldx, ldx, sX, ps_x, 0, 2};
+      gemm_gen<T>(l2, &u2, true, false, nf, cnt, L.gen_tile, st);
     }
   }
   // fronts with fewer than Bsz eliminated rows have one k x k block (threads over the
@@ -2120,8 +2136,8 @@ void schur_update(DevLevel& L, T* F, int M, int N, int K, long offA, long offB, 
     }
   }
   ProfScope pg(PROF_LU_GEMM, st);
-  gemm_gen<T>(M, N, K, (T)-1, true, F + offA, L.m, mm, F + offB, L.m, mm, F + offC, L.m, mm, L.nf,
-              0, 0, st);
+  const GemmSide<T> g{M, N, K, F + offA, L.m, mm, 0, F + offB, L.m, mm, 0, F + offC, L.m, mm, 0, 0, 0};
+  gemm_gen<T>(g, nullptr, true, true, L.nf, 1, 0, st);
   pg.done(fl, 1, st);
 }
 
@@ -2317,21 +2333,17 @@ cudaError_t schur_update_raw(int prec, bool tc, bool split, int M, int N, int K,
   if (prec == SP_PREC_FP32 && tc)
     return tc_schur_update(M, N, K, (const float*)A, lda, sA, (const float*)B, ldb, sB, (float*)C,
                            ldc, sC, batch, packA, packB, split, status, st);
-  if (prec == SP_PREC_FP32) {
-    if (K <= kNB)
-      gemm_sub<float>(M, N, K, (const float*)A, lda, sA, (const float*)B, ldb, sB, (float*)C, ldc,
-                      sC, batch, st);
-    else
-      gemm_gen<float>(M, N, K, -1.f, true, (const float*)A, lda, sA, (const float*)B, ldb, sB,
-                      (float*)C, ldc, sC, batch, 0, 0, st);
-  } else {
-    if (K <= kNB)
-      gemm_sub<double>(M, N, K, (const double*)A, lda, sA, (const double*)B, ldb, sB, (double*)C,
-                       ldc, sC, batch, st);
-    else
-      gemm_gen<double>(M, N, K, -1.0, true, (const double*)A, lda, sA, (const double*)B, ldb, sB,
-                       (double*)C, ldc, sC, batch, 0, 0, st);
-  }
+  auto go = [&](auto t) {
+    using T = decltype(t);
+    if (K <= kNB) {
+      gemm_sub<T>(M, N, K, (const T*)A, lda, sA, (const T*)B, ldb, sB, (T*)C, ldc, sC, batch, st);
+    } else {
+      const GemmSide<T> g{M, N, K, (const T*)A, lda, sA, 0, (const T*)B, ldb, sB, 0, (T*)C, ldc, sC, 0, 0, 0};
+      gemm_gen<T>(g, nullptr, true, true, batch, 1, 0, st);
+    }
+  };
+  if (prec == SP_PREC_FP32) go(0.f);
+  else go(0.0);
   return cudaGetLastError();
 }
 
@@ -2343,7 +2355,7 @@ int factor_outer_block(int prec, bool tc, int m, int k) {
 }
 
 size_t invert_scratch_elems(int nf, int k, int ib) {
-  return (size_t)nf * ((size_t)2 * k * (ib + 1) + (size_t)k * (ib / 2));
+  return (size_t)nf * ((size_t)2 * k * (ib + 1) + (size_t)2 * k * (ib / 2));
 }
 
 cudaError_t factor_copy16(DevLevel& L, cudaStream_t st) {
