@@ -858,6 +858,13 @@ static sp_status setup_impl(int d, int n, int b, int P, const double* shifts, sp
       SP_CK(upload(c.get(), &D.asm_cvar, cvar));
     }
     SP_CK(upload(c.get(), &D.ea_map, S.ea_map));
+    if (S.mc > S.kc) {
+      const int nbd = S.mc - S.kc;
+      std::vector<int> inv((size_t)S.m << d, -1);
+      for (int dl = 0; dl < (1 << d); ++dl)
+        for (int i = 0; i < nbd; ++i) inv[(size_t)dl * S.m + S.ea_map[(size_t)dl * nbd + i]] = i;
+      SP_CK(upload(c.get(), &D.ea_inv, inv));
+    }
     SP_CK(dalloc(c.get(), &D.front, fsz * (size_t)D.nf * S.m * S.m));
     SP_CK(dalloc(c.get(), &D.perm, sizeof(int) * (size_t)D.nf * std::max(1, S.k)));
     SP_CK(dalloc(c.get(), &D.piv, sizeof(int) * (size_t)D.nf * std::max(1, S.k)));

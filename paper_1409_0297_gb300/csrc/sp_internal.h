@@ -65,6 +65,7 @@ struct DevLevel {
   int* asm_tidx = nullptr;
   int* asm_cvar = nullptr;
   int* ea_map = nullptr;    // 2^d x (mc - kc)
+  int* ea_inv = nullptr;    // 2^d x m: the entry of ea_map[child] that holds the row, or -1
   void* front = nullptr;    // nf x m x m of double (FP64) or float (FP32)
   int* perm = nullptr;      // nf x k row permutation of the eliminated block
   int* piv = nullptr;       // nf x k pivot rows (LAPACK style, 0-based within the front)

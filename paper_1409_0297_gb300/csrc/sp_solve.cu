@@ -27,7 +27,6 @@ namespace sp {
 namespace {
 
 constexpr int kBS = 32;
-constexpr size_t kVecSmem = 192 * 1024;  // largest vector staged in shared memory
 
 template <class VT> struct Scalar;
 template <> struct Scalar<double2> { using T = double; };
@@ -410,71 +409,44 @@ __global__ void __launch_bounds__(256) backward_kernel(const T* __restrict__ fro
 }
 
 // ---- sweeps of levels whose L11, U11 hold their inverses -------------------------
-// tmp (m per front): Pi b1 (k entries) then b2 (m - k entries).
+// tmp (m per front): Pi b1 (k entries) then b2 (m - k entries).  One thread per row: the
+// stencil output at the row's point (rows < k), then the children's update vectors through
+// the inverse of the extend-add maps (ea_inv[dl m + v]: the entry of child dl that lands in
+// row v, or -1) in the children's order, as gather_rhs adds them.  Rows spread over the GPU
+// where one CTA per front scattered the children one after the other (3D 64^3 root: 227 us
+// of an application of 2.28 ms).
 template <class VT>
 __global__ void __launch_bounds__(256) inv_gather_kernel(
     int d, int m, int k, int nb1, const int* __restrict__ gidx, const int* __restrict__ perm,
     const VT* __restrict__ rhsQ, const VT* __restrict__ cupd, int mc, int kc,
-    const int* __restrict__ ea_map, VT* tmp, long N, long custr) {
+    const int* __restrict__ ea_inv, VT* tmp, long N, long custr) {
   pdl_wait();
-  extern __shared__ unsigned char smraw[];
-  VT* b = reinterpret_cast<VT*>(smraw);
-  const int f = blockIdx.x;
-  rhsQ += blockIdx.y * N;
-  if (cupd) cupd += blockIdx.y * custr;
-  tmp += (long)blockIdx.y * gridDim.x * m;
-  gather_rhs(d, f, m, k, nb1, gidx, rhsQ, cupd, mc, kc, ea_map, b);
-  const int* pr = perm + (long)f * k;
-  VT* t = tmp + (long)f * m;
-  for (int j = threadIdx.x; j < k; j += blockDim.x) t[j] = b[pr[j]];
-  for (int j = k + threadIdx.x; j < m; j += blockDim.x) t[j] = b[j];
-}
-
-// The same for fronts whose right-hand side does not fit in shared memory: the
-// front's work vector tmp is assembled in place in global memory, the eliminated
-// part permuted through the forward-result buffer y (free at this point).
-template <class VT>
-__global__ void __launch_bounds__(1024) inv_gather_global_kernel(
-    int d, int m, int k, int nb1, const int* __restrict__ gidx, const int* __restrict__ perm,
-    const VT* __restrict__ rhsQ, const VT* __restrict__ cupd, int mc, int kc,
-    const int* __restrict__ ea_map, VT* tmp, VT* ybuf, long N, long custr) {
-  pdl_wait();
-  const int f = blockIdx.x;
-  rhsQ += blockIdx.y * N;
-  if (cupd) cupd += blockIdx.y * custr;
-  tmp += (long)blockIdx.y * gridDim.x * m;
-  ybuf += (long)blockIdx.y * gridDim.x * k;
-  VT* t = tmp + (long)f * m;
-  for (int v = threadIdx.x; v < m; v += blockDim.x)
-    t[v] = (v < k) ? rhsQ[gidx[(long)f * m + v]] : vzero<VT>();
-  __syncthreads();
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= m) return;
+  const int f = blockIdx.y;
+  const long vz = blockIdx.z;
+  const int v = j < k ? perm[(long)f * k + j] : j;
+  VT b = v < k ? rhsQ[vz * N + gidx[(long)f * m + v]] : vzero<VT>();
   if (cupd) {
-    const int nbd = mc - kc;
+    const long nbd = mc - kc;
+    const VT* cu = cupd + vz * custr;
     for (int dl = 0; dl < (1 << d); ++dl) {
+      const int i = ea_inv[(long)dl * m + v];
+      if (i < 0) continue;
       int ff = f, cid = 0, stride = 1;
       for (int a = 0; a < d; ++a) {
-        int bc = ff % nb1;
+        const int bc = ff % nb1;
         ff /= nb1;
         cid += (2 * bc + ((dl >> a) & 1)) * stride;
         stride *= 2 * nb1;
       }
       cid += ff * stride;  // problem ff of a group
-      const VT* cu = cupd + (long)cid * nbd;
-      const int* mp = ea_map + (long)dl * nbd;
-      for (int i = threadIdx.x; i < nbd; i += blockDim.x) {
-        VT v = cu[i];
-        VT& tt = t[mp[i]];
-        tt.x += v.x;
-        tt.y += v.y;
-      }
-      __syncthreads();
+      const VT c = cu[cid * nbd + i];
+      b.x += c.x;
+      b.y += c.y;
     }
   }
-  const int* pr = perm + (long)f * k;
-  VT* y = ybuf + (long)f * k;
-  for (int j = threadIdx.x; j < k; j += blockDim.x) y[j] = t[pr[j]];
-  __syncthreads();
-  for (int j = threadIdx.x; j < k; j += blockDim.x) t[j] = y[j];
+  tmp[(vz * gridDim.y + f) * m + j] = b;
 }
 
 // Diagonal-block products of the levels whose diagonal blocks (size L.ib) hold
@@ -771,7 +743,6 @@ template <class VT, class T>
 void set_attrs() {
   cudaFuncSetAttribute(forward_kernel<VT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   cudaFuncSetAttribute(backward_kernel<VT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  cudaFuncSetAttribute(inv_gather_kernel<VT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   cudaFuncSetAttribute(inv_gemv_kernel<VT, T, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   cudaFuncSetAttribute(inv_gemv_kernel<VT, T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   cudaFuncSetAttribute(inv_gemv_kernel<VT, __half, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
@@ -889,16 +860,10 @@ cudaError_t forward_t(int d, DevLevel& L, const DevLevel* child, const void* rhs
         d, (const T*)L.front, L.m, L.k, L.nb1, L.gidx, L.perm, (const VT*)rhsQ, cup, L.mc, L.kc,
         L.ea_map, (VT*)L.upd, (VT*)L.y, N, custr);
   } else {
-    dim3 g(L.nf, nv);
-    if (sizeof(VT) * (size_t)L.m <= kVecSmem)
-      launch_k(L.pdl != 0, inv_gather_kernel<VT>, dim3(g), dim3(256), sizeof(VT) * L.m, st, 
-          d, L.m, L.k, L.nb1, L.gidx, L.perm, (const VT*)rhsQ, cup, L.mc, L.kc, L.ea_map,
-          (VT*)L.tmp, N, custr);
-    else
-      launch_k(L.pdl != 0, inv_gather_global_kernel<VT>, dim3(g), dim3(1024), 0, st, d, L.m, L.k, L.nb1, L.gidx, L.perm,
-                                                        (const VT*)rhsQ, cup, L.mc, L.kc,
-                                                        L.ea_map, (VT*)L.tmp, (VT*)L.y, N,
-                                                        custr);
+    const int tb = std::min(256, (L.m + 31) / 32 * 32);
+    dim3 g((unsigned)((L.m + tb - 1) / tb), L.nf, nv);
+    launch_k(L.pdl != 0, inv_gather_kernel<VT>, dim3(g), dim3(tb), 0, st, d, L.m, L.k, L.nb1, L.gidx,
+             L.perm, (const VT*)rhsQ, cup, L.mc, L.kc, L.ea_inv, (VT*)L.tmp, N, custr);
     launches = 1;
     // right-looking: after the diagonal block [j0, j1) of y, the rows below take
     // that column block's contribution; the last block's rows are those of L21,
