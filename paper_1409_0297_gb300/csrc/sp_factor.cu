@@ -1225,22 +1225,28 @@ __global__ void __launch_bounds__(256) lu_laswp_kernel(T* fronts, int m, int k, 
 }
 
 // Batched C[M x N] -= A[M x K] B[K x N], K <= kNB, column-major with leading
-// dimensions lda/ldb/ldc and per-batch strides (blockIdx.y = batch).  TILE x TILE
+// dimensions lda/ldb/ldc and per-batch strides (blockIdx.y = batch); FP32.  TILE x TILE
 // per CTA (TILE = 64: 4 x 4 per thread, TILE = 32: 2 x 2 per thread; the launcher
 // picks the one that wastes less work on the padding of the last tile row and
-// column).  Used for the Schur update of the LU.
+// column): rows tx + 16 a, columns ty + 16 b, so a warp's C accesses stay contiguous.  The
+// staged rows of A hold a thread's values side by side and those of B four steps of depth,
+// so vector loads feed it (two per sixteen FMAs; as scalars, eight).  Bound by C traffic and
+// the latency of one depth-32 pass per launch.  3D 64^3, root launches of the 32-wide tile:
+// 10.2 -> 6.3 us, of the 64-wide 11.2 -> 8.2 us; 8 x 4 per thread (128 x 64) was slower on the
+// leaves (two CTAs per SM).  Every entry adds its products in the order of l.
 template <class T, int TILE>
 __global__ void __launch_bounds__(256) gemm_sub_kernel(int M, int N, int K, const T* A, int lda,
                                                        long sA, const T* B, int ldb, long sB,
                                                        T* C, int ldc, long sC, int tilesM) {
   constexpr int R = TILE / 16;
+  constexpr int pB = kNB + 4;  // B rows: 16-byte steps, spread over the banks
   A += blockIdx.y * sA;
   B += blockIdx.y * sB;
   C += blockIdx.y * sC;
   const int tr = blockIdx.x % tilesM, tc = blockIdx.x / tilesM;
   const int r0 = tr * TILE, c0 = tc * TILE;
-  __shared__ T As[kNB][TILE];
-  __shared__ T Bs[kNB][TILE + 1];
+  __shared__ __align__(16) T As[kNB][TILE];   // [l][(i % 16) R + i / 16]
+  __shared__ __align__(16) T Bs[TILE][pB];    // [c][l]
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
   // this thread's C entries are loaded first, so their latency overlaps the staging of
   // A and B and the products (the update is bound by C traffic)
@@ -1254,32 +1260,43 @@ __global__ void __launch_bounds__(256) gemm_sub_kernel(int M, int N, int K, cons
       cpre[a][b] = (r < M && c < N) ? C[r + (long)c * ldc] : (T)0;
     }
   }
-  for (int e = threadIdx.x; e < K * TILE; e += blockDim.x) {
-    int i = e % TILE, l = e / TILE;
-    int r = r0 + i;
-    As[l][i] = (r < M) ? A[r + (long)l * lda] : (T)0;
+  // the depth is padded to a multiple of four with zeros
+  const int K4 = (K + 3) & ~3;
+  for (int e = threadIdx.x; e < K4 * TILE; e += 256) {
+    const int sl = e % TILE, l = e / TILE;
+    const int r = r0 + (sl % R) * 16 + sl / R;
+    As[l][sl] = (r < M && l < K) ? A[r + (long)l * lda] : (T)0;
   }
-  for (int e = threadIdx.x; e < K * TILE; e += blockDim.x) {
-    int l = e % K, jc = e / K;
-    int c = c0 + jc;
-    Bs[l][jc] = (c < N) ? B[l + (long)c * ldb] : (T)0;
+  for (int e = threadIdx.x; e < kNB * TILE; e += 256) {
+    const int l = e % kNB, jc = e / kNB;
+    const int c = c0 + jc;
+    Bs[jc][l] = (c < N && l < K) ? B[l + (long)c * ldb] : (T)0;
   }
   __syncthreads();
+  struct alignas(R * sizeof(T)) VecA {
+    T v[R];
+  };
+  struct alignas(4 * sizeof(T)) VecB {
+    T v[4];
+  };
   T acc[R][R];
 #pragma unroll
   for (int a = 0; a < R; ++a)
 #pragma unroll
     for (int b = 0; b < R; ++b) acc[a][b] = 0;
-  for (int l = 0; l < K; ++l) {
-    T av[R], bv[R];
+#pragma unroll 2
+  for (int l = 0; l < K4; l += 4) {
+    VecB bv[R];
 #pragma unroll
-    for (int a = 0; a < R; ++a) av[a] = As[l][tx + 16 * a];
+    for (int b = 0; b < R; ++b) bv[b] = *reinterpret_cast<const VecB*>(&Bs[ty + 16 * b][l]);
 #pragma unroll
-    for (int b = 0; b < R; ++b) bv[b] = Bs[l][ty + 16 * b];
+    for (int u = 0; u < 4; ++u) {
+      const VecA av = *reinterpret_cast<const VecA*>(&As[l + u][tx * R]);
 #pragma unroll
-    for (int a = 0; a < R; ++a)
+      for (int a = 0; a < R; ++a)
 #pragma unroll
-      for (int b = 0; b < R; ++b) acc[a][b] += av[a] * bv[b];
+        for (int b = 0; b < R; ++b) acc[a][b] += av.v[a] * bv[b].v[u];
+    }
   }
 #pragma unroll
   for (int b = 0; b < R; ++b) {
@@ -1769,10 +1786,8 @@ void gemm_sub(int M, int N, int K, const T* A, int lda, long sA, const T* B, int
     const int t = tile == 32 || (tile == 0 && w64 > 1.1 * w32) ? 32 : 64;
     const int tilesM = (M + t - 1) / t, tilesN = (N + t - 1) / t;
     dim3 g(tilesM * tilesN, batch);
-    if (t == 32)
-      gemm_sub_kernel<T, 32><<<g, 256, 0, st>>>(M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, tilesM);
-    else
-      gemm_sub_kernel<T, 64><<<g, 256, 0, st>>>(M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, tilesM);
+    auto kern = t == 32 ? gemm_sub_kernel<T, 32> : gemm_sub_kernel<T, 64>;
+    kern<<<g, 256, 0, st>>>(M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, tilesM);
   }
 }
 
