@@ -1604,8 +1604,9 @@ __device__ __forceinline__ double add_digits(double acc, const float* S, int es,
 // ONE: K <= 32 (one chunk; C read while the products run).  Arguments as gemm_gen_kernel,
 // alpha = -1 (neg = the sign bit) or 1.
 template <bool ONE>
-__global__ void __launch_bounds__(256, ONE ? 2 : 1)
-    gemm_f64_kernel(GemmSide<double> g0, GemmSide<double> g1, unsigned neg, int beta_one, int nb2) {
+__global__ void __launch_bounds__(256, ONE ? 2 : 1) gemm_f64_kernel(GemmSide<double> g0,
+                                                                  GemmSide<double> g1, unsigned neg,
+                                                                  int beta_one, int nb2) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __half* Ad = reinterpret_cast<__half*>(smraw);
   __half* Bd = Ad + kDig * kDigPlane;

@@ -55,9 +55,10 @@ struct PassArgs {
   const T* Dn;     // MID
   const VT* addx;  // POST_ADD
   const VT* tw;         // w_n^t = exp(-2 pi i t / n), t < n / 2
-  long S;               // stride between consecutive elements of a line
-  long nlines;          // number of lines of this axis, all vectors
-  long vlines, vstride; // lines per vector, entries per vector (vectors stacked)
+  unsigned S;           // stride between consecutive elements of a line
+  unsigned nlines;      // number of lines of this axis, all vectors
+  unsigned vlines;      // lines per vector
+  long vstride;         // entries per vector (vectors stacked)
   int n, W, U;          // U threads per line
   int ld;               // entries between two lines in shared memory
   int steps;
@@ -135,15 +136,28 @@ constexpr int kVal = 6;
 template <int r>
 constexpr int kPer = r == 4 ? 1 : 2;
 
+// The product l of the radices before a step: a power of two (sh its logarithm) except
+// behind a radix 3 (sh < 0), so that the remainders of a step are masks, not divisions (a
+// small grid's pass is one chain of latencies).
+struct Radix {
+  int l = 1, sh = 0;
+  __device__ __forceinline__ void grow(int r) {
+    l *= r;
+    sh = (sh < 0 || r == 3) ? -1 : sh + (r >> 1);  // r = 2: 1, r = 4: 2
+  }
+  __device__ __forceinline__ int mod(int b) const { return sh >= 0 ? b & (l - 1) : b % l; }
+  __device__ __forceinline__ int quot(int b) const { return sh >= 0 ? b >> sh : b / l; }
+};
+
 // The twiddles of a step of radix r at l, w_{l r}^{(b mod l) k} for k = 1 .. r - 1 of each
 // butterfly, loaded ahead of the exchange that the step waits for.
 template <int r, bool INV, class VT>
-__device__ __forceinline__ void load_tw(const PassArgs<VT>& a, int bb, int l, VT* tw) {
+__device__ __forceinline__ void load_tw(const PassArgs<VT>& a, int bb, const Radix& l, VT* tw) {
   const int nb = a.n / r;
 #pragma unroll
   for (int j = 0; j < kPer<r>; ++j) {
     const int b = bb + j * a.U;
-    const int t = b < nb ? (b % l) * (nb / l) : 0;  // w_{l r}^1 = w_n^(n / (l r))
+    const int t = b < nb ? l.mod(b) * l.quot(nb) : 0;  // w_{l r}^1 = w_n^(n / (l r))
 #pragma unroll
     for (int k = 1; k < r; ++k) tw[j * (r - 1) + k - 1] = tw_at<INV>(a, t * k);
   }
@@ -170,15 +184,16 @@ __device__ __forceinline__ void step_reg(const PassArgs<VT>& a, const VT* line, 
   }
 }
 template <int r, class VT>
-__device__ __forceinline__ void put_line(const PassArgs<VT>& a, VT* line, int bb, int l, const VT* v) {
+__device__ __forceinline__ void put_line(const PassArgs<VT>& a, VT* line, int bb, const Radix& l,
+                                         const VT* v) {
   const int nb = a.n / r;
 #pragma unroll
   for (int j = 0; j < kPer<r>; ++j) {
     const int b = bb + j * a.U;
     if (b >= nb) continue;
-    const int m = b % l, o = (b - m) * r + m;
+    const int m = l.mod(b), o = (b - m) * r + m;
 #pragma unroll
-    for (int k = 0; k < r; ++k) line[spos(o + k * l)] = v[j * r + k];
+    for (int k = 0; k < r; ++k) line[spos(o + k * l.l)] = v[j * r + k];
   }
 }
 
@@ -188,7 +203,7 @@ __device__ __forceinline__ void put_line(const PassArgs<VT>& a, VT* line, int bb
 template <bool INV, class VT>
 __device__ __forceinline__ void transform(const PassArgs<VT>& a, VT* line, int bb, bool live, VT* v) {
   VT tw[4];  // kPer (r - 1) twiddles of the next step
-  int l = 1;
+  Radix l;
   for (int s = 0; s < a.steps; ++s) {
     const int r = a.rad[INV ? a.steps - 1 - s : s];
     const bool first = s == 0, last = s == a.steps - 1;
@@ -198,7 +213,9 @@ __device__ __forceinline__ void transform(const PassArgs<VT>& a, VT* line, int b
       else step_reg<3, INV>(a, line, bb, first, tw, v);
     }
     if (!last) {
-      const int nx = a.rad[INV ? a.steps - 2 - s : s + 1], ln = l * r;
+      const int nx = a.rad[INV ? a.steps - 2 - s : s + 1];
+      Radix ln = l;
+      ln.grow(r);
       if (live) {
         if (nx == 4) load_tw<4, INV>(a, bb, ln, tw);
         else if (nx == 2) load_tw<2, INV>(a, bb, ln, tw);
@@ -212,7 +229,7 @@ __device__ __forceinline__ void transform(const PassArgs<VT>& a, VT* line, int b
       }
       __syncthreads();
     }
-    l *= r;
+    l.grow(r);
   }
 }
 
@@ -244,13 +261,14 @@ __global__ void __launch_bounds__(1024) fft_pass_kernel(PassArgs<VT> a) {
   // lines side by side along axis 0, element-interleaved along the others (coalesced)
   const int tid = threadIdx.x;
   const int w = axis0 ? tid / a.U : tid % a.W, bb = axis0 ? tid - w * a.U : tid / a.W;
-  const long t = (long)blockIdx.x * a.W + w;
+  const unsigned t = blockIdx.x * (unsigned)a.W + (unsigned)w;
   const bool live = w < a.W && bb < a.U && t < a.nlines;
   VT* line = reinterpret_cast<VT*>(smraw) + (long)w * a.ld;
-  const long vec = t / a.vlines, tl = t - vec * a.vlines;
-  const long hi = tl / a.S, base = (tl - hi * a.S) + hi * a.S * a.n;  // within the vector
+  const unsigned vec = a.nlines == a.vlines ? 0u : t / a.vlines, tl = t - vec * a.vlines;
+  const unsigned hi = axis0 ? tl : tl / a.S;
+  const long base = (long)(tl - hi * a.S) + (long)hi * a.S * a.n;  // within the vector
   const long voff = vec * a.vstride;
-  const long qoff = (a.qper > 1 ? vec % a.qper * a.vstride : 0) + base;
+  const long qoff = (a.qper > 1 ? vec % (unsigned)a.qper * a.vstride : 0) + base;
   const VT* in = a.in + voff + base;
   VT v[kVal];
   const int rf = a.mode == 1 ? a.rad[a.steps - 1] : a.rad[0];                 // radix read first
@@ -306,12 +324,13 @@ cudaError_t run_pass(int d, int n, const VT* tw, const typename Real<VT>::T* Dn,
   }
   long S = 1;
   for (int i = 0; i < axis; ++i) S *= n;
-  a.S = S;
+  a.S = (unsigned)S;
   long N = 1;
   for (int i = 0; i < d; ++i) N *= n;
-  a.vlines = N / n;
+  if (N / n * nvec > 0x7fffffffL) return cudaErrorInvalidValue;  // beyond every context's size
+  a.vlines = (unsigned)(N / n);
   a.vstride = N;
-  a.nlines = a.vlines * nvec;
+  a.nlines = a.vlines * (unsigned)nvec;
   a.U = (n + 3) / 4;
   if (a.U > 1024) return cudaErrorInvalidValue;
   // lines per CTA: eight (whole 128-byte lines across an axis > 0) while there are six CTAs
@@ -319,7 +338,7 @@ cudaError_t run_pass(int d, int n, const VT* tw, const typename Real<VT>::T* Dn,
   int least = axis > 0 ? 2 : 1;
   while (least * a.U < 32) least *= 2;
   a.W = std::max(8, least);
-  while (a.W > least && a.nlines / a.W < 912) a.W /= 2;
+  while (a.W > least && (int)a.nlines / a.W < 912) a.W /= 2;
   while (a.W > 1 && (a.W * a.U > 1024 || (axis > 0 && S % a.W))) a.W /= 2;
   a.ld = (n + n / 8 + 1) | 1;
   const size_t smem = (size_t)a.W * a.ld * sizeof(VT);
