@@ -918,11 +918,11 @@ def measure_learned(args, B, torch, dist, world):
 # text at the time (from the line that names the kernel to the first line that is a
 # lone closing brace): a changed kernel reports null until it is captured again.
 TRAFFIC = {
-    # FP64 Schur update (gemm_sub_kernel<double, 32>), all 101 launches of one 2D 512^2
-    # Helmholtz factorisation: 6.42 GB / 101 launches (ncu --metrics
+    # FP64 Schur update (gemm_f64_kernel<true>), all 101 launches of one 2D 512^2
+    # Helmholtz factorisation: 6.46 GB / 101 launches (ncu --metrics
     # dram__bytes_read.sum,dram__bytes_write.sum; command in the matching profile summary)
-    "lu_gemm": {"bytes_per_launch": 63.6e6, "source": "paper_1409_0297_gb300/csrc/sp_factor.cu",
-                "kernel": "gemm_sub_kernel(", "sha16": "6282b6619bef34c3"},
+    "lu_gemm": {"bytes_per_launch": 63.9e6, "source": "paper_1409_0297_gb300/csrc/sp_factor.cu",
+                "kernel": "gemm_f64_kernel(", "sha16": "29b43f0cee0d334b"},
 }
 
 
@@ -1212,9 +1212,19 @@ def run_ours(args):
     hbm = peaks.get("hbm_gbs", 6800.0)
     fp64_peak_tflops = 1.25  # nominal GB300 FP64 rate (no FP64 entry in the measured peaks)
     alu_classes = {"lu_panel", "lu_trsm", "lu_gemm", "lu_trinv"}
+    # FP64 products by exact digit products on the tensor cores: three FP64 instructions per
+    # output and 32-deep chunk where an FMA loop takes 32
+    digit_classes = {"lu_gemm", "lu_trinv"}
 
     def roof(k, vals):
         ms_, nl, wk = vals
+        if k in digit_classes:
+            ach = wk / (ms_ / 1e3) / 1e12
+            peak = fp64_peak_tflops * 32 / 3
+            return {"kernel": k, "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+                    "frac": ach / peak, "traffic": recorded_traffic(k),
+                    "peak_source": "nominal FP64 1.25 TFLOP/s x 32 / 3 (digit products: three FP64 "
+                                   "instructions per output and 32-deep chunk)"}
         if k in alu_classes:
             ach = wk / (ms_ / 1e3) / 1e12
             return {"kernel": k, "bound": "alu", "achieved": ach, "peak": fp64_peak_tflops,
