@@ -48,7 +48,7 @@ typedef enum {
   SP_ERR_NOCONV = 4,    /* GMRES stopped at maxit above tol (the iterate is still returned) */
   SP_ERR_OOM = 5,       /* device or host allocation failed, or the host could not start
                            the set-up's worker threads */
-  SP_ERR_TIMEOUT = 6,   /* a bounded device wait (tensor-core pipeline, grid panel) ran out */
+  SP_ERR_TIMEOUT = 6,   /* a bounded device wait (tensor-core pipeline, panel) ran out */
   SP_ERR_CUDA = 7,      /* a CUDA runtime call failed */
   SP_ERR_STATE = 8      /* call out of order (e.g. sp_apply before sp_factor) */
 } sp_status;
@@ -119,9 +119,9 @@ typedef struct {
                         (four operand stages); 4: as 0 in thread-block clusters of two
                         CTAs that share each B tile by TMA multicast (slower: 557 against
                         637 TFLOP/s at 3D 128^3).  All give the same bits. */
-  long long wait_limit_ns; /* limit of each bounded wait of the cooperative grid panel
-                        (the LU panel of fronts too tall for a thread-block cluster:
-                        every CTA polls the pivot candidates its peers publish) in
+  long long wait_limit_ns; /* limit of each bounded wait of the cluster and grid panels
+                        (the LU panel of fronts split over several CTAs, which wait for
+                        the pivot candidates that their peers push or publish) in
                         nanoseconds of the GPU's global timer; 0 (default) = 2e9 (2 s),
                         else 1 ... 6e10.  When a wait runs out the panel stops and
                         sp_factor returns SP_ERR_TIMEOUT; destroy that context. */
@@ -132,13 +132,15 @@ typedef struct {
                         work vectors in shared memory; on levels with few fronts a
                         thread-block cluster of up to 16 CTAs per front walks the diagonal
                         blocks itself).  0 (default): fused only on levels whose fronts
-                        fill the GPU without clusters, chains elsewhere; 1: chains
+                        fill the GPU without clusters and have 128 rows or more,
+                        chains elsewhere; 1: chains
                         everywhere; 2: fused wherever the vectors fit.  All are exact
                         applications of the same factor; they round differently. */
-  int panel_pivoting; /* pivoting of the cooperative grid panel in the FP32 forms (fronts too
-                        tall for a thread-block cluster, the 3D upper levels): 0 (default)
-                        partial pivoting column by column (two publication rounds per
-                        column); 1 tournament pivoting (communication-avoiding LU: each CTA
+  int panel_pivoting; /* pivoting of the tallest panels in the FP32 forms (fronts of more than
+                        ~6800 rows, the 3D upper levels): 0 (default)
+                        partial pivoting column by column (in registers of a thread-block
+                        cluster up to 24576 rows, beyond by a cooperative grid with two
+                        publication rounds per column); 1 tournament pivoting (communication-avoiding LU: each CTA
                         picks 32 candidate rows by partial pivoting on its rows, groups of
                         16 CTAs and then all CTAs play the winners off, and every row is
                         eliminated against the 32 chosen ones at once: three publication
