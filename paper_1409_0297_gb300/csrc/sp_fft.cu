@@ -131,10 +131,12 @@ __device__ __forceinline__ VT tw_at(const PassArgs<VT>& a, int t) {
   return v;
 }
 
-// values a thread holds: one butterfly of radix 4, two of radix 2, two of radix 3
-constexpr int kVal = 6;
-template <int r>
-constexpr int kPer = r == 4 ? 1 : 2;
+// values a thread holds: G butterflies of radix 4, 2 G of radix 2 or 3 (G = 2 for n >= 2048,
+// so that a line of 8192 points is one CTA)
+template <int G>
+constexpr int kVal = 6 * G;
+template <int r, int G>
+constexpr int kPer = (r == 4 ? 1 : 2) * G;
 
 // The product l of the radices before a step: a power of two (sh its logarithm) except
 // behind a radix 3 (sh < 0), so that the remainders of a step are masks, not divisions (a
@@ -150,12 +152,13 @@ struct Radix {
 };
 
 // The twiddles of a step of radix r at l, w_{l r}^{(b mod l) k} for k = 1 .. r - 1 of each
-// butterfly, loaded ahead of the exchange that the step waits for.
+// butterfly, loaded ahead of the exchange that the step waits for (G = 1; the threads of
+// longer lines have no registers left for them and load them in the step).
 template <int r, bool INV, class VT>
 __device__ __forceinline__ void load_tw(const PassArgs<VT>& a, int bb, const Radix& l, VT* tw) {
   const int nb = a.n / r;
 #pragma unroll
-  for (int j = 0; j < kPer<r>; ++j) {
+  for (int j = 0; j < kPer<r, 1>; ++j) {
     const int b = bb + j * a.U;
     const int t = b < nb ? l.mod(b) * l.quot(nb) : 0;  // w_{l r}^1 = w_n^(n / (l r))
 #pragma unroll
@@ -165,30 +168,32 @@ __device__ __forceinline__ void load_tw(const PassArgs<VT>& a, int bb, const Rad
 
 // One step of radix r at l for the butterflies b = bb + j U of a line: from the values in v
 // (first: already there, no twiddles) or from the line in shared memory, to registers.
-template <int r, bool INV, class VT>
+template <int r, bool INV, int G, class VT>
 __device__ __forceinline__ void step_reg(const PassArgs<VT>& a, const VT* line, int bb, bool first,
-                                         const VT* tw, VT* v) {
+                                         const Radix& l, const VT* tw, VT* v) {
   const int nb = a.n / r;
 #pragma unroll
-  for (int j = 0; j < kPer<r>; ++j) {
+  for (int j = 0; j < kPer<r, G>; ++j) {
     const int b = bb + j * a.U;
     if (b >= nb) continue;
     VT* x = v + j * r;
     if (!first) {
 #pragma unroll
       for (int k = 0; k < r; ++k) x[k] = line[spos(b + k * nb)];
+      const int t = G > 1 ? l.mod(b) * l.quot(nb) : 0;
 #pragma unroll
-      for (int k = 1; k < r; ++k) x[k] = cmul(x[k], tw[j * (r - 1) + k - 1]);
+      for (int k = 1; k < r; ++k)
+        x[k] = cmul(x[k], G > 1 ? tw_at<INV>(a, t * k) : tw[j * (r - 1) + k - 1]);
     }
     dft_reg<r, INV>(x);
   }
 }
-template <int r, class VT>
+template <int r, int G, class VT>
 __device__ __forceinline__ void put_line(const PassArgs<VT>& a, VT* line, int bb, const Radix& l,
                                          const VT* v) {
   const int nb = a.n / r;
 #pragma unroll
-  for (int j = 0; j < kPer<r>; ++j) {
+  for (int j = 0; j < kPer<r, G>; ++j) {
     const int b = bb + j * a.U;
     if (b >= nb) continue;
     const int m = l.mod(b), o = (b - m) * r + m;
@@ -200,32 +205,32 @@ __device__ __forceinline__ void put_line(const PassArgs<VT>& a, VT* line, int bb
 // The transform of one line: on entry the first step's inputs are in v, on return the last
 // step's outputs (element b + k n / r of butterfly b), radices rad[0 .. steps) or, INV, in
 // reverse.
-template <bool INV, class VT>
+template <bool INV, int G, class VT>
 __device__ __forceinline__ void transform(const PassArgs<VT>& a, VT* line, int bb, bool live, VT* v) {
-  VT tw[4];  // kPer (r - 1) twiddles of the next step
+  VT tw[4];  // G = 1: kPer (r - 1) twiddles of the next step
   Radix l;
   for (int s = 0; s < a.steps; ++s) {
     const int r = a.rad[INV ? a.steps - 1 - s : s];
     const bool first = s == 0, last = s == a.steps - 1;
     if (live) {
-      if (r == 4) step_reg<4, INV>(a, line, bb, first, tw, v);
-      else if (r == 2) step_reg<2, INV>(a, line, bb, first, tw, v);
-      else step_reg<3, INV>(a, line, bb, first, tw, v);
+      if (r == 4) step_reg<4, INV, G>(a, line, bb, first, l, tw, v);
+      else if (r == 2) step_reg<2, INV, G>(a, line, bb, first, l, tw, v);
+      else step_reg<3, INV, G>(a, line, bb, first, l, tw, v);
     }
     if (!last) {
       const int nx = a.rad[INV ? a.steps - 2 - s : s + 1];
       Radix ln = l;
       ln.grow(r);
-      if (live) {
+      if (G == 1 && live) {
         if (nx == 4) load_tw<4, INV>(a, bb, ln, tw);
         else if (nx == 2) load_tw<2, INV>(a, bb, ln, tw);
         else load_tw<3, INV>(a, bb, ln, tw);
       }
       __syncthreads();  // the line has been read
       if (live) {
-        if (r == 4) put_line<4>(a, line, bb, l, v);
-        else if (r == 2) put_line<2>(a, line, bb, l, v);
-        else put_line<3>(a, line, bb, l, v);
+        if (r == 4) put_line<4, G>(a, line, bb, l, v);
+        else if (r == 2) put_line<2, G>(a, line, bb, l, v);
+        else put_line<3, G>(a, line, bb, l, v);
       }
       __syncthreads();
     }
@@ -235,13 +240,13 @@ __device__ __forceinline__ void transform(const PassArgs<VT>& a, VT* line, int b
 
 // fn(value, element index) for the values of a step of radix r read or written at
 // b + k n / r
-template <class VT, class Fn>
+template <int G, class VT, class Fn>
 __device__ __forceinline__ void each_value(const PassArgs<VT>& a, int r, int bb, VT* v, Fn fn) {
   const int nb = a.n / r;
   auto go = [&](auto rr) {
     constexpr int R = decltype(rr)::value;
 #pragma unroll
-    for (int j = 0; j < kPer<R>; ++j) {
+    for (int j = 0; j < kPer<R, G>; ++j) {
       const int b = bb + j * a.U;
       if (b >= nb) continue;
 #pragma unroll
@@ -253,7 +258,7 @@ __device__ __forceinline__ void each_value(const PassArgs<VT>& a, int r, int bb,
   else go(std::integral_constant<int, 3>{});
 }
 
-template <class VT>
+template <class VT, int G>
 __global__ void __launch_bounds__(1024) fft_pass_kernel(PassArgs<VT> a) {
   using T = typename Real<VT>::T;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -270,35 +275,35 @@ __global__ void __launch_bounds__(1024) fft_pass_kernel(PassArgs<VT> a) {
   const long voff = vec * a.vstride;
   const long qoff = (a.qper > 1 ? vec % (unsigned)a.qper * a.vstride : 0) + base;
   const VT* in = a.in + voff + base;
-  VT v[kVal];
+  VT v[kVal<G>];
   const int rf = a.mode == 1 ? a.rad[a.steps - 1] : a.rad[0];                 // radix read first
   const int rl = a.mode == 0 ? a.rad[a.steps - 1] : a.rad[0];                 // radix written last
   if (live) {
-    each_value(a, rf, bb, v, [&](VT& x, int i) { x = in[(long)i * a.S]; });
+    each_value<G>(a, rf, bb, v, [&](VT& x, int i) { x = in[(long)i * a.S]; });
     if (a.q)
-      each_value(a, rf, bb, v, [&](VT& x, int i) {
+      each_value<G>(a, rf, bb, v, [&](VT& x, int i) {
         const T qq = a.q[qoff + (long)i * a.S];
         x.x *= qq;
         x.y *= qq;
       });
   }
-  if (a.mode != 1) transform<false>(a, line, bb, live, v);
+  if (a.mode != 1) transform<false, G>(a, line, bb, live, v);
   if (a.mode == 2) {
     if (live)
-      each_value(a, a.rad[a.steps - 1], bb, v, [&](VT& x, int i) {
+      each_value<G>(a, a.rad[a.steps - 1], bb, v, [&](VT& x, int i) {
         const T dn = a.Dn[qoff + (long)i * a.S];
         x.x *= dn;
         x.y *= dn;
       });
   }
-  if (a.mode != 0) transform<true>(a, line, bb, live, v);
+  if (a.mode != 0) transform<true, G>(a, line, bb, live, v);
   if (live) {
     VT* out = a.out + voff + base;
     if (a.addx) {
       const VT* add = a.addx + voff + base;
-      each_value(a, rl, bb, v, [&](VT& x, int i) { x = cadd(x, add[(long)i * a.S]); });
+      each_value<G>(a, rl, bb, v, [&](VT& x, int i) { x = cadd(x, add[(long)i * a.S]); });
     }
-    each_value(a, rl, bb, v, [&](VT& x, int i) { out[(long)i * a.S] = x; });
+    each_value<G>(a, rl, bb, v, [&](VT& x, int i) { out[(long)i * a.S] = x; });
   }
 }
 
@@ -331,26 +336,32 @@ cudaError_t run_pass(int d, int n, const VT* tw, const typename Real<VT>::T* Dn,
   a.vlines = (unsigned)(N / n);
   a.vstride = N;
   a.nlines = a.vlines * (unsigned)nvec;
-  a.U = (n + 3) / 4;
+  const int G = n >= 2048 ? 2 : 1;
+  a.U = (n + 4 * G - 1) / (4 * G);
   if (a.U > 1024) return cudaErrorInvalidValue;
   // lines per CTA: eight (whole 128-byte lines across an axis > 0) while there are six CTAs
-  // per SM, down to two (whole sectors) and to a full warp
-  int least = axis > 0 ? 2 : 1;
+  // per SM, down to two (whole sectors) and to a full warp; one from 1024 points on, where pairs leave
+  // too few CTAs to even out (an application at 1024^2: 364 us in pairs, 343 alone)
+  int least = axis > 0 && a.U < 256 ? 2 : 1;
   while (least * a.U < 32) least *= 2;
   a.W = std::max(8, least);
   while (a.W > least && (int)a.nlines / a.W < 912) a.W /= 2;
-  while (a.W > 1 && (a.W * a.U > 1024 || (axis > 0 && S % a.W))) a.W /= 2;
   a.ld = (n + n / 8 + 1) | 1;
+  while (a.W > 1 && (a.W * a.U > 1024 || (long)a.W * a.ld * sizeof(VT) > 128 * 1024 ||
+                     (axis > 0 && S % a.W)))
+    a.W /= 2;
   const size_t smem = (size_t)a.W * a.ld * sizeof(VT);
   const unsigned grid = (unsigned)((a.nlines + a.W - 1) / a.W);
   static bool attr_set = false;
   if (!attr_set) {
-    cudaFuncSetAttribute(fft_pass_kernel<VT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(fft_pass_kernel<VT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(fft_pass_kernel<VT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr_set = true;
   }
   const double es = sizeof(VT);
   ProfScope ps(PROF_FFT, st);
-  fft_pass_kernel<VT><<<grid, (unsigned)((a.W * a.U + 31) / 32 * 32), smem, st>>>(a);
+  auto kern = G == 2 ? fft_pass_kernel<VT, 2> : fft_pass_kernel<VT, 1>;
+  kern<<<grid, (unsigned)((a.W * a.U + 31) / 32 * 32), smem, st>>>(a);
   ps.done((double)N * nvec * (2 * es + (q ? es / 2 : 0.0) + (mode == 2 ? es / 2 : 0.0) +
                              (addx ? es : 0.0)),
           1, st);
