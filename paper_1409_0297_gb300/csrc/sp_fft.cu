@@ -131,8 +131,9 @@ __device__ __forceinline__ VT tw_at(const PassArgs<VT>& a, int t) {
   return v;
 }
 
-// values a thread holds: G butterflies of radix 4, 2 G of radix 2 or 3 (G = 2 for n >= 2048,
-// so that a line of 8192 points is one CTA)
+// values a thread holds: G butterflies of radix 4, 2 G of radix 2 or 3 (G = 2 for n >= 1536,
+// so that a line of 8192 points is one CTA and more than two CTAs of a shorter one share an
+// SM: an application at 1536^2 takes 880 us, with G = 1 904)
 template <int G>
 constexpr int kVal = 6 * G;
 template <int r, int G>
@@ -336,15 +337,16 @@ cudaError_t run_pass(int d, int n, const VT* tw, const typename Real<VT>::T* Dn,
   a.vlines = (unsigned)(N / n);
   a.vstride = N;
   a.nlines = a.vlines * (unsigned)nvec;
-  const int G = n >= 2048 ? 2 : 1;
+  const int G = n >= 1536 ? 2 : 1;
   a.U = (n + 4 * G - 1) / (4 * G);
   if (a.U > 1024) return cudaErrorInvalidValue;
   // lines per CTA: eight (whole 128-byte lines across an axis > 0) while there are six CTAs
-  // per SM, down to two (whole sectors) and to a full warp; one from 1024 points on, where pairs leave
-  // too few CTAs to even out (an application at 1024^2: 364 us in pairs, 343 alone)
-  int least = axis > 0 && a.U < 256 ? 2 : 1;
+  // per SM, down to two (whole sectors) and to a full warp; one from 1024 points on, where
+  // pairs leave too few CTAs to even out (an application at 1024^2: 364 us in pairs, 341
+  // alone; at 2048^2: 1526 and 1513)
+  int least = axis > 0 && n < 1024 ? 2 : 1;
   while (least * a.U < 32) least *= 2;
-  a.W = std::max(8, least);
+  a.W = n < 1024 ? std::max(8, least) : 1;
   while (a.W > least && (int)a.nlines / a.W < 912) a.W /= 2;
   a.ld = (n + n / 8 + 1) | 1;
   while (a.W > 1 && (a.W * a.U > 1024 || (long)a.W * a.ld * sizeof(VT) > 128 * 1024 ||

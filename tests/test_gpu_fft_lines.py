@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("d,n,b", [(2, 8, 2), (2, 12, 3), (2, 24, 3), (2, 48, 6), (2, 96, 6),
-                                   (2, 2048, 32), (3, 8, 2), (3, 12, 3), (3, 24, 3)])
+                                   (2, 1536, 12), (2, 2048, 32), (3, 8, 2), (3, 12, 3), (3, 24, 3)])
 def test_operator_against_numpy(d, n, b):
     import torch
 
