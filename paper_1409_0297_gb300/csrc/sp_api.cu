@@ -1672,6 +1672,23 @@ sp_status sp_schur_update(sp_precision prec, int M, int N, int K, const void* A,
   return SP_ERR_OOM;
 }
 
+// Not in the public header: the tests of the panel and inverse kernels call it.
+// status: bit 1 a pivot below the threshold, bit 2 a wait that ran out.
+sp_status sp_test_front_lu(sp_precision prec, int m, int k, int nf, int grid_panel, double pivot_tol,
+                           long long wait_ns, void* fronts, int* piv, int* perm, int* status_host) {
+  if ((prec != SP_PREC_FP64 && prec != SP_PREC_FP32) || k < 1 || m < k || m > 8192 || nf < 1 ||
+      nf > 4096 || wait_ns < 1 || !fronts || !piv || !perm || !status_host)
+    return SP_ERR_ARG;
+  int* ds = nullptr;
+  cudaError_t e = cudaMalloc(&ds, sizeof(int));
+  if (e == cudaSuccess)
+    e = front_lu_raw(prec, m, k, nf, grid_panel, pivot_tol, (unsigned long long)wait_ns, fronts, piv, perm,
+                     ds, nullptr);
+  if (e == cudaSuccess) e = cudaMemcpy(status_host, ds, sizeof(int), cudaMemcpyDeviceToHost);
+  cudaFree(ds);
+  return cuda_status(e);
+}
+
 sp_status sp_tc_probe(int split, int M, int N, int K, int reps, void* stream, double* ms_per_launch) try {
   if ((split != 0 && split != 1) || !ms_per_launch || reps < 1 || reps > 1000) return SP_ERR_ARG;
   if (M < 128 || N < 256 || K < 32 || M % 128 || N % 256 || K % 32 || M > 16384 || N > 16384 ||

@@ -417,6 +417,12 @@ __global__ void __launch_bounds__(256) lu_panel_grid_kernel(T* fronts, int m, in
 // below k (interchanges only exchange positions below k, so: slot < k - j0) and it has
 // not been a pivot; the positions are replayed once at the end.
 //
+// The pivot is the largest magnitude of the column (FP64: all bits of it), ties to the
+// smallest position, as in the textbook loop over the rows in place.  A row is at its own
+// slot until an interchange moves it, and the only rows that an interchange moves without
+// making them pivots are those of the slots 0 .. 31, so the position is one register (of
+// row r = 0) that follows the interchanges.
+//
 // Pivot step.  Each warp reduces its candidates' magnitude bits and the owner of the
 // largest posts its row; one CTA barrier; every
 // warp picks the CTA's best.  With C > 1 each CTA then pushes its best row and key into
@@ -429,22 +435,33 @@ __global__ void __launch_bounds__(256) lu_panel_grid_kernel(T* fronts, int m, in
 // The 32 columns are taken in four blocks of eight: the eight steps are unrolled with
 // the current block in registers 0-7, the columns right of it updated in groups of
 // eight (finished groups skipped), then the registers rotate by eight; the code stays
-// at eight unrolled steps.  The pivot is a largest-magnitude entry of the column (FP64:
-// up to the 20 leading mantissa bits of the magnitude), ties to the first CTA, warp, lane
-// and row.
+// at eight unrolled steps.
 //
 // What bounds it: the chain of pivot steps (FP32) and the SM's two FP64 FMAs per cycle
 // (FP64), so FP32 panels take the fewest CTAs whose registers hold them and FP64 panels
 // as many as the level leaves free (panel_shape).
 constexpr int kPanelMaxC = 16;
 
+// magnitudes as integers of the same order; a NaN is never the largest
 __device__ __forceinline__ unsigned mag_bits(float v) {
   const unsigned u = __float_as_uint(v) & 0x7fffffffu;
-  return u > 0x7f800000u ? 0u : u;  // a NaN is never the largest
+  return u > 0x7f800000u ? 0u : u;
 }
 __device__ __forceinline__ unsigned mag_bits(double v) {
   const unsigned u = (unsigned)__double2hiint(v) & 0x7fffffffu;
   return u > 0x7ff00000u || (u == 0x7ff00000u && __double2loint(v) != 0) ? 0u : u;
+}
+// the lane with the largest key, ties to the smallest position (the whole warp calls it);
+// *key becomes that lane's key
+__device__ __forceinline__ int pick_lane(unsigned* key, unsigned pos) {
+  const unsigned mine = *key, best = __reduce_max_sync(0xffffffffu, mine);
+  unsigned in = __ballot_sync(0xffffffffu, mine == best);
+  if (in & (in - 1)) {
+    const unsigned p = __reduce_min_sync(0xffffffffu, mine == best ? pos : 0xffffffffu);
+    in = __ballot_sync(0xffffffffu, mine == best && pos == p);
+  }
+  *key = best;
+  return __ffs(in) - 1;
 }
 // 1 / v: FP64 from the hardware's approximate reciprocal (20 bits) and two Newton steps
 // r += r (1 - v r), which double the correct bits (20 -> 40 -> full); magnitudes whose
@@ -548,14 +565,12 @@ __global__ void __launch_bounds__(NT)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int s0 = q * NT * R + tid;  // slot of row r: s0 + r NT
   __shared__ __align__(16) T wrow[2][W][kNB];   // posted candidate row of each warp
-  __shared__ unsigned wmag[2][W];
-  __shared__ int wslot[2][W];
+  __shared__ unsigned wmag[2][W], wpos[2][W];
   __shared__ __align__(16) T crow[2][kPanelMaxC][kNB];  // pushed rows of the cluster's CTAs
   __shared__ __align__(8) unsigned long long ckey[2][kPanelMaxC];
   __shared__ __align__(8) unsigned long long cbar[2];
-  __shared__ int spiv[kNB];   // pivot slots in order
+  __shared__ int spiv[kNB];   // pivot positions in order
   __shared__ T spv[kNB];      // pivots
-  __shared__ int spos[kNB];   // final position of the slots 0 .. 31
   const double thresh = ptol * scale[f];
   if (C > 1) {
     if (tid == 0) {
@@ -576,6 +591,7 @@ __global__ void __launch_bounds__(NT)
   int pj[R];  // pivot step of the row, -1: not a pivot
 #pragma unroll
   for (int r = 0; r < R; ++r) pj[r] = -1;
+  int pos0 = s0;  // position of row r = 0; the other rows stay at their slots
   bool ok = true, stop = false;  // this warp's last wait; the CTA gave up
 #pragma unroll 1
   for (int o = 0; o < kNB / 8; ++o) {
@@ -585,32 +601,30 @@ __global__ void __launch_bounds__(NT)
       const int jj = 8 * o + u;
       if (jj < jb && !stop) {
         const int buf = u & 1;
-        // this thread's candidate: magnitude + 1 (0: none), smallest slot first
-        unsigned mg = 0;
-        int sl = 0x7fffffff;
+        // this thread's candidate: magnitude + 1 (0: none) and position
+        unsigned mg = 0, mpos = 0xffffffffu;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          const int s = s0 + r * NT;
-          if (pj[r] < 0 && s < kl) {
-            const unsigned v = mag_bits(a[r][u]) + 1u;
-            if (v > mg) {
+          if (pj[r] < 0 && s0 + r * NT < kl) {
+            const unsigned v = mag_bits(a[r][u]) + 1u, p = (unsigned)(r == 0 ? pos0 : s0 + r * NT);
+            if (v > mg || (v == mg && p < mpos)) {
               mg = v;
-              sl = s;
+              mpos = p;
             }
           }
         }
-        const unsigned wm = __reduce_max_sync(0xffffffffu, mg);
-        const int wl = __ffs(__ballot_sync(0xffffffffu, mg == wm)) - 1;  // first lane that holds it
+        unsigned wm = mg;
+        const int wl = pick_lane(&wm, mpos);
         if (lane == wl) {
 #pragma unroll
           for (int r = 0; r < R; ++r)
-            if (s0 + r * NT == sl) {
+            if (pj[r] < 0 && (unsigned)(r == 0 ? pos0 : s0 + r * NT) == mpos) {
 #pragma unroll
               for (int g = 0; g < kNB / 8; ++g)
                 if (g < live) store8(&wrow[buf][warp][8 * g], &a[r][8 * g]);
             }
           wmag[buf][warp] = wm;
-          wslot[buf][warp] = sl;
+          wpos[buf][warp] = mpos;
         }
         if (C > 1) {
           // a warp whose last wait gave up stops its whole CTA here
@@ -625,11 +639,10 @@ __global__ void __launch_bounds__(NT)
         unsigned best = wm;
         int wb = 0;
         if (W > 1) {
-          const unsigned bm = lane < W ? wmag[buf][lane] : 0u;
-          best = __reduce_max_sync(0xffffffffu, bm);
-          wb = __ffs(__ballot_sync(0xffffffffu, lane < W && bm == best)) - 1;
+          best = lane < W ? wmag[buf][lane] : 0u;
+          wb = pick_lane(&best, lane < W ? wpos[buf][lane] : 0xffffffffu);
         }
-        int bslot = wslot[buf][wb];
+        unsigned bpos = wpos[buf][wb];
         const T* prow = wrow[buf][wb];
         if (C > 1) {
           // push the row and its key to every CTA of the cluster (destinations spread
@@ -638,7 +651,7 @@ __global__ void __launch_bounds__(NT)
           const unsigned kdst = smem_addr(&ckey[buf][q]), bar = smem_addr(&cbar[buf]);
           const T rv = wrow[buf][wb][lane];
           const unsigned long long key =
-              best ? ((unsigned long long)best << 32) | (0xffffffffu - (unsigned)bslot) : 0ull;
+              ((unsigned long long)best << 32) | bpos;
           if (tid == 0)
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
                          "r"((unsigned)(C * (kNB * sizeof(T) + 8)))
@@ -650,17 +663,16 @@ __global__ void __launch_bounds__(NT)
           }
           ok = bar_wait(bar, (jj >> 1) & 1, wait_ns);
           ok = __all_sync(0xffffffffu, ok);
-          const unsigned long long kk = lane < C ? ckey[buf][lane] : 0ull;
-          const unsigned khi = (unsigned)(kk >> 32);
-          best = __reduce_max_sync(0xffffffffu, khi);
-          const int cb = __ffs(__ballot_sync(0xffffffffu, lane < C && khi == best)) - 1;
-          bslot = (int)(0xffffffffu - (unsigned)ckey[buf][cb]);
+          const unsigned long long kk = lane < C ? ckey[buf][lane] : 0xffffffffull;
+          best = (unsigned)(kk >> 32);
+          const int cb = pick_lane(&best, (unsigned)kk);
+          bpos = (unsigned)ckey[buf][cb];
           prow = crow[buf][cb];
         }
         if (ok) {
           T pv = prow[u];
           if (tid == 0) {
-            spiv[jj] = best ? bslot : -1;  // there is a candidate inside k columns, always
+            spiv[jj] = best ? (int)bpos : jj;  // there is a candidate inside k columns, always
             spv[jj] = best ? pv : (T)0;
           }
           if (!nonzero(pv)) pv = (T)(thresh > 0 ? thresh : 1e-30);
@@ -668,10 +680,11 @@ __global__ void __launch_bounds__(NT)
           T l[R];
 #pragma unroll
           for (int r = 0; r < R; ++r) {
-            if (s0 + r * NT == bslot) pj[r] = jj;
+            if (pj[r] < 0 && (unsigned)(r == 0 ? pos0 : s0 + r * NT) == bpos) pj[r] = jj;
             l[r] = pj[r] < 0 ? a[r][u] * inv : (T)0;
             if (pj[r] < 0) a[r][u] = l[r];
           }
+          if (pj[0] < 0 && pos0 == jj) pos0 = (int)bpos;  // the interchange moves the row at jj
 #pragma unroll
           for (int g = 0; g < kNB / 8; ++g)
             if (g < live) {
@@ -712,54 +725,47 @@ __global__ void __launch_bounds__(NT)
         mpf[kNB + c] = -1;
       }
   } else {
-    // Replay of the interchanges: step j moves the pivot's slot to position j and the
-    // slot there to the pivot's old position.  Only the slots 0 .. 31 (whose position
-    // lane i tracks) and the pivots ever leave their own position.
+    // Replay of the interchanges from the pivots' positions, as in panel_map_kernel: step j
+    // moves the pivot's slot to position j and the slot there to the pivot's old position.
+    // Only the slots 0 .. 31 (whose position lane i tracks) and the pivots ever leave their
+    // own position.
     if (W > 1) __syncthreads();
     else __syncwarp();
-    if (warp == 0) {
-      if (q == 0 && lane < jb && !(fabs((double)spv[lane]) > thresh)) atomicOr(status, 1);
-      int pos = lane, fin = 0, pslot = lane, pdst = 0;
-      const int psb = lane < jb ? spiv[lane] : -1;
+    if (warp == 0 && q == 0) {
+      if (lane < jb && !(fabs((double)spv[lane]) > thresh)) atomicOr(status, 1);
+      int pos = lane, fin = 0, pslot = lane;
+      const int pdst = lane < jb ? spiv[lane] : lane;
       for (int j = 0; j < jb; ++j) {
-        int sb = __shfl_sync(0xffffffffu, psb, j);
-        const unsigned at = __ballot_sync(0xffffffffu, pos == j && !fin);
-        const int ia = at ? __ffs(at) - 1 : j;  // slot at position j
-        if (sb < 0) sb = ia;
-        const int pb = __shfl_sync(0xffffffffu, pos, sb & 31);
-        const int p = sb < kNB ? pb : sb;
+        const int p = __shfl_sync(0xffffffffu, pdst, j);
+        const unsigned at = __ballot_sync(0xffffffffu, pos == p && !fin);
+        const int sb = at ? __ffs(at) - 1 : p;  // slot at position p
+        const unsigned here = __ballot_sync(0xffffffffu, pos == j && !fin);
+        const int ia = __ffs(here) - 1;  // slot at position j
         if (lane == ia) pos = p;
         if (lane == sb) {
           pos = j;
           fin = 1;
         }
-        if (lane == j) {
-          pslot = sb;
-          pdst = p;
-        }
+        if (lane == j) pslot = sb;
       }
-      if (q == 0 && lane < jb) {
+      if (lane < jb) {
         pvf[lane] = j0 + pdst;
         mpf[lane] = pslot;
         mpf[kNB + lane] = fin ? -1 : pos;
       }
-      spos[lane] = pos;
-      if (q == 0) {  // the row permutation of the eliminated block, kept up to date
-        int* pm = perm + f * k + j0;
-        const int vs = lane < kl ? pm[lane] : 0;                 // at slot `lane`
-        const int vp = lane < jb ? pm[pslot] : 0;                // at this step's pivot slot
-        __syncwarp();
-        if (lane < kl && !fin) pm[pos] = vs;
-        if (lane < jb) pm[lane] = vp;
-      }
+      // the row permutation of the eliminated block, kept up to date
+      int* pm = perm + f * k + j0;
+      const int vs = lane < kl ? pm[lane] : 0;                 // at slot `lane`
+      const int vp = lane < jb ? pm[pslot] : 0;                // at this step's pivot slot
+      __syncwarp();
+      if (lane < kl && !fin) pm[pos] = vs;
+      if (lane < jb) pm[lane] = vp;
     }
-    if (W > 1) __syncthreads();
-    else __syncwarp();
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int sl = s0 + r * NT;
       if (sl < rows) {
-        const int pos = pj[r] >= 0 ? pj[r] : (sl < kNB ? spos[sl] : sl);
+        const int pos = pj[r] >= 0 ? pj[r] : (r == 0 ? pos0 : sl);
 #pragma unroll
         for (int c = 0; c < kNB; ++c)
           if (c < jb) A[pos + (long)c * m] = a[r][c];
@@ -1430,7 +1436,10 @@ __global__ void lu_perm_kernel(const int* piv, int* perm, int k, int nf) {
 // the strict lower part from L^{-1}, the upper part with the diagonal from U^{-1}; the
 // sweeps then resolve a diagonal block with a matrix-vector product instead of 32
 // dependent steps.  With one thread per column (496 FMAs and 32 divisions in a row) an FP64
-// launch took 64 us however few its blocks were.
+// launch took 64 us however few its blocks were.  The FP32 U block keeps one thread per
+// column: row i subtracts its products in the order of l = i + 1 ..., which starts with the
+// entry computed last, so four lanes could only take another order, and the FP32
+// preconditioner's bits would change with it (the chain costs FP32 ~2 us).
 template <class T>
 __global__ void __launch_bounds__(256) diag32_kernel(T* fronts, int m, int k, T* Xl, T* Xu, int ldx,
                                                      long sX) {
@@ -1447,6 +1456,26 @@ __global__ void __launch_bounds__(256) diag32_kernel(T* fronts, int m, int k, T*
   if (threadIdx.x < kNB) dinv[threadIdx.x] = (T)1 / Bk[threadIdx.x][threadIdx.x];
   __syncthreads();
   const bool upper = threadIdx.x >= 128;
+  if (sizeof(T) == sizeof(float) && upper) {
+    const int c = threadIdx.x - 128;
+    if (c >= jb) return;
+    T x[kNB];
+#pragma unroll
+    for (int i = 0; i < kNB; ++i) x[i] = i == c ? (T)1 : (T)0;
+#pragma unroll
+    for (int i = kNB - 1; i >= 0; --i) {
+      T acc = x[i];
+#pragma unroll
+      for (int l = i + 1; l < kNB; ++l) acc = fma(-Bk[i][l], x[l], acc);
+      x[i] = acc / Bk[i][i];
+    }
+    T* out = Xl == nullptr ? A + j0 + (long)(j0 + c) * m
+                           : Xu + (long)blockIdx.y * sX + j0 + (long)(j0 + c) * ldx;
+#pragma unroll
+    for (int i = 0; i < kNB; ++i)
+      if (i < jb && (Xl != nullptr || i <= c)) out[i] = x[i];
+    return;
+  }
   const int sub = threadIdx.x & 3, c = (threadIdx.x & 127) >> 2, base = threadIdx.x & 28;
   constexpr int R = kNB / 4;
   T x[R];
@@ -1992,6 +2021,7 @@ bool panel_shape(int nf, int rows, int* C, int* NT, int* R) {
 template <class T>
 bool panel_in_registers(const DevLevel& L, const FactorWork& W) {
   int c, nt, r;
+  if (W.grid_panel) return false;
   if (sizeof(T) == 4 && W.calu && grid_panel_front<T>(L.m)) return false;
   return panel_shape<T>(L.nf, L.m, &c, &nt, &r);
 }
@@ -2158,9 +2188,18 @@ void schur_update(DevLevel& L, T* F, int M, int N, int K, long offA, long offB, 
 }
 
 template <class T>
-cudaError_t factor_level_t(int d, DevLevel& L, const DevLevel* child, const double* Qcat,
-                           const double* Ccat, const double* q, double ptol, int* status,
-                           const FactorWork& W, cudaStream_t st) {
+void front_scale(DevLevel& L, cudaStream_t st) {
+  const long mm = (long)L.m * L.m;
+  cudaMemsetAsync(L.scale, 0, sizeof(double) * L.nf, st);
+  long chunks = std::min<long>(std::max<long>(1, mm / (256 * 16)), std::max<long>(1, 1216 / L.nf));
+  dim3 gs((unsigned)chunks, L.nf);
+  front_scale_kernel<T><<<gs, 256, 0, st>>>((const T*)L.front, mm, L.scale);
+}
+
+// LU of the fronts of a level and the inverses of their diagonal blocks, from the assembled
+// fronts and their largest magnitudes L.scale.
+template <class T>
+cudaError_t lu_fronts(DevLevel& L, double ptol, int* status, const FactorWork& W, cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(lu_panel_grid_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2169,38 +2208,8 @@ cudaError_t factor_level_t(int d, DevLevel& L, const DevLevel* child, const doub
                          (int)kGridPanelSmem + 1024);
     attr = true;
   }
-  const long mm = (long)L.m * L.m;
   const int m = L.m, k = L.k;
   T* F = (T*)L.front;
-  ProfScope pa(PROF_ASSEMBLE, st);
-  cudaError_t e = cudaMemsetAsync(F, 0, sizeof(T) * mm * L.nf, st);
-  if (e != cudaSuccess) return e;
-  int na = 1;
-  if (L.nasm > 0) {
-    dim3 g((L.nasm + 255) / 256, L.nf);
-    assemble_kernel<T><<<g, 256, 0, st>>>(F, L.m, L.nasm, L.asm_row, L.asm_tidx, L.asm_cvar,
-                                          L.gidx, Qcat, Ccat, q, L.nfp > 0 ? L.nfp : L.nf,
-                                          W.tab_stride);
-    ++na;
-  }
-  double abytes = (double)sizeof(T) * mm * L.nf;
-  if (child) {
-    const int nbd = L.mc - L.kc;
-    long work = (long)nbd * nbd;
-    dim3 g((unsigned)((work + 256 * kEaU - 1) / (256 * kEaU)), L.nf);
-    for (int dl = 0; dl < (1 << d); ++dl)
-      extend_add_kernel<T><<<g, 256, 0, st>>>(F, L.m, L.nb1, (const T*)child->front, L.mc, L.kc,
-                                               L.ea_map + (long)dl * nbd, dl, d);
-    na += 1 << d;
-    abytes += (double)sizeof(T) * work * child->nf;
-  }
-  cudaMemsetAsync(L.scale, 0, sizeof(double) * L.nf, st);
-  {
-    long chunks = std::min<long>(std::max<long>(1, mm / (256 * 16)), std::max<long>(1, 1216 / L.nf));
-    dim3 gs((unsigned)chunks, L.nf);
-    front_scale_kernel<T><<<gs, 256, 0, st>>>(F, mm, L.scale);
-  }
-  pa.done(abytes, na + 1, st);
   if (panel_in_registers<T>(L, W)) {
     const long np = (long)L.nf * k;
     perm_identity_kernel<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(L.perm, k, np);
@@ -2331,6 +2340,39 @@ cudaError_t factor_level_t(int d, DevLevel& L, const DevLevel* child, const doub
   return cudaGetLastError();
 }
 
+template <class T>
+cudaError_t factor_level_t(int d, DevLevel& L, const DevLevel* child, const double* Qcat,
+                           const double* Ccat, const double* q, double ptol, int* status,
+                           const FactorWork& W, cudaStream_t st) {
+  const long mm = (long)L.m * L.m;
+  T* F = (T*)L.front;
+  ProfScope pa(PROF_ASSEMBLE, st);
+  cudaError_t e = cudaMemsetAsync(F, 0, sizeof(T) * mm * L.nf, st);
+  if (e != cudaSuccess) return e;
+  int na = 1;
+  if (L.nasm > 0) {
+    dim3 g((L.nasm + 255) / 256, L.nf);
+    assemble_kernel<T><<<g, 256, 0, st>>>(F, L.m, L.nasm, L.asm_row, L.asm_tidx, L.asm_cvar,
+                                          L.gidx, Qcat, Ccat, q, L.nfp > 0 ? L.nfp : L.nf,
+                                          W.tab_stride);
+    ++na;
+  }
+  double abytes = (double)sizeof(T) * mm * L.nf;
+  if (child) {
+    const int nbd = L.mc - L.kc;
+    long work = (long)nbd * nbd;
+    dim3 g((unsigned)((work + 256 * kEaU - 1) / (256 * kEaU)), L.nf);
+    for (int dl = 0; dl < (1 << d); ++dl)
+      extend_add_kernel<T><<<g, 256, 0, st>>>(F, L.m, L.nb1, (const T*)child->front, L.mc, L.kc,
+                                               L.ea_map + (long)dl * nbd, dl, d);
+    na += 1 << d;
+    abytes += (double)sizeof(T) * work * child->nf;
+  }
+  front_scale<T>(L, st);
+  pa.done(abytes, na + 1, st);
+  return lu_fronts<T>(L, ptol, status, W, st);
+}
+
 }  // namespace
 
 cudaError_t factor_level(int prec, int d, DevLevel& L, const DevLevel* child, const double* Qcat,
@@ -2339,6 +2381,37 @@ cudaError_t factor_level(int prec, int d, DevLevel& L, const DevLevel* child, co
   if (prec == SP_PREC_FP32)
     return factor_level_t<float>(d, L, child, Qcat, Ccat, q, pivot_tol, status, W, st);
   return factor_level_t<double>(d, L, child, Qcat, Ccat, q, pivot_tol, status, W, st);
+}
+
+cudaError_t front_lu_raw(int prec, int m, int k, int nf, int grid_panel, double pivot_tol,
+                         unsigned long long wait_ns, void* fronts, int* piv, int* perm, int* status,
+                         cudaStream_t st) {
+  DevLevel L;
+  FactorWork W;
+  L.m = m;
+  L.k = k;
+  L.nf = nf;
+  L.front = fronts;
+  L.piv = piv;
+  L.perm = perm;
+  W.grid_panel = grid_panel;
+  W.wait_ns = wait_ns;
+  cudaError_t e = cudaMalloc(&L.scale, sizeof(double) * nf);
+  if (e == cudaSuccess) e = cudaMalloc(&L.pmap, sizeof(int) * 2 * kNB * nf * ((k + kNB - 1) / kNB));
+  if (e == cudaSuccess && (grid_panel || factor_grid_panel(prec, m)))
+    e = cudaMalloc(&W.gpub, sizeof(unsigned long long) * grid_panel_pub_words(nf));
+  if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), st);
+  auto go = [&](auto t) {
+    using T = decltype(t);
+    front_scale<T>(L, st);
+    return lu_fronts<T>(L, pivot_tol, status, W, st);
+  };
+  if (e == cudaSuccess) e = prec == SP_PREC_FP32 ? go(0.f) : go(0.0);
+  const cudaError_t es = cudaStreamSynchronize(st);
+  cudaFree(L.scale);
+  cudaFree(L.pmap);
+  cudaFree(W.gpub);
+  return e != cudaSuccess ? e : es;
 }
 
 cudaError_t schur_update_raw(int prec, bool tc, bool split, int M, int N, int K, const void* A,

@@ -124,6 +124,7 @@ struct FactorWork {
   bool tc_split = false;      // ... as 3xTF32 (hi/lo split, FP32 accuracy)
   int tc_epi = 0;             // epilogue of the tensor-core update (tc_schur_update's epi)
   unsigned long long wait_ns = 2000000000ull;  // limit of each grid-panel poll (global timer ns)
+  int grid_panel = 0;         // 1: every panel on the cooperative grid (tests of that panel)
   int calu = 0;               // FP32 grid panels by tournament pivoting (0: column by column)
   long tab_stride = 0;        // problem group: entries between two problems' Q / C tables
   // grid panel (fronts too tall for a cluster): per front 2 x kGridPanelMaxG
@@ -148,6 +149,14 @@ size_t grid_panel_pub_words(int nf);
 // outer block width of the blocked LU of a front (0: the 32-column right-looking
 // LU with a Schur update after every panel)
 int factor_outer_block(int prec, bool tc, int m, int k);
+
+// The factorisation of nf dense fronts (m x m, column-major, k eliminated rows) by the kernels
+// of a level, from the panels to the inverted 32-wide diagonal blocks: the panels as the level
+// takes them, or (grid_panel) on the cooperative grid; piv and perm nf x k.  Allocates its work
+// buffers and synchronises: the entry point of the tests of these kernels.
+cudaError_t front_lu_raw(int prec, int m, int k, int nf, int grid_panel, double pivot_tol,
+                         unsigned long long wait_ns, void* fronts, int* piv, int* perm, int* status,
+                         cudaStream_t st);
 
 // C[M x N] -= A[M x K] B[K x N] with the kernel the factorisation uses for the
 // form (FP64 or FP32 SIMT; FP32 with tc: tensor cores, K <= kTcMaxK)
