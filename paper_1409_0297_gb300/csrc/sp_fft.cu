@@ -7,17 +7,22 @@
 // The n^d transform is done axis by axis; a CTA owns W neighbouring lines of one axis.  A
 // line is transformed by self-sorting (Stockham) steps: with l the product of the radices
 // before a step of radix r, butterfly b takes x[b + k n / r] (k < r), multiplies by
-// w_{l r}^{(b mod l) k}, transforms and writes y[(b - b mod l) r + b mod l + k l].  A thread
+// w_{l r}^{(b mod l) k}, transforms and writes y[(b - b mod l) r + b mod l + k l].  The
+// inverse is its mirror image: the steps in reverse, each reading where the forward step
+// wrote, transforming, multiplying by the conjugate twiddles and writing where the forward
+// step read.  A thread
 // keeps its butterflies in registers; the first step reads device memory, the last writes
 // it, and between steps the line passes through shared memory once, so a line of 64 points
-// (three steps of radix 4) costs two exchanges and no bit reversal, and its first step no
+// (three steps of radix 4) costs two exchanges and no bit reversal, and the steps at l = 1 no
 // twiddles.  Fused pointwise work:
 //   first pass   x -> q x              (PRE_Q)
-//   last axis    forward, * D/N, inverse in one pass (MID): the inverse takes the radices in
-//                reverse, so its first step wants exactly the elements that the last forward
-//                step left in the thread's registers
+//   last axis    forward, * D/N, inverse in one pass (MID): the inverse's first step wants
+//                exactly the elements that the last forward step left in the thread's registers
 //   final pass   out = x + result      (POST_ADD)
-// n = 2^p or 3 2^p; the radix 3 is the last forward step.
+// n = 2^p or 3 2^p: a step of radix 2 when p is odd, steps of radix 4, then the radix 3, so l
+// is always a power of two.  The bits do not depend on the launch shape: twiddles before the
+// forward and behind the inverse butterflies, q and D / N rounded before they enter one.
+// (FP32 preconditioners turn a last bit of the operator into another residual at 1e-12.)
 // What bounds it: the FP64 pipe (28 instructions per radix-4 butterfly, two lanes per SM
 // cycle) on large grids, the chain of three launches on small ones.
 #include <algorithm>
@@ -44,6 +49,10 @@ __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_doub
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 
+// a product that is rounded before it is added to anything
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+
 constexpr int kMaxSteps = 16;
 
 template <class VT>
@@ -63,6 +72,7 @@ struct PassArgs {
   int ld;               // entries between two lines in shared memory
   int steps;
   int rad[kMaxSteps];   // radices of the forward transform; the inverse runs them in reverse
+  int sh_last;          // log2 of the product of the radices before the last
   int mode;             // 0 forward, 1 inverse, 2 middle (forward, scale, inverse)
   int qper;             // q and Dn per vector: vector v reads those of v % qper (vstride apart)
 };
@@ -139,103 +149,93 @@ constexpr int kVal = 6 * G;
 template <int r, int G>
 constexpr int kPer = (r == 4 ? 1 : 2) * G;
 
-// The product l of the radices before a step: a power of two (sh its logarithm) except
-// behind a radix 3 (sh < 0), so that the remainders of a step are masks, not divisions (a
-// small grid's pass is one chain of latencies).
-struct Radix {
-  int l = 1, sh = 0;
-  __device__ __forceinline__ void grow(int r) {
-    l *= r;
-    sh = (sh < 0 || r == 3) ? -1 : sh + (r >> 1);  // r = 2: 1, r = 4: 2
-  }
-  __device__ __forceinline__ int mod(int b) const { return sh >= 0 ? b & (l - 1) : b % l; }
-  __device__ __forceinline__ int quot(int b) const { return sh >= 0 ? b >> sh : b / l; }
-};
-
-// The twiddles of a step of radix r at l, w_{l r}^{(b mod l) k} for k = 1 .. r - 1 of each
-// butterfly, loaded ahead of the exchange that the step waits for (G = 1; the threads of
+// The twiddles of a step of radix r at l = 2^sh, w_{l r}^{(b mod l) k} for k = 1 .. r - 1 of
+// each butterfly, loaded ahead of the exchange that the step waits for (G = 1; the threads of
 // longer lines have no registers left for them and load them in the step).
 template <int r, bool INV, class VT>
-__device__ __forceinline__ void load_tw(const PassArgs<VT>& a, int bb, const Radix& l, VT* tw) {
+__device__ __forceinline__ void load_tw(const PassArgs<VT>& a, int bb, int sh, VT* tw) {
   const int nb = a.n / r;
 #pragma unroll
   for (int j = 0; j < kPer<r, 1>; ++j) {
     const int b = bb + j * a.U;
-    const int t = b < nb ? l.mod(b) * l.quot(nb) : 0;  // w_{l r}^1 = w_n^(n / (l r))
+    const int t = b < nb ? (b & ((1 << sh) - 1)) * (nb >> sh) : 0;  // w_{l r}^1 = w_n^(n / (l r))
 #pragma unroll
     for (int k = 1; k < r; ++k) tw[j * (r - 1) + k - 1] = tw_at<INV>(a, t * k);
   }
 }
 
-// One step of radix r at l for the butterflies b = bb + j U of a line: from the values in v
-// (first: already there, no twiddles) or from the line in shared memory, to registers.
+// One step of radix r at l = 2^sh for the butterflies b = bb + j U of a line: from the values
+// in v (reg: already there) or from the line in shared memory, to registers.
 template <int r, bool INV, int G, class VT>
-__device__ __forceinline__ void step_reg(const PassArgs<VT>& a, const VT* line, int bb, bool first,
-                                         const Radix& l, const VT* tw, VT* v) {
-  const int nb = a.n / r;
+__device__ __forceinline__ void step_reg(const PassArgs<VT>& a, const VT* line, int bb, bool reg,
+                                         int sh, const VT* tw, VT* v) {
+  const int nb = a.n / r, lm = (1 << sh) - 1;
 #pragma unroll
   for (int j = 0; j < kPer<r, G>; ++j) {
     const int b = bb + j * a.U;
     if (b >= nb) continue;
     VT* x = v + j * r;
-    if (!first) {
+    const int m = b & lm;
+    if (!reg) {
+      const int o = (b - m) * r + m;
 #pragma unroll
-      for (int k = 0; k < r; ++k) x[k] = line[spos(b + k * nb)];
-      const int t = G > 1 ? l.mod(b) * l.quot(nb) : 0;
+      for (int k = 0; k < r; ++k) x[k] = line[spos(INV ? o + (k << sh) : b + k * nb)];
+    }
+    if (INV) dft_reg<r, INV>(x);
+    if (sh > 0) {
+      const int t = m * (nb >> sh);
 #pragma unroll
       for (int k = 1; k < r; ++k)
         x[k] = cmul(x[k], G > 1 ? tw_at<INV>(a, t * k) : tw[j * (r - 1) + k - 1]);
     }
-    dft_reg<r, INV>(x);
+    if (!INV) dft_reg<r, INV>(x);
   }
 }
-template <int r, int G, class VT>
-__device__ __forceinline__ void put_line(const PassArgs<VT>& a, VT* line, int bb, const Radix& l,
-                                         const VT* v) {
-  const int nb = a.n / r;
+template <int r, bool INV, int G, class VT>
+__device__ __forceinline__ void put_line(const PassArgs<VT>& a, VT* line, int bb, int sh, const VT* v) {
+  const int nb = a.n / r, lm = (1 << sh) - 1;
 #pragma unroll
   for (int j = 0; j < kPer<r, G>; ++j) {
     const int b = bb + j * a.U;
     if (b >= nb) continue;
-    const int m = l.mod(b), o = (b - m) * r + m;
+    const int m = b & lm, o = (b - m) * r + m;
 #pragma unroll
-    for (int k = 0; k < r; ++k) line[spos(o + k * l.l)] = v[j * r + k];
+    for (int k = 0; k < r; ++k) line[spos(INV ? b + k * nb : o + (k << sh))] = v[j * r + k];
   }
 }
 
-// The transform of one line: on entry the first step's inputs are in v, on return the last
-// step's outputs (element b + k n / r of butterfly b), radices rad[0 .. steps) or, INV, in
-// reverse.
+// The transform of one line: forward, on entry the first step's inputs are in v, on return the
+// last step's outputs (element b + k n / r of butterfly b); INV the other way round.
 template <bool INV, int G, class VT>
 __device__ __forceinline__ void transform(const PassArgs<VT>& a, VT* line, int bb, bool live, VT* v) {
   VT tw[4];  // G = 1: kPer (r - 1) twiddles of the next step
-  Radix l;
+  auto fetch = [&](int r, int sh) {
+    if (G != 1 || !live || sh == 0) return;
+    if (r == 4) load_tw<4, INV>(a, bb, sh, tw);
+    else if (r == 2) load_tw<2, INV>(a, bb, sh, tw);
+    else load_tw<3, INV>(a, bb, sh, tw);
+  };
+  int sh = INV ? a.sh_last : 0;
+  if (INV) fetch(a.rad[a.steps - 1], sh);
   for (int s = 0; s < a.steps; ++s) {
     const int r = a.rad[INV ? a.steps - 1 - s : s];
-    const bool first = s == 0, last = s == a.steps - 1;
     if (live) {
-      if (r == 4) step_reg<4, INV, G>(a, line, bb, first, l, tw, v);
-      else if (r == 2) step_reg<2, INV, G>(a, line, bb, first, l, tw, v);
-      else step_reg<3, INV, G>(a, line, bb, first, l, tw, v);
+      if (r == 4) step_reg<4, INV, G>(a, line, bb, s == 0, sh, tw, v);
+      else if (r == 2) step_reg<2, INV, G>(a, line, bb, s == 0, sh, tw, v);
+      else step_reg<3, INV, G>(a, line, bb, s == 0, sh, tw, v);
     }
-    if (!last) {
-      const int nx = a.rad[INV ? a.steps - 2 - s : s + 1];
-      Radix ln = l;
-      ln.grow(r);
-      if (G == 1 && live) {
-        if (nx == 4) load_tw<4, INV>(a, bb, ln, tw);
-        else if (nx == 2) load_tw<2, INV>(a, bb, ln, tw);
-        else load_tw<3, INV>(a, bb, ln, tw);
-      }
-      __syncthreads();  // the line has been read
-      if (live) {
-        if (r == 4) put_line<4, G>(a, line, bb, l, v);
-        else if (r == 2) put_line<2, G>(a, line, bb, l, v);
-        else put_line<3, G>(a, line, bb, l, v);
-      }
-      __syncthreads();
+    if (s == a.steps - 1) break;
+    const int rn = a.rad[INV ? a.steps - 2 - s : s + 1];
+    const int shn = INV ? sh - (rn >> 1) : sh + (r >> 1);  // log2 of 2 and 4; 3 is the last step
+    fetch(rn, shn);
+    __syncthreads();  // the line has been read
+    if (live) {
+      if (r == 4) put_line<4, INV, G>(a, line, bb, sh, v);
+      else if (r == 2) put_line<2, INV, G>(a, line, bb, sh, v);
+      else put_line<3, INV, G>(a, line, bb, sh, v);
     }
-    l.grow(r);
+    __syncthreads();
+    sh = shn;
   }
 }
 
@@ -284,8 +284,8 @@ __global__ void __launch_bounds__(1024) fft_pass_kernel(PassArgs<VT> a) {
     if (a.q)
       each_value<G>(a, rf, bb, v, [&](VT& x, int i) {
         const T qq = a.q[qoff + (long)i * a.S];
-        x.x *= qq;
-        x.y *= qq;
+        x.x = mul_rn(x.x, qq);
+        x.y = mul_rn(x.y, qq);
       });
   }
   if (a.mode != 1) transform<false, G>(a, line, bb, live, v);
@@ -293,8 +293,8 @@ __global__ void __launch_bounds__(1024) fft_pass_kernel(PassArgs<VT> a) {
     if (live)
       each_value<G>(a, a.rad[a.steps - 1], bb, v, [&](VT& x, int i) {
         const T dn = a.Dn[qoff + (long)i * a.S];
-        x.x *= dn;
-        x.y *= dn;
+        x.x = mul_rn(x.x, dn);
+        x.y = mul_rn(x.y, dn);
       });
   }
   if (a.mode != 0) transform<true, G>(a, line, bb, live, v);
@@ -322,11 +322,13 @@ cudaError_t run_pass(int d, int n, const VT* tw, const typename Real<VT>::T* Dn,
   a.addx = addx;
   a.tw = tw;
   a.n = n;
-  {  // radices: 4 as often as they go, a 2, a 3
-    int m = n % 3 == 0 ? n / 3 : n;
-    for (; m >= 4; m /= 4) a.rad[a.steps++] = 4;
-    if (m == 2) a.rad[a.steps++] = 2;
+  {  // radices: a 2 for an odd power, fours, a 3
+    int p = 0;
+    while ((n % 3 == 0 ? n / 3 : n) >> (p + 1)) ++p;
+    if (p & 1) a.rad[a.steps++] = 2;
+    for (int i = 0; i < p / 2; ++i) a.rad[a.steps++] = 4;
     if (n % 3 == 0) a.rad[a.steps++] = 3;
+    a.sh_last = n % 3 == 0 ? p : p - a.rad[a.steps - 1] / 2;
   }
   long S = 1;
   for (int i = 0; i < axis; ++i) S *= n;
