@@ -987,7 +987,7 @@ static sp_status setup_impl(int d, int n, int b, int P, const double* shifts, sp
   SP_CK(dalloc(c.get(), &c->t, sizeof(double2) * N * IM));
   SP_CK(dalloc(c.get(), &c->fbuf, sizeof(double2) * NP));
   SP_CK(dalloc(c.get(), &c->ubuf, sizeof(double2) * N * IM));
-  c->K.nblk = (int)std::min<long>(304, (N + 255) / 256);
+  c->K.nblk = krylov_blocks(N);
   SP_CK(dalloc(c.get(), &c->K.partial, sizeof(double2) * (size_t)c->K.nblk * 1024 * IM));
   SP_CK(dalloc(c.get(), &c->K.h, sizeof(double2) * 1024));
   SP_CK(cudaMallocHost(&c->host_sc, 8 * sizeof(double) * IM));
@@ -1686,6 +1686,22 @@ sp_status sp_test_front_lu(sp_precision prec, int m, int k, int nf, int grid_pan
                      ds, nullptr);
   if (e == cudaSuccess) e = cudaMemcpy(status_host, ds, sizeof(int), cudaMemcpyDeviceToHost);
   cudaFree(ds);
+  return cuda_status(e);
+}
+
+// Likewise: h_dev[j] = V_j^H w (j < nv) and *nrm_dev = ||w|| by the Gram-Schmidt kernels.
+sp_status sp_test_dots(long long N, int nv, const void* V, void* w, void* h_dev, double* nrm_dev) {
+  if (N < 1 || nv < 1 || nv > 64 || !V || !w || !h_dev || !nrm_dev) return SP_ERR_ARG;
+  KrylovWork K;
+  K.nblk = krylov_blocks(N);
+  cudaError_t e = cudaMalloc(&K.partial, sizeof(double2) * K.nblk * nv);
+  if (e == cudaSuccess) e = cudaMalloc(&K.h, sizeof(double2) * nv);
+  if (e == cudaSuccess)
+    e = kr_dots((const double2*)V, N, nv, (const double2*)w, N, K, (double2*)h_dev, nullptr);
+  if (e == cudaSuccess) e = kr_norm((const double2*)w, N, K, nrm_dev, nullptr);
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  cudaFree(K.partial);
+  cudaFree(K.h);
   return cuda_status(e);
 }
 

@@ -230,6 +230,12 @@ struct KrylovWork {
   double* nrm = nullptr;       // scalars
 };
 // h[0..nv) = V[0..nv)^H w  (V rows of length N, stride ldv)
+// CTAs of the reduction kernels for vectors of N entries: ~1024 entries each, at most two to an
+// SM.  A CTA adds its contiguous share, so this number fixes the order of every sum.
+inline int krylov_blocks(long N) {
+  const long b = (N + 1023) / 1024;
+  return (int)(b < 1 ? 1 : b > 304 ? 304 : b);
+}
 cudaError_t kr_dots(const double2* V, long ldv, int nv, const double2* w, long N,
                     KrylovWork& K, double2* h_out, cudaStream_t st);
 // w -= V h; if h2_out != null also h2 = V^H w (after the update)

@@ -19,11 +19,13 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// A CTA takes the elements i = 256 (blockIdx.x + g gridDim.x) + thread: with whole units of
-// 256 dealt out in turn, the SMs' shares of the FP64 work differ by one unit (contiguous
-// shares over 256 CTAs left the 152 SMs 19 % apart at N = 262144).
-__device__ __forceinline__ long first_of() { return (long)blockIdx.x * kThr + threadIdx.x; }
-__device__ __forceinline__ long stride_of() { return (long)gridDim.x * kThr; }
+// contiguous share of the N elements of a CTA; krylov_blocks gives the number of shares, and
+// with it the order of every sum
+__device__ __forceinline__ void chunk_of(long N, long* c0, long* c1) {
+  const long per = (N + gridDim.x - 1) / gridDim.x;
+  *c0 = (long)blockIdx.x * per;
+  *c1 = min(N, *c0 + per);
+}
 
 // The Krylov basis V is read with the evict-first hint (it is larger than L2 at
 // 512^2 and streams through it every iteration), so the preconditioner's data stays.
@@ -34,7 +36,7 @@ __device__ __forceinline__ long stride_of() { return (long)gridDim.x * kThr; }
 // values a lane still holds (15 additions and one more instead of 80: with four elements
 // per thread the 80 were as much FP64 work as the products), then over the CTA in shared
 // memory in a fixed order.
-__device__ void chunk_dots(const double2* V, long ldv, int nv, const double2* w, long N,
+__device__ void chunk_dots(const double2* V, long ldv, int nv, const double2* w, long c0, long c1,
                            double2* partial) {
   constexpr int kJ = 8;
   __shared__ double red[2 * kJ][kThr / 32];
@@ -44,7 +46,7 @@ __device__ void chunk_dots(const double2* V, long ldv, int nv, const double2* w,
     double sum[2 * kJ];  // real parts, imaginary parts
 #pragma unroll
     for (int q = 0; q < 2 * kJ; ++q) sum[q] = 0.0;
-    for (long i = first_of(); i < N; i += stride_of()) {
+    for (long i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
       const double2 wi = w[i];
 #pragma unroll
       for (int q = 0; q < kJ; ++q) {
@@ -83,10 +85,10 @@ __device__ void chunk_dots(const double2* V, long ldv, int nv, const double2* w,
 
 // w_i -= sum_j V_j[i] hs_j over the chunk, four independent partial sums (FP64 FMA
 // latency); hs in shared memory.  Returns the thread's sum of |w_i|^2.
-__device__ double chunk_update(const double2* V, long ldv, int nv, double2* w, long N,
+__device__ double chunk_update(const double2* V, long ldv, int nv, double2* w, long c0, long c1,
                                const double2* hs) {
   double nrm = 0;
-  for (long i = first_of(); i < N; i += stride_of()) {
+  for (long i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
     double ax[4] = {0, 0, 0, 0}, ay[4] = {0, 0, 0, 0};
     int j = 0;
     for (; j + 4 <= nv; j += 4) {
@@ -125,9 +127,9 @@ __device__ void cta_norm2(double s, double2* partial) {
 }
 
 // partial[blockIdx.x] = (sum over the chunk of |w_i|^2, 0)
-__device__ void chunk_norm2(const double2* w, long N, double2* partial) {
+__device__ void chunk_norm2(const double2* w, long c0, long c1, double2* partial) {
   double s = 0;
-  for (long i = first_of(); i < N; i += stride_of()) {
+  for (long i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
     double2 v = w[i];
     s = fma(v.x, v.x, fma(v.y, v.y, s));
   }
@@ -252,7 +254,9 @@ __device__ __forceinline__ void combine_at(const double2* Z, long ldz, int k, co
 
 __global__ void __launch_bounds__(kThr) dots_kernel(const double2* V, long ldv, int nv,
                                                     const double2* w, long N, double2* partial) {
-  chunk_dots(V, ldv, nv, w, N, partial);
+  long c0, c1;
+  chunk_of(N, &c0, &c1);
+  chunk_dots(V, ldv, nv, w, c0, c1, partial);
 }
 
 __global__ void __launch_bounds__(kThr) update_dots_kernel(const double2* V, long ldv, int nv,
@@ -261,10 +265,12 @@ __global__ void __launch_bounds__(kThr) update_dots_kernel(const double2* V, lon
   __shared__ double2 hs[1024];
   for (int j = threadIdx.x; j < nv; j += blockDim.x) hs[j] = h[j];
   __syncthreads();
-  chunk_update(V, ldv, nv, w, N, hs);
+  long c0, c1;
+  chunk_of(N, &c0, &c1);
+  chunk_update(V, ldv, nv, w, c0, c1, hs);
   if (partial) {
     __syncthreads();
-    chunk_dots(V, ldv, nv, w, N, partial);
+    chunk_dots(V, ldv, nv, w, c0, c1, partial);
   }
 }
 
@@ -277,7 +283,9 @@ __global__ void reduce_partials_kernel(const double2* partial, int nblk, int nv,
 }
 
 __global__ void __launch_bounds__(kThr) norm2_kernel(const double2* w, long N, double2* partial) {
-  chunk_norm2(w, N, partial);
+  long c0, c1;
+  chunk_of(N, &c0, &c1);
+  chunk_norm2(w, c0, c1, partial);
 }
 
 __global__ void sqrt_kernel(const double2* s, double* out) { out[0] = sqrt(s[0].x); }
@@ -366,7 +374,9 @@ __global__ void kb_copy_kernel(KBatch b, double2* vec, int to_z) {
 __global__ void __launch_bounds__(kThr) kb_dots_kernel(KBatch b) {
   const int i = blockIdx.y;
   if (!inst_cont(b, i)) return;
-  chunk_dots(b.V + i * b.sV, b.N, b.head[i].j + 1, b.w + i * b.N, b.N, b.partial + i * b.sP);
+  long c0, c1;
+  chunk_of(b.N, &c0, &c1);
+  chunk_dots(b.V + i * b.sV, b.N, b.head[i].j + 1, b.w + i * b.N, c0, c1, b.partial + i * b.sP);
 }
 
 // w_i -= V_i h_i (h = h1 if second = 0, else h2); then the partials of h2 = V_i^H w_i
@@ -381,12 +391,14 @@ __global__ void __launch_bounds__(kThr) kb_update_dots_kernel(KBatch b, int seco
   __syncthreads();
   const double2* V = b.V + i * b.sV;
   double2* w = b.w + i * b.N;
-  const double s = chunk_update(V, b.N, nv, w, b.N, hs);
+  long c0, c1;
+  chunk_of(b.N, &c0, &c1);
+  const double s = chunk_update(V, b.N, nv, w, c0, c1, hs);
   if (second) {
     cta_norm2(s, b.partial + i * b.sP);
   } else {
     __syncthreads();
-    chunk_dots(V, b.N, nv, w, b.N, b.partial + i * b.sP);
+    chunk_dots(V, b.N, nv, w, c0, c1, b.partial + i * b.sP);
   }
 }
 
@@ -403,7 +415,9 @@ __global__ void kb_reduce_kernel(KBatch b, int which) {
 // partials of |x_i|^2 (x with instance stride N)
 __global__ void __launch_bounds__(kThr) kb_norm2_kernel(KBatch b, const double2* x) {
   const int i = blockIdx.y;
-  chunk_norm2(x + i * b.N, b.N, b.partial + i * b.sP);
+  long c0, c1;
+  chunk_of(b.N, &c0, &c1);
+  chunk_norm2(x + i * b.N, c0, c1, b.partial + i * b.sP);
 }
 
 // nrm_i[slot] = sqrt(sum of the partials); one warp per instance
@@ -655,13 +669,6 @@ cudaError_t kb_copy_nrm(const KBatch& b, int I, int from, int to, cudaStream_t s
 namespace sp {
 
 namespace {
-
-// contiguous share of the N elements of a CTA
-__device__ __forceinline__ void chunk_of(long N, long* c0, long* c1) {
-  const long per = (N + gridDim.x - 1) / gridDim.x;
-  *c0 = (long)blockIdx.x * per;
-  *c1 = min(N, *c0 + per);
-}
 
 __device__ __forceinline__ void chunk_dots32(const float2* V, long ldv, int nv, const float2* w,
                                              long c0, long c1, double2* partial) {
