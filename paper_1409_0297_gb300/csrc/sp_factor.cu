@@ -451,17 +451,11 @@ __device__ __forceinline__ unsigned mag_bits(double v) {
   const unsigned u = (unsigned)__double2hiint(v) & 0x7fffffffu;
   return u > 0x7ff00000u || (u == 0x7ff00000u && __double2loint(v) != 0) ? 0u : u;
 }
-// the lane with the largest key, ties to the smallest position (the whole warp calls it);
-// *key becomes that lane's key
-__device__ __forceinline__ int pick_lane(unsigned* key, unsigned pos) {
-  const unsigned mine = *key, best = __reduce_max_sync(0xffffffffu, mine);
-  unsigned in = __ballot_sync(0xffffffffu, mine == best);
-  if (in & (in - 1)) {
-    const unsigned p = __reduce_min_sync(0xffffffffu, mine == best ? pos : 0xffffffffu);
-    in = __ballot_sync(0xffffffffu, mine == best && pos == p);
-  }
+// the largest key of the warp and, of the lanes that hold it, the smallest position
+__device__ __forceinline__ void pick(unsigned* key, unsigned* pos) {
+  const unsigned best = __reduce_max_sync(0xffffffffu, *key);
+  *pos = __reduce_min_sync(0xffffffffu, *key == best ? *pos : 0xffffffffu);
   *key = best;
-  return __ffs(in) - 1;
 }
 // 1 / v: FP64 from the hardware's approximate reciprocal (20 bits) and two Newton steps
 // r += r (1 - v r), which double the correct bits (20 -> 40 -> full); magnitudes whose
@@ -601,21 +595,27 @@ __global__ void __launch_bounds__(NT)
       const int jj = 8 * o + u;
       if (jj < jb && !stop) {
         const int buf = u & 1;
-        // this thread's candidate: magnitude + 1 (0: none) and position
+        // this thread's candidate: magnitude + 1 (0: none) and position (rows r > 0 in the
+        // order of their positions)
         unsigned mg = 0, mpos = 0xffffffffu;
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-          if (pj[r] < 0 && s0 + r * NT < kl) {
-            const unsigned v = mag_bits(a[r][u]) + 1u, p = (unsigned)(r == 0 ? pos0 : s0 + r * NT);
-            if (v > mg || (v == mg && p < mpos)) {
-              mg = v;
-              mpos = p;
-            }
+        for (int r = 1; r < R; ++r) {
+          const unsigned v = pj[r] < 0 && s0 + r * NT < kl ? mag_bits(a[r][u]) + 1u : 0u;
+          if (v > mg) {
+            mg = v;
+            mpos = (unsigned)(s0 + r * NT);
           }
         }
-        unsigned wm = mg;
-        const int wl = pick_lane(&wm, mpos);
-        if (lane == wl) {
+        {
+          const unsigned v = pj[0] < 0 && s0 < kl ? mag_bits(a[0][u]) + 1u : 0u;
+          if (v && (v > mg || (v == mg && (unsigned)pos0 < mpos))) {
+            mg = v;
+            mpos = (unsigned)pos0;
+          }
+        }
+        unsigned wm = mg, wp = mpos;
+        pick(&wm, &wp);
+        if (mg == wm && mpos == wp && wm) {
 #pragma unroll
           for (int r = 0; r < R; ++r)
             if (pj[r] < 0 && (unsigned)(r == 0 ? pos0 : s0 + r * NT) == mpos) {
@@ -623,8 +623,10 @@ __global__ void __launch_bounds__(NT)
               for (int g = 0; g < kNB / 8; ++g)
                 if (g < live) store8(&wrow[buf][warp][8 * g], &a[r][8 * g]);
             }
+        }
+        if (lane == 0) {
           wmag[buf][warp] = wm;
-          wpos[buf][warp] = mpos;
+          wpos[buf][warp] = wp;
         }
         if (C > 1) {
           // a warp whose last wait gave up stops its whole CTA here
@@ -636,13 +638,15 @@ __global__ void __launch_bounds__(NT)
           __syncwarp();
         }
         // the CTA's best
-        unsigned best = wm;
+        unsigned best = wm, bpos = wp;
         int wb = 0;
         if (W > 1) {
-          best = lane < W ? wmag[buf][lane] : 0u;
-          wb = pick_lane(&best, lane < W ? wpos[buf][lane] : 0xffffffffu);
+          const unsigned bm = lane < W ? wmag[buf][lane] : 0u, bp = lane < W ? wpos[buf][lane] : 0xffffffffu;
+          best = bm;
+          bpos = bp;
+          pick(&best, &bpos);
+          wb = __ffs(__ballot_sync(0xffffffffu, bm == best && bp == bpos)) - 1;
         }
-        unsigned bpos = wpos[buf][wb];
         const T* prow = wrow[buf][wb];
         if (C > 1) {
           // push the row and its key to every CTA of the cluster (destinations spread
@@ -650,8 +654,7 @@ __global__ void __launch_bounds__(NT)
           const unsigned rdst = smem_addr(&crow[buf][q][lane]);
           const unsigned kdst = smem_addr(&ckey[buf][q]), bar = smem_addr(&cbar[buf]);
           const T rv = wrow[buf][wb][lane];
-          const unsigned long long key =
-              ((unsigned long long)best << 32) | bpos;
+          const unsigned long long key = ((unsigned long long)best << 32) | bpos;
           if (tid == 0)
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
                          "r"((unsigned)(C * (kNB * sizeof(T) + 8)))
@@ -664,9 +667,11 @@ __global__ void __launch_bounds__(NT)
           ok = bar_wait(bar, (jj >> 1) & 1, wait_ns);
           ok = __all_sync(0xffffffffu, ok);
           const unsigned long long kk = lane < C ? ckey[buf][lane] : 0xffffffffull;
-          best = (unsigned)(kk >> 32);
-          const int cb = pick_lane(&best, (unsigned)kk);
-          bpos = (unsigned)ckey[buf][cb];
+          const unsigned km = (unsigned)(kk >> 32), kp = (unsigned)kk;
+          best = km;
+          bpos = kp;
+          pick(&best, &bpos);
+          const int cb = __ffs(__ballot_sync(0xffffffffu, km == best && kp == bpos)) - 1;
           prow = crow[buf][cb];
         }
         if (ok) {
