@@ -447,9 +447,9 @@ __device__ __forceinline__ unsigned mag_bits(float v) {
   const unsigned u = __float_as_uint(v) & 0x7fffffffu;
   return u > 0x7f800000u ? 0u : u;
 }
-__device__ __forceinline__ unsigned mag_bits(double v) {
-  const unsigned u = (unsigned)__double2hiint(v) & 0x7fffffffu;
-  return u > 0x7ff00000u || (u == 0x7ff00000u && __double2loint(v) != 0) ? 0u : u;
+__device__ __forceinline__ unsigned long long mag_bits(double v) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  return u > 0x7ff0000000000000ull ? 0ull : u;
 }
 // the largest key of the warp and, of the lanes that hold it, the smallest position
 __device__ __forceinline__ void pick(unsigned* key, unsigned* pos) {
@@ -457,24 +457,12 @@ __device__ __forceinline__ void pick(unsigned* key, unsigned* pos) {
   *pos = __reduce_min_sync(0xffffffffu, *key == best ? *pos : 0xffffffffu);
   *key = best;
 }
-// 1 / v: FP64 from the hardware's approximate reciprocal (20 bits) and two Newton steps
-// r += r (1 - v r), which double the correct bits (20 -> 40 -> full); magnitudes whose
-// reciprocal could leave the normal range by division.  A step waits for it, and every
-// FP64 instruction holds a warp's quarter of the SM for 64 cycles.
-__device__ __forceinline__ float panel_recip(float v) { return 1.0f / v; }
-__device__ __forceinline__ double panel_recip(double v) {
-  const unsigned e = ((unsigned)__double2hiint(v) >> 20) & 0x7ffu;
-  if (e - 64u > 1918u) return 1.0 / v;
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
-  r = fma(r, fma(-v, r, 1.0), r);
-  r = fma(r, fma(-v, r, 1.0), r);
-  return r;
-}
-// v != 0 without an FP64 instruction
-__device__ __forceinline__ bool nonzero(float v) { return fabsf(v) > 0.f; }
-__device__ __forceinline__ bool nonzero(double v) {
-  return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) != 0;
+__device__ __forceinline__ void pick(unsigned long long* key, unsigned* pos) {
+  const unsigned hi = (unsigned)(*key >> 32), bh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned bl = __reduce_max_sync(0xffffffffu, hi == bh ? (unsigned)*key : 0u);
+  const unsigned long long best = (unsigned long long)bh << 32 | bl;
+  *pos = __reduce_min_sync(0xffffffffu, *key == best ? *pos : 0xffffffffu);
+  *key = best;
 }
 // the panel row's columns [8 g, 8 g + 8) of `src` in shared memory (16-byte aligned)
 __device__ __forceinline__ void load8(const float* src, float* v) {
@@ -552,6 +540,7 @@ __global__ void __launch_bounds__(NT)
     lu_panel_reg_kernel(T* fronts, int m, int k, int j0, int jb, int C, int* piv, int* pmap, int* perm,
                         const double* scale, double ptol, int* status, unsigned long long wait_ns) {
   constexpr int W = NT / 32;
+  using Mag = decltype(mag_bits(T()));
   const int q = C > 1 ? (int)(blockIdx.x % C) : 0;
   const long f = blockIdx.x / C;
   T* A = fronts + f * (long)m * m + j0 + (long)j0 * m;
@@ -559,9 +548,11 @@ __global__ void __launch_bounds__(NT)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int s0 = q * NT * R + tid;  // slot of row r: s0 + r NT
   __shared__ __align__(16) T wrow[2][W][kNB];   // posted candidate row of each warp
-  __shared__ unsigned wmag[2][W], wpos[2][W];
+  __shared__ Mag wmag[2][W];
+  __shared__ unsigned wpos[2][W];
   __shared__ __align__(16) T crow[2][kPanelMaxC][kNB];  // pushed rows of the cluster's CTAs
-  __shared__ __align__(8) unsigned long long ckey[2][kPanelMaxC];
+  __shared__ __align__(8) Mag cmag[2][kPanelMaxC];
+  __shared__ unsigned cpos[2][kPanelMaxC];
   __shared__ __align__(8) unsigned long long cbar[2];
   __shared__ int spiv[kNB];   // pivot positions in order
   __shared__ T spv[kNB];      // pivots
@@ -597,23 +588,25 @@ __global__ void __launch_bounds__(NT)
         const int buf = u & 1;
         // this thread's candidate: magnitude + 1 (0: none) and position (rows r > 0 in the
         // order of their positions)
-        unsigned mg = 0, mpos = 0xffffffffu;
+        Mag mg = 0;
+        unsigned mpos = 0xffffffffu;
 #pragma unroll
         for (int r = 1; r < R; ++r) {
-          const unsigned v = pj[r] < 0 && s0 + r * NT < kl ? mag_bits(a[r][u]) + 1u : 0u;
+          const Mag v = pj[r] < 0 && s0 + r * NT < kl ? mag_bits(a[r][u]) + 1 : 0;
           if (v > mg) {
             mg = v;
             mpos = (unsigned)(s0 + r * NT);
           }
         }
         {
-          const unsigned v = pj[0] < 0 && s0 < kl ? mag_bits(a[0][u]) + 1u : 0u;
+          const Mag v = pj[0] < 0 && s0 < kl ? mag_bits(a[0][u]) + 1 : 0;
           if (v && (v > mg || (v == mg && (unsigned)pos0 < mpos))) {
             mg = v;
             mpos = (unsigned)pos0;
           }
         }
-        unsigned wm = mg, wp = mpos;
+        Mag wm = mg;
+        unsigned wp = mpos;
         pick(&wm, &wp);
         if (mg == wm && mpos == wp && wm) {
 #pragma unroll
@@ -638,10 +631,12 @@ __global__ void __launch_bounds__(NT)
           __syncwarp();
         }
         // the CTA's best
-        unsigned best = wm, bpos = wp;
+        Mag best = wm;
+        unsigned bpos = wp;
         int wb = 0;
         if (W > 1) {
-          const unsigned bm = lane < W ? wmag[buf][lane] : 0u, bp = lane < W ? wpos[buf][lane] : 0xffffffffu;
+          const Mag bm = lane < W ? wmag[buf][lane] : 0;
+          const unsigned bp = lane < W ? wpos[buf][lane] : 0xffffffffu;
           best = bm;
           bpos = bp;
           pick(&best, &bpos);
@@ -652,22 +647,23 @@ __global__ void __launch_bounds__(NT)
           // push the row and its key to every CTA of the cluster (destinations spread
           // over the warps), then wait for the C pushes of this step
           const unsigned rdst = smem_addr(&crow[buf][q][lane]);
-          const unsigned kdst = smem_addr(&ckey[buf][q]), bar = smem_addr(&cbar[buf]);
+          const unsigned kdst = smem_addr(&cmag[buf][q]), pdst = smem_addr(&cpos[buf][q]);
+          const unsigned bar = smem_addr(&cbar[buf]);
           const T rv = wrow[buf][wb][lane];
-          const unsigned long long key = ((unsigned long long)best << 32) | bpos;
           if (tid == 0)
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                         "r"((unsigned)(C * (kNB * sizeof(T) + 8)))
+                         "r"((unsigned)(C * (kNB * sizeof(T) + sizeof(Mag) + 4)))
                          : "memory");
           for (int dst = warp; dst < C; dst += W) {
             const unsigned rb = peer_addr(bar, dst);
             push(peer_addr(rdst, dst), rb, rv);
-            if (lane == 0) push(peer_addr(kdst, dst), rb, key);
+            if (lane == 0) push(peer_addr(kdst, dst), rb, best);
+            if (lane == 1) push(peer_addr(pdst, dst), rb, bpos);
           }
           ok = bar_wait(bar, (jj >> 1) & 1, wait_ns);
           ok = __all_sync(0xffffffffu, ok);
-          const unsigned long long kk = lane < C ? ckey[buf][lane] : 0xffffffffull;
-          const unsigned km = (unsigned)(kk >> 32), kp = (unsigned)kk;
+          const Mag km = lane < C ? cmag[buf][lane] : 0;
+          const unsigned kp = lane < C ? cpos[buf][lane] : 0xffffffffu;
           best = km;
           bpos = kp;
           pick(&best, &bpos);
@@ -680,8 +676,8 @@ __global__ void __launch_bounds__(NT)
             spiv[jj] = best ? (int)bpos : jj;  // there is a candidate inside k columns, always
             spv[jj] = best ? pv : (T)0;
           }
-          if (!nonzero(pv)) pv = (T)(thresh > 0 ? thresh : 1e-30);
-          const T inv = panel_recip(pv);
+          if (mag_bits(pv) == 0) pv = (T)(thresh > 0 ? thresh : 1e-30);
+          const T inv = (T)1 / pv;
           T l[R];
 #pragma unroll
           for (int r = 0; r < R; ++r) {
@@ -1435,8 +1431,7 @@ __global__ void lu_perm_kernel(const int* piv, int* perm, int k, int nf) {
 // ---- explicit triangular inverses -------------------------------------------------
 // Inverses of every 32 x 32 diagonal block of L11 (unit lower) and U11 of every front, one
 // CTA per (block, front): threads 0-127 invert the L block, 128-255 the U block, four lanes
-// per column (rows 4 r + lane % 4 in registers) as in lu_trsm_kernel, U with the
-// reciprocals of its diagonal taken once.  Xl != null: written to the matching diagonal
+// per column (rows 4 r + lane % 4 in registers) as in lu_trsm_kernel.  Xl != null: written to the matching diagonal
 // blocks of Xl and Xu (entry (i, j) at i + j ldx, front stride sX).  Xl == null: in place,
 // the strict lower part from L^{-1}, the upper part with the diagonal from U^{-1}; the
 // sweeps then resolve a diagonal block with a matrix-vector product instead of 32
@@ -1452,13 +1447,10 @@ __global__ void __launch_bounds__(256) diag32_kernel(T* fronts, int m, int k, T*
   const int jb = min(kNB, k - j0);
   T* A = fronts + (long)blockIdx.y * m * m;
   __shared__ T Bk[kNB][kNB + 1];
-  __shared__ T dinv[kNB];
   for (int e = threadIdx.x; e < kNB * kNB; e += 256) {
     const int i = e % kNB, l = e / kNB;
     Bk[i][l] = (i < jb && l < jb) ? A[(j0 + i) + (long)(j0 + l) * m] : (i == l ? (T)1 : (T)0);
   }
-  __syncthreads();
-  if (threadIdx.x < kNB) dinv[threadIdx.x] = (T)1 / Bk[threadIdx.x][threadIdx.x];
   __syncthreads();
   const bool upper = threadIdx.x >= 128;
   if (sizeof(T) == sizeof(float) && upper) {
@@ -1489,6 +1481,7 @@ __global__ void __launch_bounds__(256) diag32_kernel(T* fronts, int m, int k, T*
   if (!upper) {
 #pragma unroll
     for (int l = 0; l < kNB - 1; ++l) {
+      if (l < (c & ~7)) continue;  // still zero in the warp's eight columns
       const T xl = __shfl_sync(0xffffffffu, x[l >> 2], base | (l & 3));
 #pragma unroll
       for (int r = l >> 2; r < R; ++r)
@@ -1497,7 +1490,8 @@ __global__ void __launch_bounds__(256) diag32_kernel(T* fronts, int m, int k, T*
   } else {
 #pragma unroll
     for (int l = kNB - 1; l >= 0; --l) {
-      if (sub == (l & 3)) x[l >> 2] *= dinv[l];
+      if (l > (c | 7)) continue;
+      if (sub == (l & 3)) x[l >> 2] /= Bk[l][l];
       const T xl = __shfl_sync(0xffffffffu, x[l >> 2], base | (l & 3));
 #pragma unroll
       for (int r = 0; r <= (l >> 2); ++r)

@@ -86,10 +86,15 @@ def reference(A, k, cols):
         X, Y = np.eye(n, dtype=T), np.eye(n, dtype=T)
         for l in range(n):
             X[l + 1:] = fma(-D[l + 1:, l:l + 1], X[l:l + 1], X[l + 1:])
-        for i in reversed(range(n)):
-            for l in range(i + 1, n):
-                Y[i] = fma(-D[i, l], Y[l], Y[i])
-            Y[i] = Y[i] / D[i, i]
+        if T == np.float32:
+            for i in reversed(range(n)):
+                for l in range(i + 1, n):
+                    Y[i] = fma(-D[i, l], Y[l], Y[i])
+                Y[i] = Y[i] / D[i, i]
+        else:
+            for l in reversed(range(n)):
+                Y[l] = Y[l] / D[l, l]
+                Y[:l] = fma(-D[:l, l:l + 1], Y[l:l + 1], Y[:l])
         W[j0:e, j0:e] = np.tril(X, -1) + np.triu(Y)
     return W, piv
 
@@ -158,3 +163,15 @@ def test_fp32_bits_of_many_tall_fronts():
     got, piv, perm, st = factor(A, 33)
     assert st == 0
     check(A, 33, got, piv, perm, (0, 152), np.array([33, 300, 599]))
+
+
+@pytest.mark.parametrize("m,k,nf", [(20, 20, 3), (50, 25, 2), (70, 32, 2), (250, 32, 2), (600, 32, 2), (600, 32, 80),
+                                    (1100, 30, 1), (2100, 32, 1), (4200, 32, 1)])
+def test_fp64_pivots_and_multipliers(m, k, nf):
+    """One panel in FP64, bit for bit: pivots compared on all bits of the magnitudes (here equal in
+    their leading 30), multipliers from the correctly rounded reciprocal."""
+    rng = np.random.default_rng([m, nf])
+    A = np.where(rng.random((nf, m, m)) < 0.5, 1.0, -1.0) * (1.0 + rng.integers(0, 9, (nf, m, m)) * 2.0 ** -33)
+    got, piv, perm, st = factor(A, k)
+    assert st == 0
+    check(A, k, got, piv, perm, {0, nf - 1}, np.zeros(0, int))
