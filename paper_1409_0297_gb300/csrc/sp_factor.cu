@@ -429,8 +429,11 @@ __global__ void __launch_bounds__(256) lu_panel_grid_kernel(T* fronts, int m, in
 // all C CTAs with st.async on the receiver's mbarrier (double-buffered by the step's
 // parity: a CTA pushes step j + 2 only after it holds every push of step j + 1, which
 // its peers sent after they had read step j), so a step costs one CTA barrier and one
-// one-way trip through distributed shared memory.  Every wait gives up after wait_ns
-// (status bit 2, identity interchanges, no write-back).
+// one-way trip through distributed shared memory.  A wait that lasts longer than wait_ns
+// makes the panel report a timeout (status bit 2, identity interchanges, no write-back), but
+// the CTA goes on with the steps: its peers' pushes are in flight then, and a CTA that left
+// would be written to after its shared memory was handed on.  Only a wait of kPushDrainNs
+// more, which the resident CTAs of a cluster cannot cause, ends the panel at once.
 //
 // The 32 columns are taken in four blocks of eight: the eight steps are unrolled with
 // the current block in registers 0-7, the columns right of it updated in groups of
@@ -441,6 +444,7 @@ __global__ void __launch_bounds__(256) lu_panel_grid_kernel(T* fronts, int m, in
 // (FP64), so FP32 panels take the fewest CTAs whose registers hold them and FP64 panels
 // as many as the level leaves free (panel_shape).
 constexpr int kPanelMaxC = 16;
+constexpr unsigned long long kPushDrainNs = 2000000000ull;
 
 // magnitudes as integers of the same order; a NaN is never the largest
 __device__ __forceinline__ unsigned mag_bits(float v) {
@@ -518,20 +522,24 @@ __device__ __forceinline__ void push(unsigned dst, unsigned bar, float v) {
 __device__ __forceinline__ void push(unsigned dst, unsigned bar, double v) {
   push(dst, bar, (unsigned long long)__double_as_longlong(v));
 }
-// bounded wait for the phase of the given parity
-__device__ __forceinline__ bool bar_wait(unsigned bar, unsigned parity, unsigned long long wait_ns) {
+// bounded wait for the phase of the given parity (acquire at cluster scope: the peers' pushes):
+// *late after wait_ns, given up kPushDrainNs later
+__device__ __forceinline__ bool bar_wait(unsigned bar, unsigned parity, unsigned long long wait_ns,
+                                         bool* late) {
   const unsigned long long t0 = gtimer_ns();
   while (true) {
     unsigned done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done)
         : "r"(bar), "r"(parity)
         : "memory");
     if (done) return true;
-    if (gtimer_ns() - t0 > wait_ns) return false;
+    const unsigned long long t = gtimer_ns() - t0;
+    if (t > wait_ns) *late = true;
+    if (t > wait_ns + kPushDrainNs) return false;
   }
 }
 
@@ -551,8 +559,9 @@ __global__ void __launch_bounds__(NT)
   __shared__ Mag wmag[2][W];
   __shared__ unsigned wpos[2][W];
   __shared__ __align__(16) T crow[2][kPanelMaxC][kNB];  // pushed rows of the cluster's CTAs
-  __shared__ __align__(8) Mag cmag[2][kPanelMaxC];
-  __shared__ unsigned cpos[2][kPanelMaxC];
+  constexpr bool kWide = sizeof(Mag) == 8;  // FP64: the position does not fit beside the magnitude
+  __shared__ __align__(8) unsigned long long ckey[2][kPanelMaxC];
+  __shared__ unsigned cpos[2][kWide ? kPanelMaxC : 1];
   __shared__ __align__(8) unsigned long long cbar[2];
   __shared__ int spiv[kNB];   // pivot positions in order
   __shared__ T spv[kNB];      // pivots
@@ -578,6 +587,7 @@ __global__ void __launch_bounds__(NT)
   for (int r = 0; r < R; ++r) pj[r] = -1;
   int pos0 = s0;  // position of row r = 0; the other rows stay at their slots
   bool ok = true, stop = false;  // this warp's last wait; the CTA gave up
+  bool late = false;             // a wait of this warp ran over its limit
 #pragma unroll 1
   for (int o = 0; o < kNB / 8; ++o) {
     const int live = kNB / 8 - o;  // column groups of eight not finished (the current one included)
@@ -647,23 +657,24 @@ __global__ void __launch_bounds__(NT)
           // push the row and its key to every CTA of the cluster (destinations spread
           // over the warps), then wait for the C pushes of this step
           const unsigned rdst = smem_addr(&crow[buf][q][lane]);
-          const unsigned kdst = smem_addr(&cmag[buf][q]), pdst = smem_addr(&cpos[buf][q]);
+          const unsigned kdst = smem_addr(&ckey[buf][q]), pdst = smem_addr(&cpos[buf][kWide ? q : 0]);
           const unsigned bar = smem_addr(&cbar[buf]);
           const T rv = wrow[buf][wb][lane];
+          const unsigned long long key = kWide ? (unsigned long long)best : (unsigned long long)best << 32 | bpos;
           if (tid == 0)
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                         "r"((unsigned)(C * (kNB * sizeof(T) + sizeof(Mag) + 4)))
+                         "r"((unsigned)(C * (kNB * sizeof(T) + 8 + (kWide ? 4 : 0))))
                          : "memory");
           for (int dst = warp; dst < C; dst += W) {
             const unsigned rb = peer_addr(bar, dst);
             push(peer_addr(rdst, dst), rb, rv);
-            if (lane == 0) push(peer_addr(kdst, dst), rb, best);
-            if (lane == 1) push(peer_addr(pdst, dst), rb, bpos);
+            if (lane == 0) push(peer_addr(kdst, dst), rb, key);
+            if (kWide && lane == 1) push(peer_addr(pdst, dst), rb, bpos);
           }
-          ok = bar_wait(bar, (jj >> 1) & 1, wait_ns);
-          ok = __all_sync(0xffffffffu, ok);
-          const Mag km = lane < C ? cmag[buf][lane] : 0;
-          const unsigned kp = lane < C ? cpos[buf][lane] : 0xffffffffu;
+          ok = __all_sync(0xffffffffu, bar_wait(bar, (jj >> 1) & 1, wait_ns, &late));
+          const unsigned long long kk = lane < C ? ckey[buf][lane] : 0xffffffffull;
+          const Mag km = kWide ? (lane < C ? (Mag)kk : 0) : (Mag)(kk >> 32);
+          const unsigned kp = kWide && lane < C ? cpos[buf][lane] : (unsigned)kk;
           best = km;
           bpos = kp;
           pick(&best, &bpos);
@@ -716,7 +727,7 @@ __global__ void __launch_bounds__(NT)
   }
   int* pvf = piv + f * k + j0;
   int* mpf = pmap + (f * ((k + kNB - 1) / kNB) + j0 / kNB) * (2 * kNB);
-  if (C > 1 && __syncthreads_or(!ok || stop)) {
+  if (C > 1 && __syncthreads_or(!ok || stop || late)) {
     // later kernels of the factorisation still read this panel's interchanges
     if (tid == 0) atomicOr(status, 2);
     if (q == 0)
