@@ -398,7 +398,9 @@ sp_status sp_profile_read(sp_ctx *ctx, int cap, double *ms, int *launches, doubl
  * operand buffers).
  * A, B, C: device pointers owned by the caller; C must not overlap A or B.
  * Synchronous on `stream` (cudaStream_t or NULL).  SP_ERR_ARG for bad sizes or
- * forms, SP_ERR_TIMEOUT if a tensor-core pipeline wait ran out. */
+ * forms, SP_ERR_TIMEOUT if a tensor-core pipeline wait ran out.  FP64: every entry is off by less than 2^-48
+ * sum |a b| per 32 of depth plus two roundings of |C| + sum |a b| (an FMA loop's bound: products
+ * come from digit sums on the tensor cores where these are that accurate, else from FMAs). */
 sp_status sp_schur_update(sp_precision prec, int M, int N, int K, const void *A, int lda,
                           long long sA, const void *B, int ldb, long long sB, void *C, int ldc,
                           long long sC, int batch, void *stream);

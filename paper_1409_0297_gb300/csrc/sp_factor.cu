@@ -1548,25 +1548,44 @@ __global__ void trinv_store_kernel(T* fronts, int m, const T* Xl, const T* Xu, l
 // into seven balanced digits of nine bits, X = sum_i f_i 2^(9 i), |f_i| <= 256, each an
 // exact FP16 number.  The sums S_h = sum_{i + j = h + 6} sum_k f_i(A) f_j(B), h = 0 .. 6, are
 // then exact in the FP32 accumulators of mma.sync (at most 7 x 32 x 2^16 < 2^24), and
-// sum_k A B = 2^(Ea + Eb - 2114) sum_h S_h 2^(9 h) up to the digit pairs with i + j < 6,
-// less than 2^-56 of (row maximum) x (column maximum).  The sum of the S_h is formed as a
-// 64-bit integer and enters C with two FP64 FMAs.
+// sum_k A B = 2^(Ea + Eb - 2114) sum_h S_h 2^(9 h) up to the digit pairs with i + j < 6.  The
+// sum of the S_h is formed as a 64-bit integer and enters C with two FP64 FMAs.
+//
+// Error, in X X and whatever the entries are: digit pairs left out 2^68.6, bits cut from
+// entries more than nine binades below their row's largest 2^67.  Against sum |a b| that is
+// nothing where the large entries of the row meet those of the column, and everything where
+// they only meet zeros or far smaller ones.  So the leading digits give a lower bound of
+// sum |a b|, one more product: P = sum_k |f_6(a)| |f_6(b)|, and |X| >= (|f_6| - 0.501) 2^54.
+//   P >= 2^14 (a leading digit at its smallest times another, so a row's largest entry that
+//     meets a column's largest is enough): sum |X X| > 2^121, the 64-bit sum in units of 2^68
+//     adds 2^68 with the first FMA; the error is below 2^-51 sum |a b|.
+//   1088 <= P < 2^14: sum |X X| > 2^117.04; units of 2^63 add 2^63; below 2^-48 sum |a b|, the
+//     bound of an FMA loop of 32 steps.
+//   P < 1088: the FMA loop over the entries where row and column are both nonzero (a mask of 32
+//     bits each); no such entry: the product is zero and C stays.
 //
 // One CTA: a 64 x 64 tile, eight warps of 16 x 32 (two halves of 16 x 16, so the 56
 // accumulators of a half fit beside the fragments and two CTAs share an SM).  The tile's
 // digits are cut once into shared memory (rows of 32 halves, 80 bytes apart: conflict-free
-// for ldmatrix), 28 products of 16 x 16 x 16 per 16 x 16 block and 16 of depth.  What
-// bounds it: three FP64 instructions, ~25 integer ones and 28 / 16 x 2 tensor
+// for ldmatrix), 29 products of 16 x 16 x 16 per 16 x 16 block and 16 of depth.  What
+// bounds it: three FP64 instructions, ~25 integer ones and 29 / 16 x 2 tensor
 // instructions per output and chunk, where the FMA loop took 32 FP64 instructions.
-// Rows whose entries leave [2^-477, 2^477], and infinities and NaNs, take the FMA loop.
+// Rows whose entries leave [2^-477, 2^477] (subnormals too), and infinities and NaNs, take the
+// FMA loop for the whole tile.
 constexpr int kDig = 7;          // digits of a number
 constexpr int kDigT = 64;        // tile
 constexpr int kDigPitch = 40;    // halves between the 32-deep rows of a digit plane
 constexpr int kDigPlane = kDigT * kDigPitch;
+constexpr float kDigWeight = 1088.f;  // smallest leading-digit product sum that the digits carry
+constexpr float kDigFine = 16384.f;   // below: the 64-bit sum in finer units
 constexpr int kDigElo = 546, kDigEhi = 1500;  // biased exponents of a row's largest entry
 constexpr size_t kDigSmem = 2 * kDig * kDigPlane * sizeof(__half);
 
-__device__ __forceinline__ int f64_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+// biased exponent (1 for subnormals, 0 for zero)
+__device__ __forceinline__ int f64_exp(double x) {
+  const int hi = __double2hiint(x) & 0x7fffffff;
+  return hi >= 0x100000 ? hi >> 20 : ((hi | __double2loint(x)) != 0 ? 1 : 0);
+}
 
 // the seven digits of eight numbers on the exponent E, written as eight consecutive halves
 // of seven planes (dst: the first plane's 16 bytes)
@@ -1622,15 +1641,16 @@ __device__ __forceinline__ void mma_f16(float* c, const unsigned* a, unsigned b0
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// acc +- 2^(es - 1023) sum_h S_h 2^(9 h - 14): es the biased exponent of the unit of the
-// 64-bit sum T (its 14 lowest bits are below the dropped digit pairs)
-__device__ __forceinline__ double add_digits(double acc, const float* S, int es, unsigned neg) {
+// acc +- sum_h S_h 2^(9 h), from the 64-bit sum T of the S_h in units of 2^68 (in X X), or of
+// 2^63 (fine) where the weight keeps |T| below 2^61; es the biased exponent of the unit 2^68
+__device__ __forceinline__ double add_digits(double acc, const float* S, int es, bool fine, unsigned neg) {
   const int s0 = __float2int_rn(S[0]), s1 = __float2int_rn(S[1]), s2 = __float2int_rn(S[2]);
   const int s3 = __float2int_rn(S[3]), s4 = __float2int_rn(S[4]), s5 = __float2int_rn(S[5]);
   const int s6 = __float2int_rn(S[6]);
-  const long long low = (long long)s3 * 8192 + (long long)(s2 * 16 + ((s1 + (s0 >> 9) + 16) >> 5));
-  const long long top = (long long)(s6 * 512 + s5) * 512 + s4;
-  const long long T = (top << 22) + low;
+  const long long low = (long long)s3 * 262144 + ((long long)s2 * 512 + (s1 + ((s0 + 256) >> 9)));
+  const long long top = (long long)s6 * 262144 + ((long long)s5 * 512 + s4);
+  const long long T = fine ? (long long)((unsigned long long)top << 27) + low : (top << 22) + ((low + 16) >> 5);
+  if (fine) es -= 5;
   // T = hi 2^32 + lo as two exact doubles: 2^52 + lo, and hi - 2^20 (its 2^52 cancels)
   const double dl = __hiloint2double(0x43300000, (int)(unsigned)T);
   const double dh = __hiloint2double(0x43300000, (int)(T >> 32) ^ (int)0x80000000) -
@@ -1650,6 +1670,7 @@ __global__ void __launch_bounds__(256, ONE ? 2 : 1) gemm_f64_kernel(GemmSide<dou
   __half* Ad = reinterpret_cast<__half*>(smraw);
   __half* Bd = Ad + kDig * kDigPlane;
   __shared__ int eA[4][kDigT], eB[kDigT];
+  __shared__ __align__(4) unsigned char nzA[kDigT][4], nzB[kDigT][4];  // nonzero entries, eight to a byte
   __shared__ int s_plain;
   const GemmSide<double> g = blockIdx.z ? g1 : g0;
   const int M = g.M, N = g.N, lda = g.lda, ldb = g.ldb, ldc = g.ldc;
@@ -1698,11 +1719,17 @@ __global__ void __launch_bounds__(256, ONE ? 2 : 1) gemm_f64_kernel(GemmSide<dou
     }
     if (tid == 0) s_plain = 0;
     int ea = 0, eb = 0;
+    unsigned za = 0, zb = 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      ea = max(ea, f64_exp(xa[j]));
-      eb = max(eb, f64_exp(xb[j]));
+      const int fa = f64_exp(xa[j]), fb = f64_exp(xb[j]);
+      ea = max(ea, fa);
+      eb = max(eb, fb);
+      za |= (fa != 0 ? 1u : 0u) << j;
+      zb |= (fb != 0 ? 1u : 0u) << j;
     }
+    nzA[ai][tid >> 6] = (unsigned char)za;
+    nzB[bc][tid & 3] = (unsigned char)zb;
     eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, 1));
     eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, 2));
     eA[tid >> 6][ai] = ea;
@@ -1766,19 +1793,76 @@ __global__ void __launch_bounds__(256, ONE ? 2 : 1) gemm_f64_kernel(GemmSide<dou
           }
         }
       }
+      // the weight of each output's products
+      float Q[2][4];
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) Q[t][i] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) {
+        if (ks * 16 < kc) {
+          unsigned fa[4], fb[4];
+          ldmatrix4(fa, a_frag + 2 * ((kDig - 1) * kDigPlane + ks * 16));
+          ldmatrix4(fb, b_frag + 2 * ((kDig - 1) * kDigPlane + s * 16 * kDigPitch + ks * 16));
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            fa[i] &= 0x7fff7fffu;
+            fb[i] &= 0x7fff7fffu;
+          }
+          mma_f16(Q[0], fa, fb[0], fb[1]);
+          mma_f16(Q[1], fa, fb[2], fb[3]);
+        }
+      }
+      // the digit sums of all eight outputs without a branch between them (their FP64 chains
+      // overlap), then the few of low weight
+      unsigned low = 0;
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int row = rw + 8 * ((i >> 1) & 1), col = cw + 16 * s + 8 * (i >> 2) + (i & 1);
         const int er = max(max(eA[0][row], eA[1][row]), max(eA[2][row], eA[3][row]));
-        const int es = max(er + eB[col] - 1077, 1);
         float v[kDig];
 #pragma unroll
         for (int h = 0; h < kDig; ++h) v[h] = P[h][i >> 2][i & 3];
         double& o = acc[ONE ? 0 : s][i];
-        o = add_digits(o, v, es, neg);
-        if (ONE) {
+        const float q = Q[i >> 2][i & 3];
+        const double t = add_digits(o, v, max(er + eB[col] - 1077, 6), q < kDigFine, neg);
+        if (q >= kDigWeight) o = t;
+        else low |= 1u << i;
+      }
+      if (low) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int row = rw + 8 * ((i >> 1) & 1), col = cw + 16 * s + 8 * (i >> 2) + (i & 1);
+          unsigned both = *reinterpret_cast<const unsigned*>(nzA[row]) & *reinterpret_cast<const unsigned*>(nzB[col]);
+          if (!(low >> i & 1)) both = 0;
+          if (both) {
+            const double* ar = A + r0 + row + (long)k0 * lda;
+            const double* bc_ = B + k0 + (long)(c0 + col) * ldb;
+            double sum[4] = {0.0, 0.0, 0.0, 0.0};  // an FP64 chain a quarter as long
+            while (both) {
+              double x[4], y[4];
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const int k = __ffs(both) - 1;
+                x[u] = both ? ar[(long)k * lda] : 0.0;
+                y[u] = both ? bc_[k] : 0.0;
+                both &= both - 1;
+              }
+#pragma unroll
+              for (int u = 0; u < 4; ++u) sum[u] = fma(x[u], y[u], sum[u]);
+            }
+            const double v = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+            double& o = acc[ONE ? 0 : s][i];
+            o = neg ? o - v : o + v;
+          }
+        }
+      }
+      if (ONE) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
           const long at = out_at(s, i);
-          if (at >= 0) C[at] = o;
+          if (at >= 0) C[at] = acc[0][i];
         }
       }
     }
