@@ -132,7 +132,7 @@ typedef struct {
                         work vectors in shared memory; on levels with few fronts a
                         thread-block cluster of up to 16 CTAs per front walks the diagonal
                         blocks itself).  0 (default): fused only on levels whose fronts
-                        fill the GPU without clusters and have 128 rows or more,
+                        fill the GPU without clusters and have 100 rows or more,
                         chains elsewhere; 1: chains
                         everywhere; 2: fused wherever the vectors fit.  All are exact
                         applications of the same factor; they round differently. */
@@ -168,8 +168,9 @@ typedef struct {
                         host drives every iteration (reads the estimate after each
                         step).  Default 1. */
   int factor_storage; /* FP32-family forms (FP32, mixed, TF32, 3xTF32): 1 keeps, after each
-                        factorisation, an FP16 copy of the fronts of the levels whose sweeps
-                        run as chains of block products (the large upper levels), each front
+                        factorisation, an FP16 copy of the fronts of the levels too small to
+                        fill the GPU (fewer than two fronts per SM: the large upper levels; with
+                        sweeps = 1 all levels, with 2 those not fused), each front
                         column scaled by a power of two so its largest entry stays below
                         2^15; those sweeps then read half the bytes and sum in FP32 (Section
                         2.3's solve with the factor, at FP16 accuracy of the factor entries:

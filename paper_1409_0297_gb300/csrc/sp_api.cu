@@ -885,18 +885,22 @@ static sp_status setup_impl(int d, int n, int b, int P, const double* shifts, sp
     D.ib = c->opts.inv_block > 0 ? c->opts.inv_block
                                  : (S.k >= 16384 ? 2048 : (S.k >= 4096 ? 1024 : kInvBlockSize));
     D.pdl = c->opts.launch_overlap;
-    // fused sweeps pay on fronts with enough rows for a CTA: applying the preconditioner,
-    // leaves of 289 (169) rows 0.411 against 0.430 (0.279 against 0.308) ms with launch chains,
-    // leaves of 49 and 69 rows (four 192^2 problems) 0.308 against 0.266 ms
-    if (D.inv && (c->opts.sweeps == 2 || (c->opts.sweeps == 0 && S.m >= 128))) {
+    // fused sweeps pay on fronts with enough rows for a CTA (application of the FP32
+    // preconditioner with launch chains against fused): leaves of 25 rows at 256^2 195 / 236 us,
+    // 49 rows at 192^2 140 / 148, 81 rows at 512^2 410 / 470 (at 256^2 165.0 / 166.3), 3D 64 rows
+    // at 48^3 925 / 958; 125 rows at 3D 32^3 391 / 387, 169 rows 308 / 279, 289 rows 430 / 411.
+    bool fits = false;  // could be swept fused (sweeps = 1: never is)
+    if (D.inv && c->opts.sweeps != 1) {
       int C = 0, NT = 0;
-      if (sweep_fused_config(prec, D.nf, S.m, S.k, num_sms, max_cluster, c->opts.sweeps == 2, &C,
-                             &NT)) {
+      fits = sweep_fused_config(prec, D.nf, S.m, S.k, num_sms, max_cluster, c->opts.sweeps == 2, &C, &NT);
+      if (fits && (c->opts.sweeps == 2 || S.m >= 100)) {
         D.fused_c = C;
         D.fused_nt = NT;
       }
     }
-    if (D.inv && D.fused_c == 0 && c->opts.factor_storage == 1) {
+    // the FP16 copy is for large fronts: levels that are chained for their few rows alone keep
+    // reading FP32
+    if (D.inv && !fits && c->opts.factor_storage == 1) {
       SP_CK(dalloc(c.get(), &D.front16, (size_t)2 * D.nf * S.m * ((S.m + 1) & ~1)));
       SP_CK(dalloc(c.get(), &D.fscale16, sizeof(float) * D.nf * S.m));
     }
