@@ -17,7 +17,7 @@ LIB = os.path.join(HERE, "libsp_gb300.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["sp_host.cpp", "sp_fft.cu", "sp_factor.cu", "sp_solve.cu", "sp_krylov.cu", "sp_api.cu",
            "sp_static.cu", "sp_tc.cu", "sp_fno.cu"]
-HEADERS = ["sp_host.h", "sp_internal.h"]
+HEADERS = ["sp_device.h", "sp_host.h", "sp_internal.h"]
 
 
 def _nvcc() -> str:

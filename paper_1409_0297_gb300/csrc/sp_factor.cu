@@ -1881,12 +1881,12 @@ __global__ void __launch_bounds__(256, ONE ? 2 : 1) gemm_f64_kernel(GemmSide<dou
 
 void gemm_f64(const GemmSide<double>& g0, const GemmSide<double>* g1, bool minus, bool beta_one,
               int batch, int nb2, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(gemm_f64_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDigSmem);
-    cudaFuncSetAttribute(gemm_f64_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDigSmem);
-    attr = true;
-  }
+  static PerDevice attr;
+  attr.run([] {
+    const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t e = cudaFuncSetAttribute(gemm_f64_kernel<true>, at, (int)kDigSmem);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(gemm_f64_kernel<false>, at, (int)kDigSmem);
+  });  // a refusal shows as the launch's error
   auto tiles = [](const GemmSide<double>& g) {
     return ((g.M + kDigT - 1) / kDigT) * ((g.N + kDigT - 1) / kDigT);
   };
@@ -2048,7 +2048,7 @@ bool grid_panel_front(int m) {
 int panel_max_cluster() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 8;
-  static int cache[64] = {0};
+  static std::atomic<int> cache[64];  // 0: not asked yet
   if (cache[dev]) return cache[dev];
   int best = 8;
   auto kern = lu_panel_reg_kernel<double, 256, 3>;
@@ -2130,11 +2130,8 @@ void launch_panel_reg(DevLevel& L, T* F, int j0, int jb, int C, double ptol, int
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   if (C > 1) {
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      attr = true;
-    }
+    static PerDevice attr;
+    attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); });
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)C;
     at[0].val.clusterDim.y = 1;
@@ -2294,14 +2291,13 @@ void front_scale(DevLevel& L, cudaStream_t st) {
 // fronts and their largest magnitudes L.scale.
 template <class T>
 cudaError_t lu_fronts(DevLevel& L, double ptol, int* status, const FactorWork& W, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(lu_panel_grid_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kGridPanelSmem + 1024);
-    cudaFuncSetAttribute(lu_panel_calu_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kGridPanelSmem + 1024);
-    attr = true;
-  }
+  static PerDevice attr;
+  const cudaError_t ea = attr.run([] {
+    const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t e = cudaFuncSetAttribute(lu_panel_grid_kernel<T>, at, (int)kGridPanelSmem + 1024);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(lu_panel_calu_kernel, at, (int)kGridPanelSmem + 1024);
+  });
+  if (ea != cudaSuccess) return ea;
   const int m = L.m, k = L.k;
   T* F = (T*)L.front;
   if (panel_in_registers<T>(L, W)) {

@@ -356,12 +356,13 @@ cudaError_t run_pass(int d, int n, const VT* tw, const typename Real<VT>::T* Dn,
     a.W /= 2;
   const size_t smem = (size_t)a.W * a.ld * sizeof(VT);
   const unsigned grid = (unsigned)((a.nlines + a.W - 1) / a.W);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(fft_pass_kernel<VT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(fft_pass_kernel<VT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr_set = true;
-  }
+  static PerDevice attr;
+  const cudaError_t ea = attr.run([] {
+    const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t e = cudaFuncSetAttribute(fft_pass_kernel<VT, 1>, at, 200 * 1024);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(fft_pass_kernel<VT, 2>, at, 200 * 1024);
+  });
+  if (ea != cudaSuccess) return ea;
   const double es = sizeof(VT);
   ProfScope ps(PROF_FFT, st);
   auto kern = G == 2 ? fft_pass_kernel<VT, 2> : fft_pass_kernel<VT, 1>;

@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "../../include/sp.h"
+#include "sp_device.h"
 #include "sp_host.h"
 
 namespace sp {

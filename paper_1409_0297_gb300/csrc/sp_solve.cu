@@ -740,13 +740,15 @@ cudaError_t q_apply_t(int d, int n, int nl, const std::vector<QTypeDev>& types, 
 size_t sweep_smem(int m, int k, size_t vt) { return vt * (size_t)(m + k); }
 
 template <class VT, class T>
-void set_attrs() {
-  cudaFuncSetAttribute(forward_kernel<VT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  cudaFuncSetAttribute(backward_kernel<VT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  cudaFuncSetAttribute(inv_gemv_kernel<VT, T, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  cudaFuncSetAttribute(inv_gemv_kernel<VT, T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  cudaFuncSetAttribute(inv_gemv_kernel<VT, __half, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  cudaFuncSetAttribute(inv_gemv_kernel<VT, __half, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+cudaError_t set_attrs() {
+  const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(forward_kernel<VT, T>, at, 200 * 1024))) return e;
+  if ((e = cudaFuncSetAttribute(backward_kernel<VT, T>, at, 200 * 1024))) return e;
+  if ((e = cudaFuncSetAttribute(inv_gemv_kernel<VT, T, 16>, at, 200 * 1024))) return e;
+  if ((e = cudaFuncSetAttribute(inv_gemv_kernel<VT, T, 4>, at, 200 * 1024))) return e;
+  if ((e = cudaFuncSetAttribute(inv_gemv_kernel<VT, __half, 16>, at, 200 * 1024))) return e;
+  return cudaFuncSetAttribute(inv_gemv_kernel<VT, __half, 4>, at, 200 * 1024);
 }
 
 constexpr int kGemvTarget = 1216;  // CTAs a row-parallel product aims for (8 per SM)
@@ -840,11 +842,9 @@ template <class VT>
 cudaError_t forward_t(int d, DevLevel& L, const DevLevel* child, const void* rhsQ, void* part,
                       int nv, long N, cudaStream_t st) {
   using T = typename Scalar<VT>::T;
-  static bool attr = false;
-  if (!attr) {
-    set_attrs<VT, T>();
-    attr = true;
-  }
+  static PerDevice attr;
+  const cudaError_t ea = attr.run([] { return set_attrs<VT, T>(); });
+  if (ea != cudaSuccess) return ea;
   if (nv < 1 || nv > kMaxVec) return cudaErrorInvalidValue;
   const double kk = L.k, mk = L.m - L.k;
   ProfScope ps(PROF_FORWARD, st);
@@ -1237,19 +1237,16 @@ cudaError_t fused_launch_t(bool fwd, const FusedArgs& a, int nf, int C, int grou
   const size_t smem = fused_smem<VT, NT, NV>(a.m, a.k);
   if (smem > kFusedSmemMax) return cudaErrorInvalidValue;
   auto kern = fwd ? fused_forward_kernel<VT, T, NT, NV> : fused_backward_kernel<VT, T, NT, NV>;
-  // the attributes are set once per kernel, to the largest size any level may ask
+  // the attributes are set once per kernel and device, to the largest size any level may ask
   // for: a launch captured into a graph keeps its own request, and lowering the
   // attribute later would make that graph's launch fail
-  static bool attr_fwd = false, attr_bwd = false;
-  bool& attr = fwd ? attr_fwd : attr_bwd;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kFusedSmemMax);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static PerDevice attr_fwd, attr_bwd;
+  const cudaError_t ea = (fwd ? attr_fwd : attr_bwd).run([&] {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)kFusedSmemMax);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
+  if (ea != cudaSuccess) return ea;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(nf * C), (unsigned)groups);
   cfg.blockDim = dim3(NT);
@@ -1370,7 +1367,7 @@ int sweep_max_cluster() {
   // kernels (1024 threads, the FP64 shared memory of a 2044-wide root) can be resident
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 8;
-  static int cache[64] = {0};
+  static std::atomic<int> cache[64];  // 0: not asked yet
   if (cache[dev]) return cache[dev];
   int best = 8;
   auto kern = fused_forward_kernel<double2, double, 1024, 1>;

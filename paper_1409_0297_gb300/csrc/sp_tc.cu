@@ -596,22 +596,17 @@ size_t tc_pack_floats(int rows, int K, int batch, bool split) {
 namespace {
 
 cudaError_t tc_set_attributes() {
-  static bool attr = false;
-  if (attr) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(tc_gemm_sub_kernel<kBN, kStages, 0>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(tc_gemm_sub_kernel<kBN, kStagesRing, 2>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemRing);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(tc_gemm_sub_kernel<kBN, kStages, 1>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemRing1);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(tc_gemm_sub_kernel<kBN, kStages, 1, 2>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemRing1);
-  if (e != cudaSuccess) return e;
-  attr = true;
-  return cudaSuccess;
+  static PerDevice attr;
+  return attr.run([] {
+    const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(tc_gemm_sub_kernel<kBN, kStages, 0>, at, (int)kSmem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(tc_gemm_sub_kernel<kBN, kStagesRing, 2>, at, (int)kSmemRing);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(tc_gemm_sub_kernel<kBN, kStages, 1>, at, (int)kSmemRing1);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(tc_gemm_sub_kernel<kBN, kStages, 1, 2>, at, (int)kSmemRing1);
+  });
 }
 
 // the product kernel on already packed operands of depth Ke (a multiple of kBK)
