@@ -1081,10 +1081,13 @@ constexpr size_t kWgSmemMax = 200 * 1024;  // staged tiles of a weight-gradient 
 constexpr size_t kColsSmemMax = (512 * 16 + 512) * sizeof(float2);
 constexpr size_t kCombineSmemMax = 64 * 512 * sizeof(float);
 
+// mode mixing at the widest network and the largest batch that dims_ok accepts: a network's own
+// size would lower the limit under the launches of a larger one that is alive
+constexpr size_t kMixSmemMax = (32 * 32 + 2 * 256 * 32) * sizeof(float2);
+
 template <class TA>
-cudaError_t set_attrs(int mixB, int W) {
+cudaError_t set_attrs() {
   cudaError_t e;
-  const size_t mix = (size_t)(W * W + 2 * mixB * W) * sizeof(float2);
   const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if ((e = cudaFuncSetAttribute(chan_wgrad_kernel<TA>, at, (int)kWgSmemMax))) return e;
   if ((e = cudaFuncSetAttribute(chan_wgrad_kernel<float>, at, (int)kWgSmemMax))) return e;
@@ -1094,8 +1097,8 @@ cudaError_t set_attrs(int mixB, int W) {
   if ((e = cudaFuncSetAttribute(combine_kernel<float, float, 256>, at, (int)kCombineSmemMax))) return e;
   if ((e = cudaFuncSetAttribute(combine_kernel<float, float, 512>, at, (int)kCombineSmemMax))) return e;
   if ((e = cudaFuncSetAttribute(dft_cols_fwd_kernel, at, (int)kColsSmemMax))) return e;
-  if ((e = cudaFuncSetAttribute(spec_mix_kernel, at, (int)mix))) return e;
-  return cudaFuncSetAttribute(spec_mix_bwd_kernel, at, (int)mix);
+  if ((e = cudaFuncSetAttribute(spec_mix_kernel, at, (int)kMixSmemMax))) return e;
+  return cudaFuncSetAttribute(spec_mix_bwd_kernel, at, (int)kMixSmemMax);
 }
 
 // a tiled pointwise layer (ci <= 32); ~8 CTAs per SM, each keeping its weights over its tiles
@@ -1316,7 +1319,7 @@ sp_status fno_init(sp_fno* f, const sp_fno_dims* dims, const float* params_host,
       (e = dalloc(f, &f->npart, (size_t)3 * kNormBlocks * sizeof(double))))
     return fail(e);
   if ((e = cudaMallocHost(&f->hloss, sizeof(double)))) return fail(e);
-  if ((e = D.act_fp32 ? set_attrs<float>(B, W) : set_attrs<bf16>(B, W))) return fail(e);
+  if ((e = D.act_fp32 ? set_attrs<float>() : set_attrs<bf16>())) return fail(e);
   // twiddles e^{-2 pi i m / n}, with the product kx j0 reduced mod n before the angle
   std::vector<float2> twr((size_t)n * 16), twb(n);
   const double tau = 6.283185307179586476925286766559;
