@@ -90,7 +90,8 @@ typedef struct {
                         of every level (Schur-update and block-inverse GEMM tiles,
                         32 or 64) on a placeholder medium (q = 0) and keeps the
                         fastest; every result is bit-identical to the untuned
-                        context's.  0 (default): built-in heuristics */
+                        context's; FP64 products have one tile, 64, and nothing is
+                        timed.  0 (default): built-in heuristics */
   int max_rhs;       /* right-hand sides sp_solve_many may take at once, 1 ... 8
                         (default 1); the solve workspace is sized for it */
   int setup_route;   /* how sp_setup forms T_S = G(S, gamma^c) G(beta, gamma^c)^+:

@@ -241,9 +241,17 @@ float time_ms(cudaStream_t st, int reps, Fn fn) {
 // leave every result bit-identical: each output entry is summed in the same
 // order): each candidate of a level is timed on that level alone (a level's
 // factorisation re-assembles its fronts from its children), bottom-up, with the
-// medium in qbuf (zero at set-up: P = Q).
+// medium in qbuf (zero at set-up: P = Q).  FP64 products have one tile (64 x 64, digit products),
+// so there is nothing to time: the levels say 64.
 sp_status autotune(sp_ctx* c) {
   cudaStream_t st = c->stream;
+  if (c->prec == SP_PREC_FP64) {
+    for (DevLevel& D : c->lv) {
+      D.gemm_tile = 64;
+      if (D.inv) D.gen_tile = 64;
+    }
+    return SP_OK;
+  }
   SP_CK(cudaMemsetAsync(c->status, 0, sizeof(int), st));
   sp_status fs = factor_direct(c, c->qbuf, st);  // warm-up; leaves a valid factor
   if (fs != SP_OK) return fs;
