@@ -97,8 +97,9 @@ def _operator(d, n, s, q, x, fused):
     return (y[0] + x.real) + 1j * (y[1] + x.imag)
 
 
-@pytest.mark.parametrize("d,n,b", [(2, 4, 2), (2, 6, 3), (2, 8, 2), (2, 12, 3), (2, 32, 4), (2, 64, 4), (2, 96, 6),
-                                   (2, 128, 8), (3, 8, 2), (3, 24, 3), (3, 32, 4)])
+@pytest.mark.parametrize("d,n,b", [(2, 4, 2), (2, 6, 3), (2, 8, 2), (2, 12, 3), (2, 16, 4), (2, 32, 4), (2, 48, 6),
+                                   (2, 64, 4), (2, 96, 6), (2, 128, 8), (2, 256, 16), (2, 768, 24), (3, 4, 2),
+                                   (3, 8, 2), (3, 16, 4), (3, 24, 3), (3, 32, 4)])
 def test_operator_bits(d, n, b):
     import torch
 
@@ -117,3 +118,26 @@ def test_operator_bits(d, n, b):
     S.close()
     got = w.cpu().numpy().reshape(shape)
     assert any(np.array_equal(got, _operator(d, n, s, q, x, fused)) for fused in (True, False))
+
+
+@pytest.mark.parametrize("n,b,P", [(6, 3, 210), (4, 2, 40), (16, 4, 5)])
+def test_lines_of_stacked_vectors(n, b, P):
+    """Vectors of a group behind one another: a CTA's lines cross from one to the next (6^2: four
+    lines a CTA, six a vector).  Every problem gives the bits of a context of its own."""
+    import torch
+
+    from paper_1409_0297_gb300 import binding as B
+
+    rng = np.random.default_rng(n)
+    s = 4 * np.pi ** 2 * (10.5 + np.arange(P) % 7)
+    x = torch.from_numpy(rng.standard_normal(P * n * n) + 1j * rng.standard_normal(P * n * n)).cuda()
+    S = B.Solver(2, n, b, list(s), prec=B.SP_PREC_FP32, restart=2, setup_route=1)
+    w = torch.empty_like(x)
+    S.green(x, w)
+    S.close()
+    for p in sorted({0, 1, 2, P // 2, P - 1}):
+        S = B.Solver(2, n, b, s[p], prec=B.SP_PREC_FP32, restart=2, setup_route=1)
+        one = torch.empty(n * n, dtype=torch.complex128, device="cuda")
+        S.green(x[p * n * n:(p + 1) * n * n].clone(), one)
+        S.close()
+        assert torch.equal(w[p * n * n:(p + 1) * n * n], one)
