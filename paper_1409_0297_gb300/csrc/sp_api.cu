@@ -660,6 +660,14 @@ void sp_destroy(sp_ctx* c) {
   delete c;
 }
 
+// a set-up that fails gives back what it had allocated
+struct CtxFree {
+  void operator()(sp_ctx* c) const {
+    if (c->allocs.empty()) delete c;
+    else sp_destroy(c);
+  }
+};
+
 static sp_status setup_impl(int d, int n, int b, int P, const double* shifts, sp_precision prec,
                             const sp_opts* opts, void* stream, sp_ctx** out) {
   if (!out || !shifts || P < 1) return SP_ERR_ARG;
@@ -688,7 +696,7 @@ static sp_status setup_impl(int d, int n, int b, int P, const double* shifts, sp
     if (shift_gap(d, n, shifts[p]) < 1e-6) return SP_ERR_RESONANT;
   }
   const double s = shifts[0];
-  std::unique_ptr<sp_ctx> c(new (std::nothrow) sp_ctx());
+  std::unique_ptr<sp_ctx, CtxFree> c(new (std::nothrow) sp_ctx());
   if (!c) return SP_ERR_OOM;
   sp_default_opts(&c->opts);
   if (opts) c->opts = *opts;
