@@ -1450,7 +1450,7 @@ __global__ void lu_perm_kernel(const int* piv, int* perm, int k, int nf) {
 // launch took 64 us however few its blocks were.  The FP32 U block keeps one thread per
 // column: row i subtracts its products in the order of l = i + 1 ..., which starts with the
 // entry computed last, so four lanes could only take another order, and the FP32
-// preconditioner's bits would change with it (the chain costs FP32 ~2 us).
+// preconditioner's bits would change with it (2D 512^2, all inverses: 2.41 -> 2.49 ms).
 template <class T>
 __global__ void __launch_bounds__(256) diag32_kernel(T* fronts, int m, int k, T* Xl, T* Xu, int ldx,
                                                      long sX) {
@@ -1568,8 +1568,11 @@ __global__ void trinv_store_kernel(T* fronts, int m, const T* Xl, const T* Xu, l
 // accumulators of a half fit beside the fragments and two CTAs share an SM).  The tile's
 // digits are cut once into shared memory (rows of 32 halves, 80 bytes apart: conflict-free
 // for ldmatrix), 29 products of 16 x 16 x 16 per 16 x 16 block and 16 of depth.  What
-// bounds it: three FP64 instructions, ~25 integer ones and 29 / 16 x 2 tensor
-// instructions per output and chunk, where the FMA loop took 32 FP64 instructions.
+// bounds it: latency between the phases of a tile (load, cut, multiply, combine) and the FMA
+// loops of the outputs of low weight; no pipe is above 40 % (leaf level of 2D 512^2: FP64 38, ALU 34,
+// tensor 18).  Three FP64 instructions, ~30 integer ones and 29 / 16 x 2 tensor instructions per
+// output and chunk, where the FMA loop took 32 FP64 instructions.  All 101 updates of a 2D 512^2
+// factor 10.2 ms (FMA loop 33), 205 of 3D 32^3 39.9 (144).
 // Rows whose entries leave [2^-477, 2^477] (subnormals too), and infinities and NaNs, take the
 // FMA loop for the whole tile.
 constexpr int kDig = 7;          // digits of a number
@@ -2078,7 +2081,8 @@ int panel_max_cluster() {
 // 256 rows while the level leaves SMs free (2044 rows: 33 us on eight CTAs, 43 us on
 // two), else up to 1536 rows per CTA.  FP64: the rank-1 updates run at two FMAs per SM
 // cycle, so a level with few fronts splits each over as many SMs as there are, down to
-// ~96 rows per CTA (2044 rows: 61 us on 16 CTAs, 80 us on eight).
+// ~96 rows per CTA (2044 rows: 66 us on 16 CTAs; before the reciprocal was a division 61, and 80 on
+// eight).
 template <class T>
 bool panel_shape(int nf, int rows, int* C, int* NT, int* R) {
   const int maxc = panel_max_cluster();
