@@ -129,7 +129,7 @@ typedef struct {
                         (the LU panel of fronts split over several CTAs, which wait for
                         the pivot candidates that their peers push or publish) in
                         nanoseconds of the GPU's global timer; 0 (default) = 2e9 (2 s),
-                        else 1 ... 6e10.  When a wait runs out the panel stops and
+                        else 1 ... 6e10.  When a wait runs out the panel is given up and
                         sp_factor returns SP_ERR_TIMEOUT; destroy that context. */
   int sweeps;        /* forward / backward sweeps of the levels that keep block inverses
                         (Section 2.3's solve with the factor): a level is either swept by a
