@@ -138,7 +138,8 @@ typedef struct {
                         work vectors in shared memory; on levels with few fronts a
                         thread-block cluster of up to 16 CTAs per front walks the diagonal
                         blocks itself).  0 (default): fused only on levels whose fronts
-                        fill the GPU without clusters and have 100 rows or more,
+                        fill the GPU without clusters and have 100 rows or more
+                        (80 where a level has at most 1024 fronts),
                         chains elsewhere; 1: chains
                         everywhere; 2: fused wherever the vectors fit.  All are exact
                         applications of the same factor; they round differently. */

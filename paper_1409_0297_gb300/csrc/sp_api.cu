@@ -903,13 +903,14 @@ static sp_status setup_impl(int d, int n, int b, int P, const double* shifts, sp
     D.pdl = c->opts.launch_overlap;
     // fused sweeps pay on fronts with enough rows for a CTA (application of the FP32
     // preconditioner with launch chains against fused): leaves of 25 rows at 256^2 195 / 236 us,
-    // 49 rows at 192^2 140 / 148, 81 rows at 512^2 410 / 470 (at 256^2 165.0 / 166.3), 3D 64 rows
-    // at 48^3 925 / 958; 125 rows at 3D 32^3 391 / 387, 169 rows 308 / 279, 289 rows 430 / 411.
+    // 49 rows at 192^2 140 / 148, 81 rows at 512^2 (4096 fronts) 410 / 470, 3D 64 rows at 48^3 925 /
+    // 958; 125 rows at 3D 32^3 391 / 387, 169 rows 308 / 279, 289 rows 430 / 411.  81 rows of 1024
+    // fronts are even (256^2 165.0 / 166.3), so they stay fused and give the bits they gave.
     bool fits = false;  // could be swept fused (sweeps = 1: never is)
     if (D.inv && c->opts.sweeps != 1) {
       int C = 0, NT = 0;
       fits = sweep_fused_config(prec, D.nf, S.m, S.k, num_sms, max_cluster, c->opts.sweeps == 2, &C, &NT);
-      if (fits && (c->opts.sweeps == 2 || S.m >= 100)) {
+      if (fits && (c->opts.sweeps == 2 || S.m >= (D.nf <= 1024 ? 80 : 100))) {
         D.fused_c = C;
         D.fused_nt = NT;
       }
